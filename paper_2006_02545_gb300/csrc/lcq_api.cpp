@@ -1384,9 +1384,14 @@ static lcq_status apply_impl(lcq_ctx* ctx, const lcq_near* nr, const lcq_corr* c
   };
   bool fold = foldable(c->kp);
   for (const GroupParams& g : c->grp_h) fold = fold && foldable(g.kp);
-  double* src = nullptr;
-  auto src_free = on_exit([&] { dfree(st, src); });
+  double *src = nullptr, *part = nullptr;
+  auto src_free = on_exit([&] {
+    dfree(st, src);
+    dfree(st, part);
+  });
   CK(dalloc(st, &src, (size_t)(fold ? 10 : 9) * std::max<int64_t>(c->n_over, 1)));
+  const int parts = far_sum_parts(ctx->num_sms, nr->n_targets, c->n_over);
+  CK(dalloc(st, &part, (size_t)2 * parts * std::max<int64_t>(nr->n_targets, 1)));
   for (int d = 1; d <= kMaxDeg; ++d) {
     if (!nr->plist_count[d]) continue;
     launch_far_src(d, lc, nr->plist_dev[d], nr->plist_count[d], dv, ctx->deg[d].dV, c->q,
@@ -1394,8 +1399,9 @@ static lcq_status apply_impl(lcq_ctx* ctx, const lcq_near* nr, const lcq_corr* c
   }
   launch_far_sum(lc, nr->tgt, nr->n_targets, src, c->n_over, c->kp, nr->tgt_patch, c->src_off,
                  c->grp ? nr->tgroup : nullptr, c->grp, c->gsrc,
-                 kind == LCQ_SP ? nr->tnrm : nullptr, out, fold);
-  launch_csr_apply(lc, nr->row_ptr, nr->col, c->val, sigma, nr->tnode, nr->n_targets, jump, out);
+                 kind == LCQ_SP ? nr->tnrm : nullptr, part, parts, fold);
+  launch_csr_apply(lc, nr->row_ptr, nr->col, c->val, sigma, nr->tnode, nr->n_targets, jump, part,
+                   parts, out);
   CK(cudaGetLastError());
   return LCQ_OK;
 }

@@ -67,15 +67,20 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
   if (i < n) out[i] += boff[blockIdx.x];
 }
 
-// Direct far sum over all oversampled sources, one thread per target (tiles of sources
-// staged through shared memory); kernel values by kernel_eval_tc (table sincos and the
+// Direct far sum over the oversampled sources, one thread per target and range of sources
+// (tiles staged through shared memory): block (b, s) sums part s of gridDim.y equal parts of
+// the sources of target block b into part[s][t], and k_csr_apply adds the parts in order.  Few
+// targets alone leave the chip idle (1000 targets are 8 blocks on 152 SMs), so the launch cuts
+// the sources until there are several waves of blocks (far_sum_parts): 1000 targets and 129,000
+// sources 327 ms with one part, 10 ms so; 8,960 and 26,000 66.2 and 15.7 ms.  Kernel values by kernel_eval_tc (table sincos and the
 // Newton-refined reciprocal square root: FP64 throughout, about 48 FP64 instructions per
 // pair for the CFIE), or with fold by kernel_eval_fold on sources that carry the kernel
 // constants (about 41).
 // The sources of an on-surface target's own patch are skipped (their contribution is
 // carried entirely by the self correction).  In a batch of independent surfaces a target
 // sums only its own surface's sources [gsrc[g], gsrc[g+1]) with that surface's kernel.
-__global__ void __launch_bounds__(kThreads) k_far_sum(const double* __restrict__ tgt, int64_t NT,
+constexpr int kFarThreads = 128;
+__global__ void __launch_bounds__(kFarThreads) k_far_sum(const double* __restrict__ tgt, int64_t NT,
                                                       const double* __restrict__ src, int64_t n_over,
                                                       const KernelParams kp,
                                                       const int32_t* __restrict__ tpatch,
@@ -84,8 +89,8 @@ __global__ void __launch_bounds__(kThreads) k_far_sum(const double* __restrict__
                                                       const GroupParams* __restrict__ grp,
                                                       const int64_t* __restrict__ gsrc,
                                                       const double* __restrict__ tnrm,
-                                                      cplx* __restrict__ out, bool fold) {
-  __shared__ double s[10][kThreads];
+                                                      cplx* __restrict__ part, bool fold) {
+  __shared__ double s[10][kFarThreads];
   __shared__ unsigned long long blo, bhi;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double x0 = 0, x1 = 0, x2 = 0;
@@ -122,18 +127,20 @@ __global__ void __launch_bounds__(kThreads) k_far_sum(const double* __restrict__
     atomicMax(&bhi, (unsigned long long)hi);
   }
   __syncthreads();
-  const int64_t b0 = (int64_t)blo, b1 = (int64_t)bhi;
+  const int64_t all = (int64_t)bhi - (int64_t)blo;
+  const int64_t b0 = (int64_t)blo + all * blockIdx.y / gridDim.y;
+  const int64_t b1 = (int64_t)blo + all * (blockIdx.y + 1) / gridDim.y;
   const KernelParamsF kf = to_f32(kt);
   const bool has_ki = kt.ki != 0.0;
   float env;  // not used: the far sum needs no rounding envelope
   double re = 0.0, im = 0.0;
   const int rows = fold ? 10 : 9;
-  for (int64_t s0 = b0; s0 < b1; s0 += kThreads) {
+  for (int64_t s0 = b0; s0 < b1; s0 += kFarThreads) {
     __syncthreads();
     const int64_t q = s0 + threadIdx.x;
     for (int c = 0; c < rows; ++c) s[c][threadIdx.x] = q < b1 ? src[c * n_over + q] : 0.0;
     __syncthreads();
-    const int cnt = (int)min((int64_t)kThreads, b1 - s0);
+    const int cnt = (int)min((int64_t)kFarThreads, b1 - s0);
     if (t < NT)
       for (int k = 0; k < cnt; ++k) {
         const int64_t qq = s0 + k;
@@ -150,19 +157,24 @@ __global__ void __launch_bounds__(kThreads) k_far_sum(const double* __restrict__
         im = fma(g.im, s[7][k], im);
       }
   }
-  if (t < NT) out[t] = {re, im};
+  if (t < NT) part[blockIdx.y * NT + t] = {re, im};
 }
 
 // The correction part of the corrected potential (Sec. 5.3): warp per target row,
-// out_t += sum_row c sigma, plus jump * sigma at an on-surface target's own node.
+// out_t = the far sum's parts + sum_row c sigma, plus jump * sigma at an on-surface target's own node.
 __global__ void k_csr_apply(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                             const double* __restrict__ val, const cplx* __restrict__ sigma,
                             const int64_t* __restrict__ tnode, int64_t NT, double jump,
-                            cplx* __restrict__ out) {
+                            const cplx* __restrict__ part, int parts, cplx* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t t = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); t < NT; t += warps) {
     double re = 0.0, im = 0.0;
+    for (int k = lane; k < parts; k += 32) {
+      const cplx p = part[k * NT + t];
+      re += p.re;
+      im += p.im;
+    }
     for (int64_t e = row_ptr[t] + lane; e < row_ptr[t + 1]; e += 32) {
       const double vr = val[2 * e], vi = val[2 * e + 1];
       const cplx sg = sigma[col[e]];
@@ -172,9 +184,7 @@ __global__ void k_csr_apply(const int64_t* __restrict__ row_ptr, const int32_t* 
     re = warp_sum(re);
     im = warp_sum(im);
     if (lane == 0) {
-      cplx o = out[t];
-      o.re += re;
-      o.im += im;
+      cplx o = {re, im};
       if (jump != 0.0 && tnode[t] >= 0) {
         o.re += jump * sigma[tnode[t]].re;
         o.im += jump * sigma[tnode[t]].im;
@@ -345,15 +355,24 @@ bool launch_far_src(int d, const LaunchCommon& lc, const int* plist, int count, 
                     double* src, int64_t n_over, const KernelParams& kp, bool fold) {
   return dispatch<FarSrcL>(d, lc, plist, count, dv, Vt, qv, src_off, sigma, src, n_over, kp, fold);
 }
+// Parts that the far sum's sources are cut into: enough blocks for about four waves of eight
+// on every SM, at least 32 sources each.
+int far_sum_parts(int num_sms, int64_t NT, int64_t n_over) {
+  const int64_t tb = (NT + kFarThreads - 1) / kFarThreads;
+  if (tb <= 0) return 1;
+  const int64_t want = (32ll * num_sms + tb - 1) / tb, most = n_over / 32;
+  const int64_t s = want < most ? want : most;
+  return (int)(s < 1 ? 1 : s);
+}
 void launch_far_sum(const LaunchCommon& lc, const double* tgt, int64_t NT, const double* src,
                     int64_t n_over, const KernelParams& kp, const int32_t* tpatch,
                     const int64_t* src_off, const int32_t* tgroup, const GroupParams* grp,
-                    const int64_t* gsrc, const double* tnrm, void* out, bool fold) {
-  const int64_t g = (NT + kThreads - 1) / kThreads;
+                    const int64_t* gsrc, const double* tnrm, void* part, int parts, bool fold) {
+  const int64_t g = (NT + kFarThreads - 1) / kFarThreads;
   if (g <= 0) return;
   ++*lc.launches;
-  k_far_sum<<<(unsigned)g, kThreads, 0, lc.stream>>>(tgt, NT, src, n_over, kp, tpatch, src_off,
-                                                     tgroup, grp, gsrc, tnrm, (cplx*)out, fold);
+  k_far_sum<<<dim3((unsigned)g, (unsigned)parts), kFarThreads, 0, lc.stream>>>(
+      tgt, NT, src, n_over, kp, tpatch, src_off, tgroup, grp, gsrc, tnrm, (cplx*)part, fold);
 }
 void launch_widen_c64(const LaunchCommon& lc, const void* in, int64_t n, void* out) {
   if (n <= 0) return;
@@ -364,11 +383,11 @@ void launch_widen_c64(const LaunchCommon& lc, const void* in, int64_t n, void* o
 }
 void launch_csr_apply(const LaunchCommon& lc, const int64_t* row_ptr, const int32_t* col,
                       const double* val, const void* sigma, const int64_t* tnode, int64_t NT,
-                      double jump, void* out) {
+                      double jump, const void* part, int parts, void* out) {
   const int g = lc.num_sms * 8;
   ++*lc.launches;
   k_csr_apply<<<g, 256, 0, lc.stream>>>(row_ptr, col, val, (const cplx*)sigma, tnode, NT, jump,
-                                        (cplx*)out);
+                                        (const cplx*)part, parts, (cplx*)out);
 }
 
 // Resident blocks per SM of k_adaptive<d> (the persistent grid is this times the SM count).

@@ -155,14 +155,17 @@ bool launch_far_src(int d, const LaunchCommon& lc, const int* plist, int count, 
                     const double* Vt, const int32_t* qv, const int64_t* src_off, const void* sigma,
                     double* src, int64_t n_over, const KernelParams& kp = KernelParams{},
                     bool fold = false);
+// The sources' range cut into `parts` = far_sum_parts() equal parts, part s of target t summed into
+// part[s][t] (complex); launch_csr_apply adds them.
+int far_sum_parts(int num_sms, int64_t NT, int64_t n_over);
 void launch_far_sum(const LaunchCommon& lc, const double* tgt, int64_t NT, const double* src,
                     int64_t n_over, const KernelParams& kp, const int32_t* tpatch,
                     const int64_t* src_off, const int32_t* tgroup, const GroupParams* grp,
-                    const int64_t* gsrc, const double* tnrm, void* out, bool fold = false);
+                    const int64_t* gsrc, const double* tnrm, void* part, int parts, bool fold = false);
 void launch_widen_c64(const LaunchCommon& lc, const void* in, int64_t n, void* out);
 void launch_csr_apply(const LaunchCommon& lc, const int64_t* row_ptr, const int32_t* col,
                       const double* val, const void* sigma, const int64_t* tnode, int64_t NT,
-                      double jump, void* out);
+                      double jump, const void* part, int parts, void* out);
 int adaptive_blocks_per_sm(int d);
 
 // Unit target normals for S' (SoA [3][NT]): the chart normal at the node of an on-surface
