@@ -52,7 +52,63 @@ static __device__ double2 g_sct[kSinCosTable];
 // the same angles as two-float pairs (cos_h, cos_l, sin_h, sin_l) for the two-float kernel
 static __device__ float4 g_sctf[kSinCosTable];
 
-// Fills c_kw, c_jac, c_kwexp, g_sct and g_sctf of the calling translation unit.
+// The tables of the fixed-point kernel values (lcq_fx.cuh), from double-double sums of the
+// Taylor series (about 100 bits) rounded to 2^-62.
+static __device__ __align__(16) FxCs g_fxcs[kFxTab];
+static __device__ u64 g_fxdec[kFxTab];
+__device__ __forceinline__ FxTables fx_tables() { return {g_fxcs, g_fxdec}; }
+
+struct HostDD {
+  double h, l;
+};
+inline HostDD dd_add(HostDD a, HostDD b) {
+  const double s = a.h + b.h, v = s - a.h;
+  const double e = (a.h - (s - v)) + (b.h - v) + a.l + b.l;
+  return {s + e, e - ((s + e) - s)};
+}
+inline HostDD dd_mul(HostDD a, HostDD b) {
+  const double p = a.h * b.h;
+  const double e = fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h);
+  return {p + e, e - ((p + e) - p)};
+}
+inline HostDD dd_div(HostDD a, double b) {  // b a small integer
+  const double q = a.h / b, r = (fma(-q, b, a.h) + a.l) / b;
+  return {q + r, r - ((q + r) - q)};
+}
+inline u64 dd_fix62(HostDD a) {  // a 2^62 rounded, 0 <= a <= 1
+  const double x = a.h * 4611686018427387904.0;
+  const i64 i = (i64)x;
+  return (u64)(i + llrint((x - (double)i) + a.l * 4611686018427387904.0));
+}
+struct FxHostTables {
+  std::vector<FxCs> cs;
+  std::vector<u64> dec;
+};
+inline FxHostTables fx_build_tables() {
+  FxHostTables t{std::vector<FxCs>(kFxTab), std::vector<u64>(kFxTab)};
+  const HostDD pi = {3.141592653589793116, 1.2246467991473532e-16};
+  const HostDD ln2 = {0.69314718055994528623, 2.3190468138462996e-17};
+  for (int j = 0; j < kFxTab; ++j) {
+    const HostDD x = dd_mul(pi, {j / 2048.0, 0.0}), y = dd_mul(ln2, {-j / 1024.0, 0.0});
+    HostDD term = {1.0, 0.0}, c = {0.0, 0.0}, s = {0.0, 0.0}, t2 = {1.0, 0.0}, e = {0.0, 0.0};
+    for (int i = 0; i < 34; ++i) {
+      HostDD& into = (i & 1) ? s : c;
+      into = dd_add(into, (i & 2) ? HostDD{-term.h, -term.l} : term);
+      e = dd_add(e, t2);
+      term = dd_div(dd_mul(term, x), i + 1.0);
+      t2 = dd_div(dd_mul(t2, y), i + 1.0);
+    }
+    t.cs[j] = {dd_fix62(c), dd_fix62(s)};
+    t.dec[j] = dd_fix62(e);
+  }
+  return t;
+}
+inline const FxHostTables& fx_host_tables() {
+  static const FxHostTables t = fx_build_tables();
+  return t;
+}
+
+// Fills c_kw, c_jac, c_kwexp, g_sct, g_sctf, g_fxcs and g_fxdec of the calling translation unit.
 static inline cudaError_t upload_kw_tables(cudaStream_t st) {
   double c[kMaxBasis], jc[(kMaxDeg + 1) * (kMaxDeg + 1) * 3] = {};
   int ke[kMaxBasis];
@@ -80,6 +136,7 @@ static inline cudaError_t upload_kw_tables(cudaStream_t st) {
     const float ch = (float)sct[j].x, sh = (float)sct[j].y;
     sctf[j] = make_float4(ch, (float)(sct[j].x - ch), sh, (float)(sct[j].y - sh));
   }
+  const FxHostTables& fxt = fx_host_tables();
   cudaError_t e = cudaMemcpyToSymbolAsync(c_kw, c, sizeof(c), 0, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyToSymbolAsync(c_jac, jc, sizeof(jc), 0, cudaMemcpyHostToDevice, st);
@@ -90,6 +147,12 @@ static inline cudaError_t upload_kw_tables(cudaStream_t st) {
                                 cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyToSymbolAsync(g_sctf, sctf.data(), sizeof(float4) * kSinCosTable, 0,
+                                cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyToSymbolAsync(g_fxcs, fxt.cs.data(), sizeof(FxCs) * kFxTab, 0,
+                                cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyToSymbolAsync(g_fxdec, fxt.dec.data(), sizeof(u64) * kFxTab, 0,
                                 cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the sources live on this stack
   return e;
@@ -580,6 +643,41 @@ __device__ __forceinline__ cplx kernel_eval(const KernelParams& kp, double x0, d
   }
   return {ex * (cs * c.re - sn * c.im), ex * (cs * c.im + sn * c.re)};
 }
+
+// The pairs that the fixed-point kernel value (fx_eval) does not cover, in FP64: coincident
+// points (0), distances outside [2^-300, 2^300], phases above 2^22 turns, decays that underflow,
+// values that are not finite.  n, w, ew: the node as fx_eval takes it.  Rare, so out of line.
+static __device__ __noinline__ cplx fx_fallback(const KernelParams& kp, double d0, double d1,
+                                                double d2, FxS n0, FxS n1, FxS n2, u64 w, int ew,
+                                                double R, float* env) {
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  const double Jw = ew > kFxBad ? nan : ldexp((double)w, ew - 62) * 12.566370614359172954;
+  const double s = Jw * 2.168404344971008868e-19;  // 2^-62
+  auto val = [](FxS a) { return (double)a.h * 4294967296.0 + 2.0 * (double)a.l; };
+  KernelParams k = kp;
+  if (k.kind == 3) k.kind = 1;
+  double e = 0.0;
+  const cplx g = kernel_eval(k, d0, d1, d2, 0.0, 0.0, 0.0, val(n0) * s, val(n1) * s, val(n2) * s,
+                             Jw, R, env ? &e : nullptr);
+  if (env) *env = (float)e;
+  return g;
+}
+
+// A node for fx_eval from its unnormalized normal N (|N| the area element) and rule weight:
+// the unit normal 2^62 and W = |N| w / (4 pi) = wm 2^(ew - 62).
+__device__ __forceinline__ void fx_make_node(const double* N, double wt, FxS* n, u64* wm, int* ew) {
+  const double N2 = fma(N[0], N[0], fma(N[1], N[1], N[2] * N[2]));
+  const double ri = N2 > 0.0 ? rsqrt(N2) : 0.0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) n[c] = fx_split(fx_fix(N[c] * ri, 0));
+  const double W = N2 * ri * wt * 0.07957747154594767;
+  *wm = (u64)fx_mant(W, ew);
+  if (!isfinite(N2)) *ew = kFxBad + 1;
+}
+__device__ __forceinline__ u64 fx_join(FxS a) {
+  return ((u64)(uint32_t)a.h << 32) | (uint32_t)a.l;
+}
+__device__ __forceinline__ FxS fx_unjoin(u64 v) { return {(int)(v >> 32), (int)(uint32_t)v}; }
 
 // Kernel parameters converted to FP32 once per patch (the mixed form's pair evaluations).
 struct KernelParamsF {

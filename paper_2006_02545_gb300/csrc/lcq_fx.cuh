@@ -1,0 +1,401 @@
+// Helmholtz kernel values in 64-bit fixed-point arithmetic on the integer pipe.
+//
+// On this GPU a warp's FP64 instruction occupies its pipe for 64 cycles, a 32 x 32 + 64 bit
+// integer multiply-add for 2 and a 64-bit addition for 1.  A product of two 62-bit mantissas
+// to 62 bits is three such multiply-adds, so the whole kernel value costs less than seven
+// FP64 instructions would, with more bits: every quantity below is a 57- to 63-bit mantissa
+// on a scale that is known beforehand (or one exponent per pair), where FP64 has 53.
+//
+// The value is written without the node's area element in it:
+//   K~ = W e^{-ki r} e^{i kr r} (A + iB) / r^2,   W = Jw / (4 pi),
+//   A = Re(beta) r + c (Re(alpha) + p r),  B = Im(beta) r + c (Im(alpha) + q r),
+//   c = n.d / r (n the unit normal, d = x - X),
+//   p = Re(alpha) ki + Im(alpha) kr,  q = Im(alpha) ki - Re(alpha) kr,
+// which is alpha (1 - ikr) n.d / r^2 + beta times W e^{ikr} / r, with every term bounded by
+// its own constant times max(1, r), so that A and B are fixed-point sums at one exponent per
+// pair.  The single layer alone is W e^{ikr} / r.
+//
+// Host and device code alike: the arithmetic is plain 64-bit integers, so a host program can
+// compare it with higher precision; only the start of the reciprocal square root differs.
+#pragma once
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+#ifdef __CUDACC__
+#define LCQ_HD __host__ __device__ __forceinline__
+#else
+#define LCQ_HD inline
+#endif
+
+namespace lcq {
+
+typedef unsigned long long u64;
+typedef long long i64;
+
+LCQ_HD uint32_t fx_hi(u64 x) { return (uint32_t)(x >> 32); }
+LCQ_HD uint32_t fx_lo(u64 x) { return (uint32_t)x; }
+LCQ_HD u64 fx_wide(uint32_t a, uint32_t b) { return (u64)a * b; }
+LCQ_HD i64 fx_swide(int a, int b) { return (i64)a * b; }
+
+// a b / 2^64 for a, b < 2^63 (error below 2 units): three multiply-adds.
+LCQ_HD u64 fx_umul(u64 a, u64 b) {
+  const u64 t = fx_wide(fx_hi(a), fx_lo(b)) + fx_wide(fx_lo(a), fx_hi(b));
+  return fx_wide(fx_hi(a), fx_hi(b)) + (u64)fx_hi(t);
+}
+// a b / 2^32 for b < 2^32 and a b < 2^96.
+LCQ_HD u64 fx_umul32(u64 a, uint32_t b) {
+  return fx_wide(fx_hi(a), b) + (u64)fx_hi(fx_wide(fx_lo(a), b));
+}
+
+// A signed value as a signed high word and 31 bits of the low one, v = h 2^32 + 2 l (the last
+// bit dropped), so that the cross products are products of signed 32-bit numbers.
+struct FxS {
+  int h, l;
+};
+LCQ_HD FxS fx_split(i64 v) { return {(int)(v >> 32), (int)((uint32_t)v >> 1)}; }
+// a b / 2^64 for |a|, |b| < 2^63 with |a b| < 2^126.
+LCQ_HD i64 fx_smul(FxS a, FxS b) {
+  const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h);
+  return fx_swide(a.h, b.h) + (t >> 31);
+}
+// (a b + c d) / 2^61, |a|, |c| < 2^62.3, |b|, |d| < 2^61
+LCQ_HD i64 fx_dot2(FxS a, FxS b, FxS c, FxS d) {
+  const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h) + fx_swide(c.h, d.l) + fx_swide(c.l, d.h);
+  return ((fx_swide(a.h, b.h) + fx_swide(c.h, d.h)) << 3) + (t >> 28);
+}
+
+LCQ_HD u64 fx_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return (u64)__double_as_longlong(x);
+#else
+  u64 b;
+  memcpy(&b, &x, 8);
+  return b;
+#endif
+}
+LCQ_HD double fx_double(u64 b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double x;
+  memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+LCQ_HD int fx_max(int a, int b) { return a > b ? a : b; }
+LCQ_HD int fx_min(int a, int b) { return a < b ? a : b; }
+LCQ_HD i64 fx_sra(i64 v, int s) { return v >> (s < 63 ? s : 63); }
+
+constexpr int kFxBad = 2000;  // exponents above: not a finite number
+// x = m 2^(e - 62) with 2^61 <= |m| < 2^62 (m = 0, e = kFxZero for x = 0 and subnormals).
+constexpr int kFxZero = -4000;
+LCQ_HD i64 fx_mant(double x, int* e) {
+  const u64 b = fx_bits(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  if (ex == 0) {
+    *e = kFxZero;
+    return 0;
+  }
+  *e = ex - 1022;
+  const i64 m = (i64)(((b & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+  return (b >> 63) ? -m : m;
+}
+// x 2^62 / 2^e for |x| <= 2^e (truncated toward -infinity below the last bit)
+LCQ_HD i64 fx_fix(double x, int e) {
+  int ex;
+  const i64 m = fx_mant(x, &ex);
+  if (m == 0) return 0;
+  const int s = e - ex;
+  return s < 0 ? m * 2 : fx_sra(m, s);
+}
+
+// Constants of a kernel (one patch's, or one launch's): kind 0: S, else the general form.
+struct FxKernel {
+  u64 kt;        // |kr| / (2 pi) = kt 2^(ek - 62)
+  u64 kd;        // ki / ln 2 = kd 2^(ed - 62), 0: none
+  FxS ar, ai;    // alpha 2^(62 - ea)
+  FxS p, q;      // (p, q) 2^(62 - ep)
+  FxS br, bi;    // beta 2^(62 - eb)
+  int ek, ed, ea, ep, eb;
+  int neg;       // kr < 0: the phase's sign
+  int single;    // the single layer alone (alpha = 0, beta = 1)
+  int cplx;      // Im(alpha) or p not zero
+};
+
+// kind, k, alpha, beta as KernelParams holds them (kind 0: S, 1 and 3: D form, 2: CFIE).
+LCQ_HD FxKernel fx_kernel(int kind, double kr, double ki, double ar, double ai, double br,
+                          double bi) {
+  FxKernel f;
+  if (kind != 2) {
+    ar = kind == 0 ? 0.0 : 1.0;
+    ai = 0.0;
+    br = kind == 0 ? 1.0 : 0.0;
+    bi = 0.0;
+  }
+  f.single = kind == 0;
+  f.neg = kr < 0.0;
+  int e;
+  // kr / (2 pi) and ki / ln 2 to 58 bits: 2^64 / (2 pi) and 2^62 / ln 2 times the mantissas
+  u64 m = (u64)fx_mant(fabs(kr), &e);
+  m = fx_umul(m, 0x28be60db9391054aull);
+  for (f.ek = e; m != 0 && m < (1ull << 61); m <<= 1) --f.ek;
+  f.kt = m;
+  m = (u64)fx_mant(ki, &e);
+  m = fx_umul(m, 0x5c551d94ae0bf85eull);
+  for (f.ed = e + 2; m != 0 && m < (1ull << 61); m <<= 1) --f.ed;
+  f.kd = m;
+  const double p = ar * ki + ai * kr, q = ai * ki - ar * kr;
+  int e1, e2;
+  fx_mant(ar, &e1);
+  fx_mant(ai, &e2);
+  f.ea = fx_max(e1, e2);
+  f.ar = fx_split(fx_fix(ar, f.ea));
+  f.ai = fx_split(fx_fix(ai, f.ea));
+  fx_mant(p, &e1);
+  fx_mant(q, &e2);
+  f.ep = fx_max(e1, e2);
+  f.p = fx_split(fx_fix(p, f.ep));
+  f.q = fx_split(fx_fix(q, f.ep));
+  fx_mant(br, &e1);
+  fx_mant(bi, &e2);
+  f.eb = fx_max(e1, e2);
+  f.br = fx_split(fx_fix(br, f.eb));
+  f.bi = fx_split(fx_fix(bi, f.eb));
+  f.cplx = ai != 0.0 || p != 0.0;
+  return f;
+}
+
+
+// Sine table: (cos, sin)(2 pi j / 4096) 2^62 for j = 0..1023 (one quadrant), and the decay
+// table 2^(-j / 1024) 2^62.
+constexpr int kFxTab = 1024;
+struct FxCs {
+  u64 c, s;
+};
+struct FxTables {
+  const FxCs* cs;
+  const u64* dec;
+};
+
+// |cos|, |sin| 2^62 of the phase ph 2^-64 turns, with their
+// signs (bit 0: cos negative, bit 1: sin negative).  The top 12 bits choose quadrant and table
+// entry, the other 52 (t < 2^-12 turns) a Taylor step: 1 - cos through t^4, sin through t^5 (the
+// next terms are below 2^-66 and 2^-73), combined by the addition theorems with positive
+// numbers only.  Absolute error below 2^-60.
+LCQ_HD void fx_sincos(u64 ph, const FxCs* __restrict__ tab, u64* cs, u64* sn, int* sign) {
+  const uint32_t top = fx_hi(ph);
+  const int quad = (int)(top >> 30);
+#ifdef __CUDA_ARCH__
+  const ulonglong2 e = __ldg(reinterpret_cast<const ulonglong2*>(tab) + ((top >> 20) & 1023u));
+  const u64 C = e.x, S = e.y;
+#else
+  const u64 C = tab[(top >> 20) & 1023u].c, S = tab[(top >> 20) & 1023u].s;
+#endif
+  const u64 t = ph & 0xfffffffffffffull;              // 2^-64 turns, below 2^52
+  const uint32_t th = (uint32_t)(t >> 21), tl = (uint32_t)t & 0x1fffffu;
+  const u64 t2 = fx_wide(th, th) + (fx_wide(th, tl) >> 20);   // t^2, unit 2^-86
+  const uint32_t t2h = fx_hi(t2);                             // unit 2^-54, below 2^30
+  // 1 - cos: 2 pi^2 t^2 - (2 pi^4 / 3) t^4, unit 2^-69
+  u64 u = fx_umul(t2, 0x9de9e64df22efull);                    // 2 pi^2 2^47
+  const uint32_t v = fx_hi(fx_wide(t2h, t2h));                // unit 2^-76
+  u -= fx_hi(fx_wide(v, 0x81e0f841u));                        // (2 pi^4 / 3) 2^25
+  // sin: t (2 pi - (4 pi^3 / 3) t^2 + (4 pi^5 / 15) t^4), unit 2^-69
+  uint32_t c1 = 0xa55de731u;                                  // (4 pi^3 / 3) 2^26
+  c1 -= fx_hi(fx_wide(t2h, 0xa335e33cu)) >> 21;               // (4 pi^5 / 15) 2^25
+  const u64 P = 0x1921fb54442d1847ull - (fx_wide(t2h, c1) >> 22);  // 2 pi 2^58
+  const u64 s = fx_umul(t << 11, P);
+  const u64 tc = fx_wide(fx_hi(C), fx_lo(u)) + fx_wide(fx_lo(C), fx_hi(u)) +
+                 fx_wide(fx_hi(S), fx_lo(s)) + fx_wide(fx_lo(S), fx_hi(s));
+  const u64 dc = fx_wide(fx_hi(C), fx_hi(u)) + fx_wide(fx_hi(S), fx_hi(s)) + (u64)fx_hi(tc);
+  const u64 a = C + 1 - (dc >> 5);  // the unit keeps rounding from going below 0
+  const u64 b = S + (fx_umul(C, s) >> 5) - (fx_umul(S, u) >> 5);
+  const bool odd = quad & 1;
+  *cs = odd ? b : a;
+  *sn = odd ? a : b;
+  *sign = (int)(((quad + 1) >> 1) & 1) | (quad & 2);
+}
+
+// 2^(-x) with x = n + f, f = fr 2^-64: the factor 2^-f 2^62 (table and Taylor terms through x^4).
+LCQ_HD u64 fx_exp2n(u64 fr, const u64* __restrict__ tab) {
+  const uint32_t j = (uint32_t)(fr >> 54);
+#ifdef __CUDA_ARCH__
+  const u64 T = __ldg(tab + j);
+#else
+  const u64 T = tab[j];
+#endif
+  // y = tau ln 2, tau = low 54 bits 2^-64 < 2^-10; unit 2^-72
+  const u64 y = fx_umul((fr & 0x3fffffffffffffull) << 9, 0x58b90bfbe8e7bcd6ull);  // ln 2, 2^63
+  // 1 - e^-y = y - y^2/2 + y^3/6 - y^4/24, unit 2^-72
+  const uint32_t yh = fx_hi(y << 1);                          // unit 2^-41
+  const u64 y2 = fx_umul(y << 1, y << 1);                     // y^2, unit 2^-82
+  const uint32_t y2h = (uint32_t)(y2 >> 31);                  // unit 2^-51
+  const uint32_t y3 = fx_hi(fx_wide(y2h, yh));                // unit 2^-60
+  const uint32_t y4 = fx_hi(fx_wide(y2h, y2h));               // unit 2^-70
+  u64 w = y - (y2 >> 11) + (fx_wide(y3, 0xaaaaaaabu) >> 22) -
+                fx_hi(fx_wide(y4, 0x2aaaaaabu));
+  return T - (fx_umul(T, w) >> 8);
+}
+
+// An integer v times 2^e as FP64, rounded to nearest (below the normal range zero, overflow
+// infinity).  INT: by integer instructions (ties away from zero), where the FP64 pipe is the
+// busier one; else by the conversion instruction, which runs on that pipe.
+template <bool INT>
+LCQ_HD double fx_pack(i64 v, int e) {
+  u64 b;
+  int ex;
+  if (INT) {
+    const u64 sg = (u64)(v >> 63);
+    const u64 m = ((u64)v ^ sg) - sg;
+#ifdef __CUDA_ARCH__
+    const int lz = __clzll((long long)m);
+#else
+    const int lz = m == 0 ? 64 : __builtin_clzll(m);
+#endif
+    if (lz > 63) return 0.0;
+    ex = e + 1086 - lz;                                 // exponent field of the leading bit
+    b = ((m << lz) >> 11) + (((m << lz) >> 10) & 1ull);  // 53 bits, the leading one included
+    b += ((u64)(uint32_t)(ex - 1) << 52) | (sg & 0x8000000000000000ull);
+  } else {
+    if (v == 0) return 0.0;
+    b = fx_bits((double)v);
+    ex = (int)((b >> 52) & 0x7ff) + e;
+    b += (u64)(i64)e << 52;
+  }
+  if ((unsigned)(ex - 1) >= 2045u)
+    return fx_double(((u64)v & 0x8000000000000000ull) | (ex <= 0 ? 0ull : 0x7ff0000000000000ull));
+  return fx_double(b);
+}
+
+// The kernel value of one pair from d = x - X (FP64).  False (and nothing written) for
+// arguments that it does not cover: |d| outside [2^-300, 2^300] (zero among them), a phase
+// above 2^24 turns, a decay above 2^9 halvings, values that are not finite.  With env the
+// rounding envelope |G| Jw (eb + ea |1 - ikr| R / r^2) in FP32 (fk: |kr|, fki: ki, fe = eb, fa =
+// ea R, fw = W in FP32).
+template <bool INT>
+LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1, double d2,
+                    const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
+                    float fki, float feb, float feaR, float fw) {
+  const u64 b0 = fx_bits(d0), b1 = fx_bits(d1), b2 = fx_bits(d2);
+  const int x0 = (int)(fx_hi(b0) & 0x7fffffffu) >> 20, x1 = (int)(fx_hi(b1) & 0x7fffffffu) >> 20,
+            x2 = (int)(fx_hi(b2) & 0x7fffffffu) >> 20;
+  const int ex = fx_max(x0, fx_max(x1, x2));
+  const int sh = ex - 1022 + K.ek + 8;
+  if ((unsigned)(ex - 723) > 600u || sh > 30 || ew > kFxBad) return false;
+  const int E = ex - 1022;
+  // d = D 2^(E - 62)
+  i64 D[3];
+  {
+    const u64 b[3] = {b0, b1, b2};
+    const int xs[3] = {x0, x1, x2};
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; ++c) {
+      const u64 m = ((b[c] & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
+      const int s = fx_min(ex - xs[c], 63);
+      const i64 v = (i64)(m >> s);
+      const i64 g = (i64)b[c] >> 63;
+      D[c] = v ^ g;
+    }
+  }
+  const FxS D0 = fx_split(D[0]), D1 = fx_split(D[1]), D2 = fx_split(D[2]);
+  // r^2 = r2 2^(2E - 60), r2 in [2^58, 3 2^60]
+  const i64 cr = fx_swide(D0.h, D0.l) + fx_swide(D1.h, D1.l) + fx_swide(D2.h, D2.l);
+  const u64 r2 = (u64)(fx_swide(D0.h, D0.h) + fx_swide(D1.h, D1.h) + fx_swide(D2.h, D2.h) +
+                       (cr >> 30));
+  // 1/r = RI 2^(-61 - E): Y = 2^60 / sqrt(r2) to 22 bits from the special function unit, its
+  // residual e = 1 - r2 Y^2 exactly enough, and RI = Y 2^31 (1 + e/2 + 3 e^2 / 8)
+  const float f = (float)fx_hi(r2);
+#ifdef __CUDA_ARCH__
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
+  const uint32_t Y = __float2uint_rz(y * 17592186044416.0f);
+#else
+  const float y = 1.0f / sqrtf(f);
+  const uint32_t Y = (uint32_t)(y * 17592186044416.0f);
+#endif
+  const u64 G = fx_umul32(r2, Y);                       // sqrt(r2) 2^28
+  const i64 e1 = (i64)((1ull << 56) - fx_umul32(G, Y));  // unit 2^-56
+  const int e2 = (int)(e1 >> 8);
+  const i64 c1 = (e1 + (i64)(((int)(fx_swide(e2, e2) >> 32) * 3) >> 10)) >> 1;
+  const u64 RI = ((u64)Y << 31) + (u64)(((i64)(Y >> 4) * c1) >> 21);
+  const u64 R = fx_umul(r2 << 1, RI) << 4;              // r = R 2^(E - 62)
+  // the phase in turns 2^-64 and e^{ikr}
+  u64 ph = fx_umul(R, K.kt);                            // kr / 2 pi = ph 2^(E + ek - 60)
+  ph = sh >= 4 ? ph << (sh - 4) : ph >> fx_min(4 - sh, 63);
+  u64 cs, sn;
+  int sg;
+  fx_sincos(ph, tab.cs, &cs, &sn, &sg);
+  if (K.neg) sg ^= 2;
+  // g = W e^{-ki r} / r (single) or / r^2
+  u64 h = fx_umul(RI, w << 1);                          // W / r = h 2^(ew - E - 60)
+  int eg = ew - E - 60;
+  if (K.kd != 0) {
+    const u64 x = fx_umul(R, K.kd);                     // ki r / ln 2 = x 2^(E + ed - 60)
+    const int sx = E + K.ed + 4;                        // to unit 2^-64
+    int nn = 0;
+    u64 fr;
+    if (sx >= 0) {
+      if (sx > 13) return false;
+      nn = sx == 0 ? 0 : (int)(x >> (64 - sx));
+      fr = x << sx;
+    } else {
+      fr = x >> fx_min(-sx, 63);
+    }
+    h = fx_umul(h, fx_exp2n(fr, tab.dec) << 1) << 1;
+    eg -= nn;
+  }
+  if (env) {
+    // 1/r and r in FP32 from the estimate (E within 300: out-of-range scales saturate)
+    const int eb = fx_max(fx_min(E, 120), -120);
+#ifdef __CUDA_ARCH__
+    const float sc = __int_as_float((127 - eb) << 23);
+    const float rs = __int_as_float((127 + eb) << 23);
+#else
+    const float sc = ldexpf(1.0f, -eb), rs = ldexpf(1.0f, eb);
+#endif
+    const float fri = y * 16384.0f * sc, fr = f * y * rs * 6.103515625e-05f * 1.0f;
+    const float fo = fki * fr + 1.0f, f1 = fk * fr;
+    const float fab = sqrtf(fo * fo + f1 * f1);
+    float g = fri * fw;
+    if (fki != 0.0f) g *= expf(-fki * fr);
+    *env = g * (feb + feaR * fab * fri * fri);
+  }
+  const i64 ma = -(i64)(sg & 1), mb = -(i64)(sg >> 1);
+  if (K.single) {
+    const u64 a = fx_umul(cs, h << 2), b = fx_umul(sn, h << 2);   // unit 2^eg
+    *re = fx_pack<INT>(((i64)a ^ ma) - ma, eg);
+    *im = fx_pack<INT>(((i64)b ^ mb) - mb, eg);
+    return true;
+  }
+  const u64 g = fx_umul(RI, h << 2);                    // W / r^2 = g 2^(eg - E + 1)
+  const FxS ec = fx_split((i64)fx_umul(cs, g << 2) ^ ma);   // e^{ikr} W / r^2, the same unit
+  const FxS es = fx_split((i64)fx_umul(sn, g << 2) ^ mb);
+  // c = n.d / r, unit 2^-62
+  const i64 n01 = fx_swide(n[0].h, D0.l) + fx_swide(n[0].l, D0.h) + fx_swide(n[1].h, D1.l) +
+                  fx_swide(n[1].l, D1.h);
+  const i64 n2 = fx_swide(n[2].h, D2.l) + fx_swide(n[2].l, D2.h);
+  const i64 nd = fx_swide(n[0].h, D0.h) + fx_swide(n[1].h, D1.h) + fx_swide(n[2].h, D2.h) +
+                 (n01 >> 31) + (n2 >> 31);              // n.d 2^(60 - E)
+  const FxS c = fx_split(fx_smul(fx_split(nd << 2), fx_split((i64)RI)) << 3);
+  // A and B, unit 2^(eA - 60)
+  const FxS Rs = fx_split((i64)R);
+  const int eb = K.eb + E, ep = K.ep + E;
+  const int eA = fx_max(K.ea, fx_max(eb, ep));
+  const int sb = eA - eb, sa = eA - K.ea, sp = eA - ep;
+  i64 A = fx_sra(fx_smul(K.br, Rs), sb) + fx_sra(fx_smul(K.ar, c), sa);
+  i64 B = fx_sra(fx_smul(K.bi, Rs), sb) +
+          fx_sra(fx_smul(fx_split(fx_smul(K.q, Rs) << 2), c), sp);
+  if (K.cplx) {
+    A += fx_sra(fx_smul(fx_split(fx_smul(K.p, Rs) << 2), c), sp);
+    B += fx_sra(fx_smul(K.ai, c), sa);
+  }
+  const FxS As = fx_split(A), Bs = fx_split(B), Bn = {-Bs.h, -Bs.l};
+  const int ev = eA + eg - E + 2;
+  *re = fx_pack<INT>(fx_dot2(As, ec, Bn, es), ev);
+  *im = fx_pack<INT>(fx_dot2(As, es, Bs, ec), ev);
+  return true;
+}
+
+}  // namespace lcq

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/lcq.h"
+#include "lcq_fx.cuh"
 
 namespace lcq {
 
@@ -43,11 +44,12 @@ struct KernelParams {
   double ar, ai;     // alpha
   double br, bi;     // beta
   double eb, ea;     // rounding-envelope weights: |beta| and |alpha| (1,0 for S; 0,1 for D)
+  FxKernel fx;       // the same constants in fixed point (lcq_fx.cuh)
 };
 
 inline KernelParams make_kernel_params(int kind, double kr, double ki, double ar, double ai,
                                        double br, double bi) {
-  KernelParams kp{kind, kr, ki, ar, ai, br, bi, 0.0, 0.0};
+  KernelParams kp{kind, kr, ki, ar, ai, br, bi, 0.0, 0.0, fx_kernel(kind, kr, ki, ar, ai, br, bi)};
   if (kind == 0) {
     kp.ar = kp.ai = kp.br = kp.bi = 0.0;
     kp.eb = 1.0;

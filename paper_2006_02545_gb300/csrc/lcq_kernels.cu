@@ -71,11 +71,12 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
 // (tiles staged through shared memory): block (b, s) sums part s of gridDim.y equal parts of
 // the sources of target block b into part[s][t], and k_csr_apply adds the parts in order.  Few
 // targets alone leave the chip idle (1000 targets are 8 blocks on 152 SMs), so the launch cuts
-// the sources until there are several waves of blocks (far_sum_parts): 1000 targets and 129,000
-// sources 327 ms with one part, 10 ms so; 8,960 and 26,000 66.2 and 15.7 ms.  Kernel values by kernel_eval_tc (table sincos and the
-// Newton-refined reciprocal square root: FP64 throughout, about 48 FP64 instructions per
-// pair for the CFIE), or with fold by kernel_eval_fold on sources that carry the kernel
-// constants (about 41).
+// the sources until there are several waves of blocks (far_sum_parts).
+// The kernel values are fixed-point (fx_eval): of FP64 there are only the difference x - X and
+// the four multiply-adds of the density (448 cycles of the FP64 pipe a pair and warp, beside
+// about 440 integer instructions for the single layer).  35,840 targets x 127,606 sources, CFIE:
+// 407 ms with FP64 kernel values (41 FP64 instructions a pair), 129 ms so; 8,960 x 25,920, S: 15.7
+// and 4.4 ms.  More warps per SM (128, 96, 80, 64 registers) and two sources a step: within 3%.
 // The sources of an on-surface target's own patch are skipped (their contribution is
 // carried entirely by the self correction).  In a batch of independent surfaces a target
 // sums only its own surface's sources [gsrc[g], gsrc[g+1]) with that surface's kernel.
@@ -89,14 +90,14 @@ __global__ void __launch_bounds__(kFarThreads) k_far_sum(const double* __restric
                                                       const GroupParams* __restrict__ grp,
                                                       const int64_t* __restrict__ gsrc,
                                                       const double* __restrict__ tnrm,
-                                                      cplx* __restrict__ part, bool fold) {
-  __shared__ double s[10][kFarThreads];
+                                                      cplx* __restrict__ part) {
+  __shared__ ulonglong2 s[5][kFarThreads];  // X0 X1 | X2 n0 | n1 n2 | w ew | density
   __shared__ unsigned long long blo, bhi;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double x0 = 0, x1 = 0, x2 = 0;
   int64_t skip0 = -1, skip1 = -1, lo = 0, hi = 0;
-  double nx[3] = {0.0, 0.0, 0.0};
-  KernelParams kt = kp;
+  FxS nx[3] = {{0, 0}, {0, 0}, {0, 0}};
+  const KernelParams* kt = &kp;
   if (threadIdx.x == 0) {
     blo = ~0ull;
     bhi = 0ull;
@@ -106,11 +107,8 @@ __global__ void __launch_bounds__(kFarThreads) k_far_sum(const double* __restric
     x0 = tgt[t];
     x1 = tgt[NT + t];
     x2 = tgt[2 * NT + t];
-    if (tnrm) {
-      nx[0] = tnrm[t];
-      nx[1] = tnrm[NT + t];
-      nx[2] = tnrm[2 * NT + t];
-    }
+    if (tnrm)  // S': the double-layer form with -n_x in the place of the source's normal
+      for (int c = 0; c < 3; ++c) nx[c] = fx_split(fx_fix(-tnrm[c * NT + t], 0));
     const int tp = tpatch[t];
     if (tp >= 0) {
       skip0 = src_off[tp];
@@ -119,7 +117,7 @@ __global__ void __launch_bounds__(kFarThreads) k_far_sum(const double* __restric
     hi = n_over;
     if (tgroup) {
       const int g = tgroup[t];
-      kt = grp[g].kp;
+      kt = &grp[g].kp;
       lo = gsrc[g];
       hi = gsrc[g + 1];
     }
@@ -130,32 +128,46 @@ __global__ void __launch_bounds__(kFarThreads) k_far_sum(const double* __restric
   const int64_t all = (int64_t)bhi - (int64_t)blo;
   const int64_t b0 = (int64_t)blo + all * blockIdx.y / gridDim.y;
   const int64_t b1 = (int64_t)blo + all * (blockIdx.y + 1) / gridDim.y;
-  const KernelParamsF kf = to_f32(kt);
-  const bool has_ki = kt.ki != 0.0;
-  float env;  // not used: the far sum needs no rounding envelope
+  const FxKernel kf = kt->fx;
+  const FxTables tab = fx_tables();
   double re = 0.0, im = 0.0;
-  const int rows = fold ? 10 : 9;
   for (int64_t s0 = b0; s0 < b1; s0 += kFarThreads) {
     __syncthreads();
     const int64_t q = s0 + threadIdx.x;
-    for (int c = 0; c < rows; ++c) s[c][threadIdx.x] = q < b1 ? src[c * n_over + q] : 0.0;
+    if (q < b1) {
+      auto row = [&](int c) { return (u64)__double_as_longlong(src[c * n_over + q]); };
+      s[0][threadIdx.x] = make_ulonglong2(row(0), row(1));
+      s[1][threadIdx.x] = make_ulonglong2(row(2), row(3));
+      s[2][threadIdx.x] = make_ulonglong2(row(4), row(5));
+      s[3][threadIdx.x] = make_ulonglong2(row(6), row(9));
+      s[4][threadIdx.x] = make_ulonglong2(row(7), row(8));
+    }
     __syncthreads();
     const int cnt = (int)min((int64_t)kFarThreads, b1 - s0);
-    if (t < NT)
-      for (int k = 0; k < cnt; ++k) {
-        const int64_t qq = s0 + k;
-        if (qq < lo || qq >= hi || (qq >= skip0 && qq < skip1)) continue;
-        const cplx g =
-            fold ? kernel_eval_fold(kt.kind, kt.kr, kf, g_sct, x0, x1, x2, s[0][k], s[1][k],
-                                    s[2][k], s[3][k], s[4][k], s[5][k], s[6][k], s[9][k], 0.0f,
-                                    0.0f, &env)
-                 : kernel_eval_tc(kt, kf, g_sct, x0, x1, x2, s[0][k], s[1][k], s[2][k], s[3][k],
-                                  s[4][k], s[5][k], s[6][k], 0.0f, 0.0f, &env, nx, has_ki);
-        re = fma(g.re, s[7][k], re);
-        re = fma(-g.im, s[8][k], re);
-        im = fma(g.re, s[8][k], im);
-        im = fma(g.im, s[7][k], im);
+    // this target's sources of the tile: [ka, kb) without [kc, kd)
+    const int ka = (int)max(min(lo - s0, (int64_t)cnt), (int64_t)0), kb = (int)min(hi - s0, (int64_t)cnt);
+    const int kc = (int)max(min(skip0 - s0, (int64_t)cnt), (int64_t)0);
+    const int kd = (int)max(min(skip1 - s0, (int64_t)cnt), (int64_t)0);
+    for (int k = 0; k < cnt; ++k) {
+      if (k < ka || k >= kb || (k >= kc && k < kd)) continue;
+      const ulonglong2 a = s[0][k], b = s[1][k], c = s[2][k], d = s[3][k];
+      FxS n[3] = {fx_unjoin(b.y), fx_unjoin(c.x), fx_unjoin(c.y)};
+      if (tnrm) {
+        n[0] = nx[0];
+        n[1] = nx[1];
+        n[2] = nx[2];
       }
+      const double d0 = x0 - fx_double(a.x), d1 = x1 - fx_double(a.y), d2 = x2 - fx_double(b.x);
+      cplx g;
+      if (!fx_eval<true>(kf, tab, d0, d1, d2, n, d.x, (int)d.y, &g.re, &g.im, nullptr, 0.0f, 0.0f,
+                         0.0f, 0.0f, 0.0f))
+        g = fx_fallback(*kt, d0, d1, d2, n[0], n[1], n[2], d.x, (int)d.y, 0.0, nullptr);
+      const double sr = fx_double(s[4][k].x), si = fx_double(s[4][k].y);
+      re = fma(g.re, sr, re);
+      re = fma(-g.im, si, re);
+      im = fma(g.re, si, im);
+      im = fma(g.im, sr, im);
+    }
   }
   if (t < NT) part[blockIdx.y * NT + t] = {re, im};
 }
@@ -352,8 +364,8 @@ bool launch_v2c(int d, const LaunchCommon& lc, const int* plist, int count, cons
 }
 bool launch_far_src(int d, const LaunchCommon& lc, const int* plist, int count, const Dev& dv,
                     const double* Vt, const int32_t* qv, const int64_t* src_off, const void* sigma,
-                    double* src, int64_t n_over, const KernelParams& kp, bool fold) {
-  return dispatch<FarSrcL>(d, lc, plist, count, dv, Vt, qv, src_off, sigma, src, n_over, kp, fold);
+                    double* src, int64_t n_over, bool fx) {
+  return dispatch<FarSrcL>(d, lc, plist, count, dv, Vt, qv, src_off, sigma, src, n_over, fx);
 }
 // Parts that the far sum's sources are cut into: enough blocks for about four waves of eight
 // on every SM, at least 32 sources each.
@@ -367,12 +379,12 @@ int far_sum_parts(int num_sms, int64_t NT, int64_t n_over) {
 void launch_far_sum(const LaunchCommon& lc, const double* tgt, int64_t NT, const double* src,
                     int64_t n_over, const KernelParams& kp, const int32_t* tpatch,
                     const int64_t* src_off, const int32_t* tgroup, const GroupParams* grp,
-                    const int64_t* gsrc, const double* tnrm, void* part, int parts, bool fold) {
+                    const int64_t* gsrc, const double* tnrm, void* part, int parts) {
   const int64_t g = (NT + kFarThreads - 1) / kFarThreads;
   if (g <= 0) return;
   ++*lc.launches;
   k_far_sum<<<dim3((unsigned)g, (unsigned)parts), kFarThreads, 0, lc.stream>>>(
-      tgt, NT, src, n_over, kp, tpatch, src_off, tgroup, grp, gsrc, tnrm, (cplx*)part, fold);
+      tgt, NT, src, n_over, kp, tpatch, src_off, tgroup, grp, gsrc, tnrm, (cplx*)part);
 }
 void launch_widen_c64(const LaunchCommon& lc, const void* in, int64_t n, void* out) {
   if (n <= 0) return;
