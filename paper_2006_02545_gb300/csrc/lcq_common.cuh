@@ -96,8 +96,39 @@ struct Cfg {
   static constexpr int BS = n + 1;
   static constexpr int TT = 16;
   // doubles of shared workspace used by block_moments
-  static constexpr int WS = CH * BS + 7 * CH + 3 * TT * CH + 6 * TT;
+  static constexpr int WS = CH * BS + 8 * CH + 3 * TT * CH + 6 * TT;
 };
+
+// Unit normal of a target (S') as fx_eval takes a node's, negated: S' is the double-layer
+// form with -n_x in the place of the source's normal.
+template <class TA>
+__device__ __forceinline__ void load_fx_normal(const TA& ta, int i, const double* xrel, u64* out) {
+  double n[3];
+  ta.nrm(i, xrel, n);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[c] = fx_join(fx_split(fx_fix(-n[c], 0)));
+}
+
+// Kernel value of target x and the node at X (stride sx), normal nn (stride sn), W = w 2^(ew-62);
+// env: the rounding envelope (FP32) for patch radius R.
+__device__ __forceinline__ cplx fx_value(const KernelParams& kp, const FxKernel& fx,
+                                         const KernelParamsF& kf, const FxTables& tab,
+                                         const double* x, const double* X, int sx, const u64* nn,
+                                         int sn, u64 w, int ew, float R, float* env) {
+  const double d0 = x[0] - X[0], d1 = x[1] - X[sx], d2 = x[2] - X[2 * sx];
+  const FxS n[3] = {fx_unjoin(nn[0]), fx_unjoin(nn[sn]), fx_unjoin(nn[2 * sn])};
+  cplx g;
+  // W in FP32 for the envelope: its leading 24 bits at its exponent
+  float fw = 0.0f;
+  if (env) {
+    const int e = min(max(ew, -120), 120);
+    fw = (float)(uint32_t)(w >> 32) * 9.31322575e-10f * __int_as_float((127 + e) << 23);
+  }
+  if (!fx_eval<false>(fx, tab, d0, d1, d2, n, w, ew, &g.re, &g.im, env, kf.kr, kf.ki, kf.eb,
+                      kf.ea * R, fw))
+    g = fx_fallback(kp, d0, d1, d2, n[0], n[1], n[2], w, ew, (double)R, env);
+  return g;
+}
 
 struct SegMap {
   double ax, ay, e1x, e1y, e2x, e2y, det;
@@ -122,16 +153,19 @@ __device__ void block_moments(const double* cf, const double* cfd, const double*
   using C = Cfg<D>;
   double* B = sm;
   double* Xs = B + C::CH * C::BS;
-  double* Ns = Xs + 3 * C::CH;
-  double* Js = Ns + 3 * C::CH;
-  cplx* G = reinterpret_cast<cplx*>(Js + C::CH);
+  u64* Ns = reinterpret_cast<u64*>(Xs + 3 * C::CH);  // nodes as fx_eval takes them
+  u64* Ws = Ns + 3 * C::CH;
+  u64* Es = Ws + C::CH;
+  cplx* G = reinterpret_cast<cplx*>(Es + C::CH);
   double* Ev = reinterpret_cast<double*>(G + C::TT * C::CH);
   double* tx = Ev + C::TT * C::CH;
-  double* tn = tx + 3 * C::TT;  // target normals (S')
+  u64* tn = reinterpret_cast<u64*>(tx + 3 * C::TT);  // target normals (S')
   static_assert(C::n < C::BS, "the basis rows need a spare column");
   (void)ostride;
   const KernelParamsF kf = to_f32(kp);
-  const bool has_ki = kp.ki != 0.0;
+  const FxKernel& fx = kp.fx;  // read at its uses: as a register copy it spills (224 B)
+  const FxTables tab = fx_tables();
+  const float fR = (float)R;
   const int total = nseg * Q;
   // The rules are conical products, rows of mr nodes sharing v, and every segment map
   // here keeps v a function of the rule's v alone (e1y = 0: T0 and all its midpoint
@@ -176,13 +210,17 @@ __device__ void block_moments(const double* cf, const double* cfd, const double*
       }
       if (ENV) B[ql * C::BS + C::n] = 1.0;  // the envelope's column
       cross3(Xu, Xv, Nn);
-      const double J = sqrt(Nn[0] * Nn[0] + Nn[1] * Nn[1] + Nn[2] * Nn[2]);
+      FxS nn[3];
+      u64 wm;
+      int ew;
+      fx_make_node(Nn, w, nn, &wm, &ew);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         Xs[c * C::CH + ql] = X[c];
-        Ns[c * C::CH + ql] = Nn[c] * w;
+        Ns[c * C::CH + ql] = fx_join(nn[c]);
       }
-      Js[ql] = J * w;
+      Ws[ql] = wm;
+      Es[ql] = (u64)(i64)ew;
     }
     __syncthreads();
     for (int t0 = 0; t0 < T; t0 += C::TT) {
@@ -193,28 +231,18 @@ __device__ void block_moments(const double* cf, const double* cfd, const double*
         xp[0] -= cen[0];
         xp[1] -= cen[1];
         xp[2] -= cen[2];
-        if (kp.kind == 3) ta.nrm(t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
+        if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
       }
       __syncthreads();
-      // kernel values by the table sincos and the Newton-refined 1/sqrt; with ENV the
-      // FP64 form with its rounding envelope
+      // kernel values in fixed point (lcq_fx.cuh); with ENV also their FP32 rounding envelope
       for (int e = threadIdx.x; e < nt * nch; e += blockDim.x) {
         const int i = e / nch, ql = e - i * nch;
-        if (ENV) {
-          double ev = 0.0;
-          G[i * C::CH + ql] = kernel_eval(kp, tx[3 * i], tx[3 * i + 1], tx[3 * i + 2], Xs[ql],
-                                          Xs[C::CH + ql], Xs[2 * C::CH + ql], Ns[ql],
-                                          Ns[C::CH + ql], Ns[2 * C::CH + ql], Js[ql], R, &ev,
-                                          tn + 3 * i);
-          Ev[i * C::CH + ql] = ev;
-        } else {
-          float unused;
-          G[i * C::CH + ql] = kernel_eval_tc(kp, kf, g_sct, tx[3 * i], tx[3 * i + 1],
-                                             tx[3 * i + 2], Xs[ql], Xs[C::CH + ql],
-                                             Xs[2 * C::CH + ql], Ns[ql], Ns[C::CH + ql],
-                                             Ns[2 * C::CH + ql], Js[ql], 0.0f, 0.0f, &unused,
-                                             tn + 3 * i, has_ki);
-        }
+        const u64* nn = kp.kind == 3 ? tn + 3 * i : Ns + ql;
+        const int st = kp.kind == 3 ? 1 : C::CH;
+        float ev = 0.0f;
+        G[i * C::CH + ql] = fx_value(kp, fx, kf, tab, tx + 3 * i, Xs + ql, C::CH, nn, st, Ws[ql],
+                                     (int)Es[ql], fR, ENV ? &ev : nullptr);
+        if (ENV) Ev[i * C::CH + ql] = (double)ev;
       }
       __syncthreads();
       // one thread per (target, nm), outputs packed densely; with ENV the extra index nm = n
@@ -437,16 +465,20 @@ __device__ void block_moments_tc(const double* cf, const double* cfd, const doub
   float* Nf = reinterpret_cast<float*>(smb + C::OFF_NF);
   int* rowE = reinterpret_cast<int*>(smb + C::OFF_ROWE);
   double* tx = reinterpret_cast<double*>(smb + C::OFF_TX);
-  double* tn = tx + 3 * C::TT;
+  u64* tn = reinterpret_cast<u64*>(tx + 3 * C::TT);
   int* colinfo = reinterpret_cast<int*>(smb + C::OFF_CI);  // (piece << 16) | node, 0xffff: pad
   int* pcs = reinterpret_cast<int*>(smb + C::OFF_PC);      // [piece][sg, l0, nq, po, row0, rb, first]
   const KernelParamsF kf = to_f32(kp);
   const float fR = f32_bits(R);
   const bool mixed = form == 1;
-  const bool has_ki = kp.ki != 0.0;
-  // real k, kinds S, D and CFIE with a real alpha: constants folded into the node data
-  const bool fold = !mixed && !has_ki && kp.kind <= 2 && kp.ai == 0.0;
-  const bool ffe = fold && form == 2;  // two-float kernel values
+  // two-float kernel values: real k, kinds S, D and CFIE with a real alpha, whose constants are
+  // folded into the node data
+  const bool ffe = form == 2 && kp.ki == 0.0 && kp.kind <= 2 && kp.ai == 0.0;
+  const FxKernel& fx = kp.fx;  // read at its uses: as a register copy it spills (224 B)
+  const FxTables tab = fx_tables();
+  u64* Nfx = reinterpret_cast<u64*>(Ns);  // nodes as fx_eval takes them, in the FP64 slots
+  u64* Wfx = reinterpret_cast<u64*>(Js);
+  u64* Efx = reinterpret_cast<u64*>(Ks);
   const float escale = mixed ? (float)(kF32Floor / kRoundingFloor)
                              : ffe ? (float)(kTwoFloatFloor / kRoundingFloor) : 1.0f;
   const ff krf = ff_of(kp.kr);
@@ -562,27 +594,32 @@ __device__ void block_moments_tc(const double* cf, const double* cfd, const doub
           for (int idx = 0; idx < n; ++idx) store_basis_slices<D>(Bsl, idx, p, K[idx]);
         }
         cross3(Xu, Xv, Nn);
-        const double N2 = fma(Nn[0], Nn[0], fma(Nn[1], Nn[1], Nn[2] * Nn[2]));
-        const double Jw = N2 > 0.0 ? N2 * rsqrt_nr(N2) * w : 0.0;
-        const double wn = fold ? w * fa_n : w;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          Xs[c * C::CH + p] = X[c];
-          if (ffe) Nff[c * C::CH + p] = ff_of(Nn[c] * wn);
-          else Ns[c * C::CH + p] = Nn[c] * wn;
-        }
-        if (ffe) {
-          Jff[p] = ff_of(Jw * fj_r);
-          Kff[p] = ff_of(Jw * fj_i);
+        for (int c = 0; c < 3; ++c) Xs[c * C::CH + p] = X[c];
+        if (mixed || ffe) {
+          const double N2 = fma(Nn[0], Nn[0], fma(Nn[1], Nn[1], Nn[2] * Nn[2]));
+          const double Jw = N2 > 0.0 ? N2 * rsqrt_nr(N2) * w : 0.0;
+          if (ffe) {
+            const double wn = w * fa_n;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) Nff[c * C::CH + p] = ff_of(Nn[c] * wn);
+            Jff[p] = ff_of(Jw * fj_r);
+            Kff[p] = ff_of(Jw * fj_i);
+            Jf[p] = f32_bits(Jw * kInv4Pi);
+          } else {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) Nf[c * C::CH + p] = (float)(Nn[c] * w);
+            Jf[p] = (float)Jw;
+          }
         } else {
-          Js[p] = fold ? Jw * fj_r : Jw;
-          Ks[p] = fold ? Jw * fj_i : 0.0;
-        }
-        Jf[p] = f32_bits(fold ? Jw * kInv4Pi : Jw);
-        if (mixed) {
+          FxS nn[3];
+          u64 wm;
+          int ew;
+          fx_make_node(Nn, w, nn, &wm, &ew);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) Nf[c * C::CH + p] = (float)(Nn[c] * w);
-          Jf[p] = (float)Jw;
+          for (int c = 0; c < 3; ++c) Nfx[c * C::CH + p] = fx_join(nn[c]);
+          Wfx[p] = wm;
+          Efx[p] = (u64)(i64)ew;
         }
       }
     }
@@ -595,7 +632,7 @@ __device__ void block_moments_tc(const double* cf, const double* cfd, const doub
         xp[0] -= cen[0];
         xp[1] -= cen[1];
         xp[2] -= cen[2];
-        if (kp.kind == 3) ta.nrm(t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
+        if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
       }
       __syncthreads();
       // (2) kernel values and envelopes of the real columns; zeros in the padding ones
@@ -626,14 +663,10 @@ __device__ void block_moments_tc(const double* cf, const double* cfd, const doub
             g = kernel_eval_ff(kp.kind, kp.kr, krf, kf, g_sct, g_sctf, tx[3 * i], tx[3 * i + 1],
                                tx[3 * i + 2], Xs[p], Xs[C::CH + p], Xs[2 * C::CH + p], Np,
                                Jff[p], Kff[p], Jf[p], fR, &ev);
-          } else if (fold) {
-            g = kernel_eval_fold(kp.kind, kp.kr, kf, g_sct, tx[3 * i], tx[3 * i + 1],
-                                 tx[3 * i + 2], Xs[p], Xs[C::CH + p], Xs[2 * C::CH + p], Ns[p],
-                                 Ns[C::CH + p], Ns[2 * C::CH + p], Js[p], Ks[p], Jf[p], fR, &ev);
           } else {
-            g = kernel_eval_tc(kp, kf, g_sct, tx[3 * i], tx[3 * i + 1], tx[3 * i + 2], Xs[p],
-                               Xs[C::CH + p], Xs[2 * C::CH + p], Ns[p], Ns[C::CH + p],
-                               Ns[2 * C::CH + p], Js[p], Jf[p], fR, &ev, tn + 3 * i, has_ki);
+            const u64* nn = kp.kind == 3 ? tn + 3 * i : Nfx + p;
+            g = fx_value(kp, fx, kf, tab, tx + 3 * i, Xs + p, C::CH, nn,
+                         kp.kind == 3 ? 1 : C::CH, Wfx[p], (int)Efx[p], fR, &ev);
           }
           Gs[i * C::CH + p] = g;
         }

@@ -475,7 +475,9 @@ __global__ void __launch_bounds__(128) k_self(Dev dv, const int32_t* __restrict_
       total = off;
     }
     __syncthreads();
-    const KernelParamsF kfs = to_f32(kps);
+    const FxTables tab = fx_tables();
+    FxS nPx[3];  // S': the source's normal replaced by -n_x
+    for (int c = 0; c < 3; ++c) nPx[c] = fx_split(fx_fix(-nP[c], 0));
     chart_taylor<D>(P[0], P[1], cf, krows, tX);  // krows is free until the first chunk
     // the target is the chart's value at the node: x - X(P + delta) = -(dX)
     // chunks of 128 nodes: each thread forms one node's kernel value and basis row in
@@ -514,10 +516,14 @@ __global__ void __launch_bounds__(128) k_self(Dev dv, const int32_t* __restrict_
         kw_geometry_proj<D, false>(P[0] + du, P[1] + dvv, cf, cfd, nullptr, Xu, Xv, Kq);
         chart_chord<D>(tX, du, dvv, dX);
         cross3(Xu, Xv, Nn);
-        const double J = sqrt(Nn[0] * Nn[0] + Nn[1] * Nn[1] + Nn[2] * Nn[2]);
-        float unused;
-        gk = kernel_eval_tc(kps, kfs, g_sct, 0.0, 0.0, 0.0, dX[0], dX[1], dX[2], Nn[0] * w,
-                            Nn[1] * w, Nn[2] * w, J * w, 0.0f, 0.0f, &unused, nP, kps.ki != 0.0);
+        FxS nn[3];
+        u64 wm;
+        int ew;
+        fx_make_node(Nn, w, nn, &wm, &ew);
+        const FxS* nu = kps.kind == 3 ? nPx : nn;
+        if (!fx_eval<false>(kps.fx, tab, -dX[0], -dX[1], -dX[2], nu, wm, ew, &gk.re, &gk.im, nullptr,
+                            0.0f, 0.0f, 0.0f, 0.0f, 0.0f))
+          gk = fx_fallback(kps, -dX[0], -dX[1], -dX[2], nu[0], nu[1], nu[2], wm, ew, 0.0, nullptr);
       } else {
         for (int e = 0; e < n; ++e) Kq[e] = 0.0;
       }
