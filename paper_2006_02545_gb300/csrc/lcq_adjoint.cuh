@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(kThreads) k_grad_rules(
   __shared__ SegMap segs[1];
   __shared__ KernelParams kps;
   __shared__ double red[nwarps * n3];
+  __shared__ double gscr[5 * kGradTile];
   double* Mw = red + (threadIdx.x >> 5) * n3;
   const bool lead = (threadIdx.x & 31) == 0;
   for (int b = blockIdx.x; b < count; b += gridDim.x) {
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(kThreads) k_grad_rules(
                             const cplx c = g[dv.pair_tgt[pl[i]]];
                             return {c.re, -c.im};
                           },
-                          kps, shat, dv.cen + 3 * j, Mw);
+                          kps, shat, dv.cen + 3 * j, Mw, gscr);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < n3; e += blockDim.x) {

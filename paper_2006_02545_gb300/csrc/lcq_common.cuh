@@ -286,128 +286,90 @@ __device__ void block_moments(const double* cf, const double* cfd, const double*
   }
 }
 
-// The split of kernel rows for the tensor-core moments (block_moments_tc below), with the
-// contraction over the nodes on the tensor cores by the exact NS-slice split (lcq_tc.cuh):
-// NS = 8 for FP64 kernel values, NS = 5 for the mixed form's FP32 ones.
-// Chunks never straddle a segment: segment sg's Q nodes are cut into parts of at most
-// TcCfg::CH nodes, each padded with zero columns to a multiple of 16 (the MMA depth), and
-// each chunk's contribution is assembled in FP64 and written (first part) or added.
-// Per chunk: (1) geometry, thread per node: X, N w, J w and the basis row (FP64); (2) per
-// tile of 8 targets: kernel values and envelopes, thread per (target, node); (3) one warp
-// per target splits the Re and Im rows of its kernel values on their own power-of-two
-// scales into NS f16 slices; (4) one warp per n-tile of 8 basis columns slices its basis
-// values (fixed per-column bounds) into MMA fragments and accumulates the diagonals
-// i + j <= 8 (FP64; i + j < 5 for the mixed form) over
-// the chunk's 16-node steps with mma.sync, then assembles and stores the 8 x 8 complex
-// block.  smb: TcCfg<D>::BYTES of shared memory (16-byte aligned); sct: the sincos table.
-// Rows t (Re) and t + 8 (Im) of the kernel values, VPL consecutive columns q0.. per lane,
-// on their own power-of-two scales into NS f16 slices of the swizzled A array (one warp).
-template <int D, int NS, int VPL, class V>
-__device__ __forceinline__ void split_row_pair(const V* re, const V* im, bool on, uint16_t* Asl,
-                                               int t, int q0, int* rowE) {
-  using C = TcCfg<D>;
-  int fr = 0, fi = 0;
-  bool bad = false;
-#pragma unroll
-  for (int v = 0; v < VPL; ++v) {
-    const int a = exp_field(re[v]), b = exp_field(im[v]);
-    bad = bad || exp_nonfinite(a, V()) || exp_nonfinite(b, V());
-    fr = max(fr, a);
-    fi = max(fi, b);
-  }
-  fr = (int)__reduce_max_sync(0xffffffffu, (unsigned)fr);
-  fi = (int)__reduce_max_sync(0xffffffffu, (unsigned)fi);
-  bad = __any_sync(0xffffffffu, bad);
-  const int Er = exp_bound(fr, V()), Ei = exp_bound(fi, V());
-  if ((threadIdx.x & 31) == 0) {
-    rowE[t] = !on ? 0 : (bad ? kPoisonExp : Er);
-    rowE[t + 8] = !on ? 0 : (bad ? kPoisonExp : Ei);
-  }
-#pragma unroll
-  for (int part = 0; part < 2; ++part) {
-    const V* x = part ? im : re;
-    const int E = part ? Ei : Er;
-    const int row = t + 8 * part;
-    unsigned long long M[VPL];
-    uint32_t sg[VPL / 2];
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) M[v] = on ? fix_mag<NS>(x[v], E) : 0ull;
-#pragma unroll
-    for (int v = 0; v < VPL / 2; ++v) sg[v] = sign_bits(x[2 * v], x[2 * v + 1]);
-    uint16_t* dst = Asl + C::swz(row, q0);
-#pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      uint16_t* d = dst + (size_t)i * 16 * C::CH;
-      const uint32_t w0 = half2_ints(slice_of<NS>(M[0], i), slice_of<NS>(M[1], i), sg[0]);
-      if (VPL == 4) {
-        const uint32_t w1 = half2_ints(slice_of<NS>(M[2], i), slice_of<NS>(M[3], i), sg[1]);
-        *reinterpret_cast<uint2*>(d) = make_uint2(w0, w1);
-      } else {
-        *reinterpret_cast<uint32_t*>(d) = w0;
-      }
-    }
-  }
+// A kernel value of a row as slices on the row's power-of-two scale 2^E (|x| < 2^E).
+__device__ __forceinline__ uint2 row_slices(double x, int E) {
+  return slice_bytes(fix_mag<8>(x, E), __double2hiint(x) < 0);
 }
-
-// The 8 slices of basis value K_nm (column idx) of node k into the swizzled B array.
-template <int D>
-__device__ __forceinline__ void store_basis_slices(uint16_t* Bsl, int idx, int k, double v) {
-  using C = TcCfg<D>;
-  const unsigned long long M = fix_mag<8>(v, c_kwexp[idx]);
-  const bool neg = __double2hiint(v) < 0;
-  uint16_t* b = Bsl + C::swz(idx, k);
-#pragma unroll
-  for (int i = 0; i < 8; i += 2) {
-    const uint32_t h = half2_pair(slice_of<8>(M, i), slice_of<8>(M, i + 1), neg);
-    b[(size_t)i * C::NP * C::CH] = (uint16_t)(h & 0xffffu);
-    b[(size_t)(i + 1) * C::NP * C::CH] = (uint16_t)(h >> 16);
-  }
+__device__ __forceinline__ uint2 row_slices(float x, int E) {  // five slices
+  return slice_bytes(fix_mag<5>(x, E) << 21, __float_as_int(x) < 0);
 }
 
 // One n-tile (basis columns 8 ct .. 8 ct + 7) of one piece of the chunk (columns kbeg ..
 // kend - 1, one segment sg): the diagonals d = i + j < ND of the slice products over the
-// k-steps (A and B fragments by ldmatrix), then the assembled complex 8 x 8 block into the
-// outputs (stored when first, else added).
-template <int D, int NS, int ND, class OR>
-__device__ __forceinline__ void tc_tile(const uint16_t* Bsl, const uint16_t* Asl, const int* rowE,
-                                        int ct, int kbeg, int kend, int nt, int t0, int sg,
-                                        bool first, OR orow) {
+// k-steps, then the assembled complex 8 x 8 block into the outputs (stored when first, else
+// added).  A lane's share of the operands is four columns of one target (Re and Im) and of one
+// basis function; it turns their slice bytes into f16 pairs as it needs them.
+template <int FMAX>
+struct RowType {
+  using type = double;
+};
+template <>
+struct RowType<0xff> {
+  using type = float;
+};
+// rowE[2 g], [2 g + 1]: exponent fields of the rows' scales; FMAX the field of infinities and NaN.
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+template <int D, int NS, int ND, int FMAX, class OR>
+__device__ __forceinline__ void tc_tile(const uint2* Bs, const uint4* G, const int* rowE, int ct,
+                                        int kbeg, int kend, int nt, int t0, int sg, bool first,
+                                        OR orow) {
   using C = TcCfg<D>;
   constexpr int n = C::n;
-  constexpr int NB = (NS + 1) / 2;  // slice pairs of B loaded per k-step
   const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const int nb = ct * 8 + g;
   float acc[ND][4];
 #pragma unroll
   for (int d = 0; d < ND; ++d) acc[d][0] = acc[d][1] = acc[d][2] = acc[d][3] = 0.0f;
-  const int arow = (lane & 7) + ((lane >> 3) & 1) * 8, acol = (lane >> 4) * 8;
-  const int brow = ct * 8 + (lane & 7), bcol = ((lane >> 3) & 1) * 8, bsl = lane >> 4;
+  const uint4* gp = G + g * C::GST + 2 * c;
+  const uint2* bp = Bs + (nb < n ? nb : 0) * C::BST + 2 * c;
+#pragma unroll 1
   for (int k0 = kbeg; k0 < kend; k0 += 16) {
-    uint32_t bf[2 * NB][2];
+    uint4 b0 = *reinterpret_cast<const uint4*>(bp + k0);
+    uint4 b1 = *reinterpret_cast<const uint4*>(bp + k0 + 8);
+    if (nb >= n) b0 = b1 = make_uint4(kZeroSlices, kZeroSlices, kZeroSlices, kZeroSlices);
+    const uint4 z = make_uint4(kZeroSlices, kZeroSlices, kZeroSlices, kZeroSlices);
+    const uint4 v0 = g < nt ? gp[k0] : z, v1 = g < nt ? gp[k0 + 1] : z;
+    const uint4 v2 = g < nt ? gp[k0 + 8] : z, v3 = g < nt ? gp[k0 + 9] : z;
+    uint32_t bf[NS][2];
+    auto bslice = [&](auto I) {
+      constexpr int i = decltype(I)::value;
+      if constexpr (i < NS) {
+        bf[i][0] = half2_slice<i>(make_uint2(b0.x, b0.y), make_uint2(b0.z, b0.w));
+        bf[i][1] = half2_slice<i>(make_uint2(b1.x, b1.y), make_uint2(b1.z, b1.w));
+      }
+    };
+    bslice(IntC<0>{}); bslice(IntC<1>{}); bslice(IntC<2>{}); bslice(IntC<3>{});
+    bslice(IntC<4>{}); bslice(IntC<5>{}); bslice(IntC<6>{}); bslice(IntC<7>{});
+    auto aslice = [&](auto I) {
+      constexpr int i = decltype(I)::value;
+      if constexpr (i < NS) {
+        const uint32_t af[4] = {half2_slice<i>(make_uint2(v0.x, v0.y), make_uint2(v1.x, v1.y)),
+                                half2_slice<i>(make_uint2(v0.z, v0.w), make_uint2(v1.z, v1.w)),
+                                half2_slice<i>(make_uint2(v2.x, v2.y), make_uint2(v3.x, v3.y)),
+                                half2_slice<i>(make_uint2(v2.z, v2.w), make_uint2(v3.z, v3.w))};
 #pragma unroll
-    for (int p = 0; p < NB; ++p) {
-      uint32_t r[4];
-      ldsm_x4(r, Bsl + (size_t)(2 * p + bsl) * C::NP * C::CH + C::swz(brow, k0 + bcol));
-      bf[2 * p][0] = r[0];
-      bf[2 * p][1] = r[1];
-      bf[2 * p + 1][0] = r[2];
-      bf[2 * p + 1][1] = r[3];
-    }
-#pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      uint32_t af[4];
-      ldsm_x4(af, Asl + (size_t)i * 16 * C::CH + C::swz(arow, k0 + acol));
-#pragma unroll
-      for (int j = 0; j < NS && i + j < ND; ++j) mma_f16_16816(acc[i + j], af, bf[j]);
-    }
+        for (int j = 0; j < NS; ++j)
+          if (i + j < ND) mma_f16_16816(acc[i + j < ND ? i + j : 0], af, bf[j]);
+      }
+    };
+    aslice(IntC<0>{}); aslice(IntC<1>{}); aslice(IntC<2>{}); aslice(IntC<3>{});
+    aslice(IntC<4>{}); aslice(IntC<5>{}); aslice(IntC<6>{}); aslice(IntC<7>{});
   }
   if (g < nt) {
+    using V = typename RowType<FMAX>::type;
+    const bool bad = rowE[2 * g] == FMAX || rowE[2 * g + 1] == FMAX;
+    const int Er = bad ? kPoisonExp : exp_bound(rowE[2 * g], V());
+    const int Ei = bad ? kPoisonExp : exp_bound(rowE[2 * g + 1], V());
 #pragma unroll
     for (int cc = 0; cc < 2; ++cc) {
       const int nm = ct * 8 + 2 * c + cc;
       if (nm >= n) continue;
       const int e2 = c_kwexp[nm];
-      const double re = assemble<ND>(acc, cc, rowE[g] + e2);
-      const double im = assemble<ND>(acc, 2 + cc, rowE[g + 8] + e2);
+      const double re = assemble<ND>(acc, cc, Er + e2);
+      const double im = assemble<ND>(acc, 2 + cc, Ei + e2);
       cplx* dst = reinterpret_cast<cplx*>(orow(t0 + g)) + (int64_t)sg * n + nm;
       if (first) {
         dst->re = re;
@@ -424,311 +386,350 @@ __device__ __forceinline__ void tc_tile(const uint16_t* Bsl, const uint16_t* Asl
 // I[i][seg][nm] = sum_{q in seg} w_q K(x_i, X_q) J_q K_nm(u_q, v_q) and, when eout is not
 // null, eout[i * nseg + seg] = sum_q of the kernel's rounding envelope (FP32 sums), with the
 // contraction over the nodes on the tensor cores by the exact slice split (lcq_tc.cuh):
-// 8 slices per FP64 operand and the diagonals i + j <= 8 for FP64 kernel values; for the mixed
-// form's FP32 kernel values 5 slices and the diagonals i + j <= 4.
-// A chunk is a run of pieces (segment sg, its nodes l0 .. l0 + nq - 1), each padded with
-// zero columns to a multiple of 16 (the MMA depth), packed while they fit in TcCfg::CH
-// columns: the four children of a small rule share one chunk.  Each piece's contribution is
-// assembled in FP64 and written (the segment's first part) or added.
-// Per chunk: (1) geometry, thread per real node (padding columns are zeroed apart, so no
-// lane of the FP64 work idles): X, N w, J w (FP64), and each basis value split into 8 f16
-// slices on its column's fixed bound as it is formed (integer work that runs in the shadow
-// of the FP64 geometry); (2) per tile of 8 targets: kernel values and envelopes, thread per
-// (target, real node); (3) one warp per target splits the Re and Im rows of its kernel
-// values on their own power-of-two scales; (4) one warp per n-tile of 8 basis columns
-// accumulates the diagonals over each piece's 16-node steps with mma.sync, both operands read
-// by ldmatrix, and assembles and stores its 8 x 8 complex block.
-// For real k and kinds S, D and CFIE with a real alpha the kernel constants are folded into
-// the node data (kernel_eval_fold).  smb: TcCfg<D>::BYTES of shared memory (16-byte aligned).
-// form: 0 FP64 kernel values; 1 FP32 ones (the mixed form for eps >= kMixedMinEps); 2
-// two-float ones (kernel_eval_ff; the mixed form below that) where the constants fold, else
-// FP64.
+// 8 slices per operand and the diagonals i + j <= 8; for the mixed form's FP32 kernel values 5
+// slices and the diagonals i + j <= 4.
+// A chunk is a run of pieces (segment sg, its nodes l0 .. l0 + nq - 1), each padded to a multiple
+// of 16 (the MMA depth), that fill up to CH columns, a thread (degrees 8-10: two) per column: the
+// four children of a small rule share one chunk, a large rule is cut where the chunk ends.
+// Per chunk: (1) row factors, a thread per (row, m); (2) point, normal and basis values of the
+// thread's node in fixed point (lcq_fxgeom.cuh); the point stays in registers, the basis goes to
+// shared memory as slices.  Per tile of 8 targets: (3) the thread's kernel values (fx_core:
+// fixed point; or two-float, or FP32), with the largest exponent of each target's Re and Im over a
+// piece (integer maxima); (4) their slices on that scale; (5) a warp per piece and 8 basis columns:
+// mma.sync on fragments built from the slice bytes.  Storing an operand as 8 bytes (not as 8
+// f16) lets a chunk hold 256 columns where it held 128, so that every thread has a node and the
+// barriers come half as often; they, not the pipes, bounded the kernel (1280-patch CFIE, eps
+// 1e-9: issue slots 32% busy before).
+// S: exponent of the fixed-point positions (block_scale).  form: 0 FP64 (fixed point); 1 FP32
+// kernel values (the mixed form for eps >= kMixedMinEps); 2 two-float ones (kernel_eval_ff; the
+// mixed form below that) where the constants fold, else FP64.
+template <int D, int FORM, class TA, class OR>
+__device__ __forceinline__ void block_moments_form(
+    const FxChart<D>& ch, int S, const double* __restrict__ ru, const double* __restrict__ rv,
+    const double* __restrict__ rw, int Q, const SegMap* segs, int nseg, const TA& ta, int T, OR orow,
+    const KernelParams& kp, unsigned char* smb, const double* cen, double R, double* eout) {
+  using C = TcCfg<D>;
+  constexpr int n = C::n;
+  constexpr bool mixed = FORM == 1, ffe = FORM == 2, fixed = FORM == 0;
+  uint4* G = reinterpret_cast<uint4*>(smb + C::OFF_G);
+  u64* rows = reinterpret_cast<u64*>(smb + C::OFF_G);
+  uint2* Bs = reinterpret_cast<uint2*>(smb + C::OFF_B);
+  double* tx = reinterpret_cast<double*>(smb + C::OFF_TX);
+  i64* txi = reinterpret_cast<i64*>(tx);  // fixed-point targets, in the FP64 slots
+  u64* tn = reinterpret_cast<u64*>(tx + 3 * C::TT);
+  float* Ep = reinterpret_cast<float*>(smb + C::OFF_EP);
+  int* rowE = reinterpret_cast<int*>(smb + C::OFF_RE);
+  int* pcs = reinterpret_cast<int*>(smb + C::OFF_PC);  // [piece][sg, l0, nq, po, row0, rb, first]
+  int* te = reinterpret_cast<int*>(smb + C::OFF_TE);
+  const KernelParamsF kf = to_f32(kp);
+  const float fR = f32_bits(R);
+  const FxKernel& fx = kp.fx;  // read at its uses: as a register copy it spills
+  const FxTables tab = fx_tables();
+  constexpr double kInv4Pi = 0.07957747154594767;
+  const float escale = mixed ? (float)(kF32Floor / kRoundingFloor)
+                             : ffe ? (float)(kTwoFloatFloor / kRoundingFloor) : 1.0f;
+  const int warp = threadIdx.x >> 5;
+  const int col = threadIdx.x % C::CH, part = threadIdx.x / C::CH;
+  // conical rules: rows of mr nodes sharing v, which every segment map here (T0 and its
+  // midpoint descendants) keeps a function of the rule's v alone
+  const int mr = (int)lrintf(sqrtf((float)Q));
+  using RW = FxRow<D>;
+  constexpr int kRowMax = C::G_BYTES / 8 / RW::size;
+  int sg_next = 0, l_next = 0;
+  while (sg_next < nseg) {
+    // plan the chunk (uniform across the block); thread 0 records it for indexed lookups.  A
+    // piece is cut at the end of the chunk when at least 64 columns are left, or at the end of
+    // the row area.  The FP32 tier cuts a rule into equal parts of at most CHG nodes instead and
+    // lets the parts that fit CHG columns share a row scale (a group): with five slices the
+    // scale shows in the moments' last digits, and its refinement decisions follow those.
+    int np = 0, ncp = 0, nrow = 0, gcp = 0, g0 = 0;
+    __syncthreads();
+    while (sg_next < nseg && np < C::MAXP && ncp < C::CH) {
+      int nq = Q - l_next;
+      const int room = C::CH - ncp;
+      if (mixed) {
+        const int nparts = (Q + C::CHG - 1) / C::CHG;
+        nq = min(nq, (Q + nparts - 1) / nparts);
+        const int pad = (nq + 15) & ~15;
+        if (gcp > 0 && gcp + pad > C::CHG) {
+          gcp = 0;
+          if (room < C::CHG) break;
+          g0 = np;
+        }
+        gcp += pad;
+      } else if (((nq + 15) & ~15) > room) {
+        if (np > 0 && room < 64) break;
+        nq = room;
+      }
+      const int r0 = l_next / mr;
+      int prow = (l_next + nq - 1) / mr - r0 + 1;
+      if (nrow + prow > kRowMax) {
+        if (np > 0) break;
+        nq = ((r0 + kRowMax) * mr - l_next) & ~15;  // rows of a first piece beyond the area
+        prow = (l_next + nq - 1) / mr - r0 + 1;
+      }
+      if (threadIdx.x == 0) {
+        int* pc = pcs + 8 * np;
+        pc[0] = sg_next;
+        pc[1] = l_next;
+        pc[2] = nq;
+        pc[3] = ncp;
+        pc[4] = r0;
+        pc[5] = nrow;
+        pc[6] = l_next == 0;
+        pc[7] = mixed ? g0 : np;  // piece whose row scales it uses
+      }
+      nrow += prow;
+      ncp += (nq + 15) & ~15;
+      ++np;
+      l_next += nq;
+      if (l_next >= Q) {
+        l_next = 0;
+        ++sg_next;
+      }
+    }
+    __syncthreads();
+    // (1) m-major, so that the lanes of a warp share m and with it the loop length
+    for (int e = threadIdx.x; e < nrow * (D + 1); e += blockDim.x) {
+      const int m = e / nrow, rr = e - m * nrow;
+      int k = 0;
+      for (int kk = 1; kk < np; ++kk)
+        if (pcs[8 * kk + 5] <= rr) k = kk;
+      const int* pc = pcs + 8 * k;
+      const SegMap& Sg = segs[pc[0]];
+      const int l = (pc[4] + rr - pc[5]) * mr;
+      fx_row_factors<D>(Sg.ay + ru[l] * Sg.e1y + rv[l] * Sg.e2y, m, ch, rows + rr * RW::size);
+    }
+    __syncthreads();
+    // (2) this thread's node
+    int pk = 0;  // its piece
+    for (int kk = 1; kk < np; ++kk)
+      if (pcs[8 * kk + 3] <= col) pk = kk;
+    const int ql = col - pcs[8 * pk + 3];
+    const bool in = col < ncp, real = in && ql < pcs[8 * pk + 2];
+    const int pe = pcs[8 * pk + 7];  // the piece that holds its row scales
+    i64 Xi[3] = {0, 0, 0};   // fixed: point and node for fx_eval_int
+    FxS nn[3] = {{0, 0}, {0, 0}, {0, 0}};
+    u64 wm = 0;
+    int ew = 0;
+    double Xd[3] = {0, 0, 0};  // two-float and FP32: point, weighted normal and area
+    ff Nff[3] = {{0, 0}, {0, 0}, {0, 0}}, Jff = {0, 0}, Kff = {0, 0};
+    float Nf[3] = {0, 0, 0}, Jf = 0.0f;
+    if (real) {
+      const int* pc = pcs + 8 * pk;
+      const SegMap& Sg = segs[pc[0]];
+      const int l = pc[1] + ql;
+      const double r0 = ru[l], r1 = rv[l];
+      const double u = Sg.ax + r0 * Sg.e1x + r1 * Sg.e2x;
+      const double v = Sg.ay + r0 * Sg.e1y + r1 * Sg.e2y;
+      const FxS s = fx_split(fx_fix(2.0 * u + v - 1.0, 0));
+      const u64* row = rows + (pc[5] + l / mr - pc[4]) * RW::size;
+      fx_basis_point<D>(s, row, part, C::PARTS, [&](int idx, i64 kv) {
+        const u64 sgn = (u64)(kv >> 63);
+        const u64 M = ((((u64)kv ^ sgn) - sgn) + 4) >> 3;  // 56 bits, rounded
+        Bs[idx * C::BST + col] = slice_bytes(M < (1ull << 56) ? M : (1ull << 56) - 1, kv < 0);
+      });
+      i64 X[3], N[3];
+      fx_chart_point<D>(s, row, X, N);
+      const double w = rw[l] * Sg.det;
+      if (fixed) {
+        const int k = S - ch.sx;  // >= 1
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Xi[c] = fx_sra(X[c] << 3, k);
+        fx_node_from_normal(N, ch.su + ch.sv + 1, w, nn, &wm, &ew);
+        if (ch.bad) ew = kFxBad + 1;
+        const int e = min(max(ew, -120), 120);
+        Jf = (float)(uint32_t)(wm >> 32) * 9.31322575e-10f * __int_as_float((127 + e) << 23);
+      } else {
+        double Nn[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          Xd[c] = ch.bad ? __longlong_as_double(0x7ff8000000000000ll)
+                         : fx_pack<false>(X[c], ch.sx - 59);
+          Nn[c] = fx_pack<false>(N[c], ch.su + ch.sv - 61);
+        }
+        const double N2 = fma(Nn[0], Nn[0], fma(Nn[1], Nn[1], Nn[2] * Nn[2]));
+        const double Jw = N2 > 0.0 ? N2 * rsqrt_nr(N2) * w : 0.0;
+        if (ffe) {
+          const double wn = w * (kp.kind == 1 ? 1.0 : kp.ar) * kInv4Pi;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) Nff[c] = ff_of(Nn[c] * wn);
+          Jff = ff_of(Jw * ((kp.kind == 0 ? 1.0 : kp.br) * kInv4Pi));
+          Kff = ff_of(Jw * (kp.bi * kInv4Pi));
+          Jf = f32_bits(Jw * kInv4Pi);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) Nf[c] = (float)(Nn[c] * w);
+          Jf = (float)Jw;
+        }
+      }
+    } else if (in) {
+#pragma unroll 1
+      for (int idx = part; idx < n; idx += C::PARTS)
+        Bs[idx * C::BST + col] = make_uint2(kZeroSlices, kZeroSlices);
+    }
+    for (int t0 = 0; t0 < T; t0 += C::TT) {
+      const int nt = min(C::TT, T - t0);
+      for (int e = threadIdx.x; e < C::MAXP * C::TT * 2; e += blockDim.x) rowE[e] = 0;
+      if (threadIdx.x < nt) {
+        double xp[3];
+        ta.pos(t0 + threadIdx.x, xp);
+        bool fin = true;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          xp[c] -= cen[c];
+          fin = fin && isfinite(xp[c]);
+          if (fixed) txi[3 * threadIdx.x + c] = fx_fix(xp[c], S);
+          else tx[3 * threadIdx.x + c] = xp[c];
+        }
+        te[threadIdx.x] = fin ? -100000 : kFxBad + 1;
+        if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
+      }
+      __syncthreads();
+      // (3) the column's kernel values; zeros in padding columns
+      if (in) {  // whole half-warps: pieces are multiples of 16 columns
+        const unsigned half = 0xffffu << (threadIdx.x & 16);
+#pragma unroll 1
+        for (int i = part; i < nt; i += C::PARTS) {
+          float ev = 0.0f;
+          uint32_t ex = 0;  // exponent fields of Re (high half) and Im
+          if (mixed) {
+            float2 g = make_float2(0.0f, 0.0f);
+            const double d0 = tx[3 * i] - Xd[0], d1 = tx[3 * i + 1] - Xd[1],
+                         d2 = tx[3 * i + 2] - Xd[2];
+            const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
+            if (real && r2 > 0.0)
+              g = kernel_eval_f32f(kp, kf, d0, d1, d2, r2, Nf[0], Nf[1], Nf[2], Jf, fR, &ev);
+            ex = ((uint32_t)exp_field(g.x) << 16) | (uint32_t)exp_field(g.y);
+            *reinterpret_cast<float4*>(G + i * C::GST + col) = make_float4(g.x, g.y, ev, 0.0f);
+          } else {
+            cplx g = {0.0, 0.0};
+            if (real) {
+              if (ffe) {
+                g = kernel_eval_ff(kp.kind, kp.kr, ff_of(kp.kr), kf, g_sct, g_sctf, tx[3 * i],
+                                   tx[3 * i + 1], tx[3 * i + 2], Xd[0], Xd[1], Xd[2], Nff, Jff, Kff,
+                                   Jf, fR, &ev);
+              } else {
+                FxS nt3[3] = {nn[0], nn[1], nn[2]};
+                if (kp.kind == 3) {
+                  nt3[0] = fx_unjoin(tn[3 * i]);
+                  nt3[1] = fx_unjoin(tn[3 * i + 1]);
+                  nt3[2] = fx_unjoin(tn[3 * i + 2]);
+                }
+                const i64 d0 = txi[3 * i] - Xi[0], d1 = txi[3 * i + 1] - Xi[1],
+                          d2 = txi[3 * i + 2] - Xi[2];
+                const int e2 = max(ew, te[i]);
+                if (!fx_eval_int<false>(fx, tab, d0, d1, d2, S, nt3, wm, e2, &g.re, &g.im, &ev,
+                                        kf.kr, kf.ki, kf.eb, kf.ea * fR, Jf))
+                  g = fx_fallback(kp, fx_pack<false>(d0, S - 62), fx_pack<false>(d1, S - 62),
+                                  fx_pack<false>(d2, S - 62), nt3[0], nt3[1], nt3[2], wm, e2,
+                                  (double)fR, &ev);
+              }
+            }
+            ex = ((uint32_t)exp_field(g.re) << 16) | (uint32_t)exp_field(g.im);
+            *reinterpret_cast<cplx*>(G + i * C::GST + col) = g;
+          }
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) {
+            ex = __vmaxu2(ex, __shfl_xor_sync(half, ex, o));
+            ev += __shfl_xor_sync(half, ev, o);
+          }
+          if ((threadIdx.x & 15) == 0) {
+            atomicMax(rowE + (pe * C::TT + i) * 2, (int)(ex >> 16));
+            atomicMax(rowE + (pe * C::TT + i) * 2 + 1, (int)(ex & 0xffffu));
+            Ep[i * C::MAXP + (col >> 4)] = ev;
+          }
+        }
+      }
+      __syncthreads();
+      // envelope sums: a thread per (target, piece) over the half-warps' sums; the FP32 tier, whose
+      // floor is 2e-6 of them, a warp per target over the columns
+      if (eout && mixed) {
+        const int lane = threadIdx.x & 31;
+        if (warp < nt)
+          for (int k = 0; k < np; ++k) {
+            const int* pc = pcs + 8 * k;
+            float es = 0.0f;
+            for (int q = lane; q < pc[2]; q += 32)
+              es += reinterpret_cast<const float4*>(G + warp * C::GST + pc[3] + q)->z;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
+            if (lane == 0) {
+              double* ed = eout + (int64_t)(t0 + warp) * nseg + pc[0];
+              const double v = (double)(es * escale);
+              *ed = pc[6] ? v : *ed + v;
+            }
+          }
+        __syncthreads();  // the slices overwrite the columns
+      } else if (eout) {
+        // one thread per target, its pieces in order (two may belong to one segment)
+        if (threadIdx.x < nt)
+          for (int k = 0; k < np; ++k) {
+            const int* pc = pcs + 8 * k;
+            float es = 0.0f;
+            for (int h = pc[3] >> 4; h < (pc[3] + pc[2] + 15) >> 4; ++h)
+              es += Ep[threadIdx.x * C::MAXP + h];
+            double* ed = eout + (int64_t)(t0 + threadIdx.x) * nseg + pc[0];
+            const double v = (double)(es * escale);
+            *ed = pc[6] ? v : *ed + v;
+          }
+      }
+      // (4) slices of the column's values on their rows' scales
+      if (in) {
+#pragma unroll 1
+        for (int i = part; i < nt; i += C::PARTS) {
+          const int* E = rowE + (pe * C::TT + i) * 2;
+          uint4* gp = G + i * C::GST + col;
+          uint2 a, b;
+          if (mixed) {
+            const float2 g = *reinterpret_cast<const float2*>(gp);  // the envelope beside it is done
+            a = row_slices(g.x, exp_bound(E[0], 0.0f));
+            b = row_slices(g.y, exp_bound(E[1], 0.0f));
+          } else {
+            const cplx g = *reinterpret_cast<const cplx*>(gp);
+            a = row_slices(g.re, exp_bound(E[0], 0.0));
+            b = row_slices(g.im, exp_bound(E[1], 0.0));
+          }
+          *gp = make_uint4(a.x, a.y, b.x, b.y);
+        }
+      }
+      __syncthreads();
+      // (5) tensor-core contraction, a warp per n-tile and piece; pieces of one segment add to the
+      // same outputs, so the first one's warp takes them all, in order
+      for (int e = warp; e < np * C::NTILE; e += kThreads / 32) {
+        const int ct = e % C::NTILE;
+        int k = e / C::NTILE;
+        if (k > 0 && pcs[8 * (k - 1)] == pcs[8 * k]) continue;
+        do {
+          const int* pc = pcs + 8 * k;
+          const int kb = pc[3], ke = pc[3] + ((pc[2] + 15) & ~15);
+          const int* E = rowE + pc[7] * C::TT * 2;
+          if (mixed)
+            tc_tile<D, 5, 5, 0x00ff>(Bs, G, E, ct, kb, ke, nt, t0, pc[0], pc[6] != 0, orow);
+          else
+            tc_tile<D, 8, 9, 0x7ff>(Bs, G, E, ct, kb, ke, nt, t0, pc[0], pc[6] != 0, orow);
+          ++k;
+        } while (k < np && pcs[8 * k] == pcs[8 * (k - 1)]);
+      }
+      __syncthreads();
+    }
+  }
+}
+
 template <int D, class TA, class OR>
-__device__ void block_moments_tc(const double* cf, const double* cfd, const double* __restrict__ ru,
+__device__ void block_moments_tc(const FxChart<D>& ch, int S, const double* __restrict__ ru,
                                  const double* __restrict__ rv, const double* __restrict__ rw,
                                  int Q, const SegMap* segs, int nseg, const TA& ta, int T, OR orow,
                                  const KernelParams& kp, unsigned char* smb, const double* cen,
                                  double R, double* eout, int form) {
-  using C = TcCfg<D>;
-  constexpr int n = C::n;
-  double* Xs = reinterpret_cast<double*>(smb + C::OFF_X);
-  double* Ns = reinterpret_cast<double*>(smb + C::OFF_N);
-  double* Js = reinterpret_cast<double*>(smb + C::OFF_J);
-  double* Ks = reinterpret_cast<double*>(smb + C::OFF_K);
-  uint16_t* Bsl = reinterpret_cast<uint16_t*>(smb + C::OFF_BS);
-  cplx* Gs = reinterpret_cast<cplx*>(smb + C::OFF_G);
-  float2* Gf = reinterpret_cast<float2*>(smb + C::OFF_G);
-  uint16_t* Asl = reinterpret_cast<uint16_t*>(smb + C::OFF_G);
-  double* rows = reinterpret_cast<double*>(smb + C::OFF_G);
-  float* Ef = reinterpret_cast<float*>(smb + C::OFF_EF);
-  float* Jf = reinterpret_cast<float*>(smb + C::OFF_JF);
-  float* Nf = reinterpret_cast<float*>(smb + C::OFF_NF);
-  int* rowE = reinterpret_cast<int*>(smb + C::OFF_ROWE);
-  double* tx = reinterpret_cast<double*>(smb + C::OFF_TX);
-  u64* tn = reinterpret_cast<u64*>(tx + 3 * C::TT);
-  int* colinfo = reinterpret_cast<int*>(smb + C::OFF_CI);  // (piece << 16) | node, 0xffff: pad
-  int* pcs = reinterpret_cast<int*>(smb + C::OFF_PC);      // [piece][sg, l0, nq, po, row0, rb, first]
-  const KernelParamsF kf = to_f32(kp);
-  const float fR = f32_bits(R);
-  const bool mixed = form == 1;
   // two-float kernel values: real k, kinds S, D and CFIE with a real alpha, whose constants are
   // folded into the node data
-  const bool ffe = form == 2 && kp.ki == 0.0 && kp.kind <= 2 && kp.ai == 0.0;
-  const FxKernel& fx = kp.fx;  // read at its uses: as a register copy it spills (224 B)
-  const FxTables tab = fx_tables();
-  u64* Nfx = reinterpret_cast<u64*>(Ns);  // nodes as fx_eval takes them, in the FP64 slots
-  u64* Wfx = reinterpret_cast<u64*>(Js);
-  u64* Efx = reinterpret_cast<u64*>(Ks);
-  const float escale = mixed ? (float)(kF32Floor / kRoundingFloor)
-                             : ffe ? (float)(kTwoFloatFloor / kRoundingFloor) : 1.0f;
-  const ff krf = ff_of(kp.kr);
-  ff* Nff = reinterpret_cast<ff*>(Ns);  // two-float node data in the FP64 slots
-  ff* Jff = reinterpret_cast<ff*>(Js);
-  ff* Kff = reinterpret_cast<ff*>(Ks);
-  constexpr double kInv4Pi = 0.07957747154594767;
-  const double fa_n = (kp.kind == 1 ? 1.0 : kp.ar) * kInv4Pi;
-  const double fj_r = (kp.kind == 0 ? 1.0 : kp.br) * kInv4Pi, fj_i = kp.bi * kInv4Pi;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  // conical rules: rows of mr nodes sharing v (see block_moments)
-  const int mr = (int)lrint(sqrt((double)Q));
-  bool by_rows = mr * mr == Q;
-  for (int sg = 0; sg < nseg; ++sg) by_rows = by_rows && segs[sg].e1y == 0.0;
-  using RW = KwRow<D>;
-  constexpr int kRowMax = C::G_BYTES / 8 / RW::size;
-  const int nparts = (Q + C::CH - 1) / C::CH;
-  const int psize = (Q + nparts - 1) / nparts;
-  // the padding columns n .. NP-1 of the basis slices stay zero
-  __syncthreads();
-  for (int e = threadIdx.x; e < C::NSMAX * (C::NP - n) * C::CH; e += blockDim.x) {
-    const int i = e / ((C::NP - n) * C::CH), r = e - i * (C::NP - n) * C::CH;
-    const int col = n + r / C::CH, k = r - (col - n) * C::CH;
-    Bsl[(size_t)i * C::NP * C::CH + C::swz(col, k)] = 0;
-  }
-  int sg_next = 0, part_next = 0;
-  while (sg_next < nseg) {
-    // plan the chunk (uniform across the block); thread 0 records it for indexed lookups
-    int np = 0, ncp = 0, nrow = 0, ncr = 0;
-    __syncthreads();
-    while (sg_next < nseg && np < C::MAXP) {
-      const int l0 = part_next * psize, nq = min(psize, Q - l0), pad = (nq + 15) & ~15;
-      if (np > 0 && ncp + pad > C::CH) break;
-      if (threadIdx.x == 0) {
-        int* pc = pcs + 8 * np;
-        pc[0] = sg_next;
-        pc[1] = l0;
-        pc[2] = nq;
-        pc[3] = ncp;
-        pc[4] = by_rows ? l0 / mr : 0;
-        pc[5] = nrow;
-        pc[6] = part_next == 0;
-        pc[7] = ncr;
-      }
-      nrow += by_rows ? (l0 + nq - 1) / mr - l0 / mr + 1 : 0;
-      ncp += pad;
-      ncr += nq;
-      ++np;
-      if (++part_next == nparts) {
-        part_next = 0;
-        ++sg_next;
-      }
-    }
-    const bool use_rows = by_rows && nrow <= kRowMax;
-    __syncthreads();
-    for (int p = threadIdx.x; p < ncp; p += blockDim.x) {
-      int k = 0;
-      for (int kk = 1; kk < np; ++kk)
-        if (pcs[8 * kk + 3] <= p) k = kk;
-      const int ql = p - pcs[8 * k + 3];
-      colinfo[p] = (k << 16) | (ql < pcs[8 * k + 2] ? ql : 0xffff);
-    }
-    if (use_rows) {
-      // m-major, so that the lanes of a warp share m and with it the loop length
-      for (int e = threadIdx.x; e < nrow * (D + 1); e += blockDim.x) {
-        const int m = e / nrow, rr = e - m * nrow;
-        int k = 0;
-        for (int kk = 1; kk < np; ++kk)
-          if (pcs[8 * kk + 5] <= rr) k = kk;
-        const int* pc = pcs + 8 * k;
-        const SegMap& S = segs[pc[0]];
-        const int l = (pc[4] + rr - pc[5]) * mr;
-        kw_row_factors<D>(S.ay + ru[l] * S.e1y + rv[l] * S.e2y, m, cf, cfd, rows + rr * RW::size);
-      }
-    }
-    __syncthreads();
-    // column of the r-th real node of the chunk (the pieces' real columns are contiguous):
-    // the FP64 loops run over real nodes only, so that no lane of theirs idles on padding
-    auto real_col = [&](int r) {
-      int k = 0;
-      for (int kk = 1; kk < np; ++kk)
-        if (pcs[8 * kk + 7] <= r) k = kk;
-      return pcs[8 * k + 3] + (r - pcs[8 * k + 7]);
-    };
-    // padding columns: zero basis slices
-    for (int p = threadIdx.x; p < ncp; p += blockDim.x)
-      if ((colinfo[p] & 0xffff) == 0xffff) {
-#pragma unroll 1
-        for (int idx = 0; idx < n; ++idx)
-#pragma unroll
-          for (int i = 0; i < 8; ++i) Bsl[(size_t)i * C::NP * C::CH + C::swz(idx, p)] = 0;
-      }
-    // (1) geometry and basis slices, thread per real node
-    for (int rn = threadIdx.x; rn < ncr; rn += blockDim.x) {
-      const int p = real_col(rn);
-      const int ci = colinfo[p], ql = ci & 0xffff;
-      {
-        const int* pc = pcs + 8 * (ci >> 16);
-        const SegMap& S = segs[pc[0]];
-        const int l = pc[1] + ql;
-        const double r0 = ru[l], r1 = rv[l];
-        const double u = S.ax + r0 * S.e1x + r1 * S.e2x;
-        const double w = rw[l] * S.det;
-        double X[3], Xu[3], Xv[3], Nn[3];
-        if (use_rows) {
-          kw_geometry_row_emit<D>(u, rows + (pc[5] + l / mr - pc[4]) * RW::size, X, Xu, Xv,
-                                  [&](int idx, double kv) { store_basis_slices<D>(Bsl, idx, p, kv); });
-        } else {
-          double K[n];
-          const double v = S.ay + r0 * S.e1y + r1 * S.e2y;
-          kw_geometry_proj<D>(u, v, cf, cfd, X, Xu, Xv, K);
-#pragma unroll 1
-          for (int idx = 0; idx < n; ++idx) store_basis_slices<D>(Bsl, idx, p, K[idx]);
-        }
-        cross3(Xu, Xv, Nn);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) Xs[c * C::CH + p] = X[c];
-        if (mixed || ffe) {
-          const double N2 = fma(Nn[0], Nn[0], fma(Nn[1], Nn[1], Nn[2] * Nn[2]));
-          const double Jw = N2 > 0.0 ? N2 * rsqrt_nr(N2) * w : 0.0;
-          if (ffe) {
-            const double wn = w * fa_n;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) Nff[c * C::CH + p] = ff_of(Nn[c] * wn);
-            Jff[p] = ff_of(Jw * fj_r);
-            Kff[p] = ff_of(Jw * fj_i);
-            Jf[p] = f32_bits(Jw * kInv4Pi);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) Nf[c * C::CH + p] = (float)(Nn[c] * w);
-            Jf[p] = (float)Jw;
-          }
-        } else {
-          FxS nn[3];
-          u64 wm;
-          int ew;
-          fx_make_node(Nn, w, nn, &wm, &ew);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) Nfx[c * C::CH + p] = fx_join(nn[c]);
-          Wfx[p] = wm;
-          Efx[p] = (u64)(i64)ew;
-        }
-      }
-    }
-    __syncthreads();
-    for (int t0 = 0; t0 < T; t0 += C::TT) {
-      const int nt = min(C::TT, T - t0);
-      if (threadIdx.x < nt) {
-        double* xp = tx + 3 * threadIdx.x;
-        ta.pos(t0 + threadIdx.x, xp);
-        xp[0] -= cen[0];
-        xp[1] -= cen[1];
-        xp[2] -= cen[2];
-        if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
-      }
-      __syncthreads();
-      // (2) kernel values and envelopes of the real columns; zeros in the padding ones
-      for (int e = threadIdx.x; e < nt * ncp; e += blockDim.x) {
-        const int i = e / ncp, p = e - i * ncp;
-        if ((colinfo[p] & 0xffff) == 0xffff) {
-          if (mixed) Gf[i * C::CH + p] = make_float2(0.0f, 0.0f);
-          else Gs[i * C::CH + p] = cplx{0.0, 0.0};
-          Ef[i * C::CH + p] = 0.0f;
-        }
-      }
-      for (int e = threadIdx.x; e < nt * ncr; e += blockDim.x) {
-        const int i = e / ncr, p = real_col(e - i * ncr);
-        float ev = 0.0f;
-        if (mixed) {
-          float2 g = make_float2(0.0f, 0.0f);
-          const double d0 = tx[3 * i] - Xs[p], d1 = tx[3 * i + 1] - Xs[C::CH + p],
-                       d2 = tx[3 * i + 2] - Xs[2 * C::CH + p];
-          const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
-          if (r2 > 0.0)
-            g = kernel_eval_f32f(kp, kf, d0, d1, d2, r2, Nf[p], Nf[C::CH + p], Nf[2 * C::CH + p],
-                                 Jf[p], fR, &ev);
-          Gf[i * C::CH + p] = g;
-        } else {
-          cplx g;
-          if (ffe) {
-            const ff Np[3] = {Nff[p], Nff[C::CH + p], Nff[2 * C::CH + p]};
-            g = kernel_eval_ff(kp.kind, kp.kr, krf, kf, g_sct, g_sctf, tx[3 * i], tx[3 * i + 1],
-                               tx[3 * i + 2], Xs[p], Xs[C::CH + p], Xs[2 * C::CH + p], Np,
-                               Jff[p], Kff[p], Jf[p], fR, &ev);
-          } else {
-            const u64* nn = kp.kind == 3 ? tn + 3 * i : Nfx + p;
-            g = fx_value(kp, fx, kf, tab, tx + 3 * i, Xs + p, C::CH, nn,
-                         kp.kind == 3 ? 1 : C::CH, Wfx[p], (int)Efx[p], fR, &ev);
-          }
-          Gs[i * C::CH + p] = g;
-        }
-        Ef[i * C::CH + p] = ev;
-      }
-      __syncthreads();
-      // envelope sums, one warp per target, one sum per piece
-      if (eout && warp < nt) {
-        for (int k = 0; k < np; ++k) {
-          const int* pc = pcs + 8 * k;
-          float es = 0.0f;
-          for (int ql = lane; ql < pc[2]; ql += 32) es += Ef[warp * C::CH + pc[3] + ql];
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
-          if (lane == 0) {
-            double* ed = eout + (int64_t)(t0 + warp) * nseg + pc[0];
-            const double v = (double)(es * escale);
-            *ed = pc[6] ? v : *ed + v;
-          }
-        }
-      }
-      // (3) split the kernel rows: warp w owns target w (rows w: Re, w + 8: Im); values are
-      // read before the barrier because the slices overwrite them
-      constexpr int VPL = C::CH / 32;
-      const int q0 = lane * VPL;
-      const bool on = warp < nt;
-      if (mixed) {
-        float re[VPL], im[VPL];
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-          const float2 g = (on && q0 + v < ncp) ? Gf[warp * C::CH + q0 + v] : make_float2(0.0f, 0.0f);
-          re[v] = g.x;
-          im[v] = g.y;
-        }
-        __syncthreads();
-        if (warp < C::TT) split_row_pair<D, 5, VPL>(re, im, on, Asl, warp, q0, rowE);
-      } else {
-        double re[VPL], im[VPL];
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-          const cplx g = (on && q0 + v < ncp) ? Gs[warp * C::CH + q0 + v] : cplx{0.0, 0.0};
-          re[v] = g.re;
-          im[v] = g.im;
-        }
-        __syncthreads();
-        if (warp < C::TT) split_row_pair<D, 8, VPL>(re, im, on, Asl, warp, q0, rowE);
-      }
-      __syncthreads();
-      // (4) tensor-core contraction, one warp per n-tile, piece by piece
-      for (int ct = warp; ct < C::NTILE; ct += nwarp) {
-        for (int k = 0; k < np; ++k) {
-          const int* pc = pcs + 8 * k;
-          const int kb = pc[3], ke = pc[3] + ((pc[2] + 15) & ~15);
-          if (mixed)
-            tc_tile<D, 5, 5>(Bsl, Asl, rowE, ct, kb, ke, nt, t0, pc[0], pc[6] != 0, orow);
-          else
-            tc_tile<D, 8, 9>(Bsl, Asl, rowE, ct, kb, ke, nt, t0, pc[0], pc[6] != 0, orow);
-        }
-      }
-      __syncthreads();
-    }
-  }
+  if (form == 1)
+    block_moments_form<D, 1>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+  else if (form == 2 && kp.ki == 0.0 && kp.kind <= 2 && kp.ai == 0.0)
+    block_moments_form<D, 2>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+  else
+    block_moments_form<D, 0>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
 }
 
 // The moments of the smallest degrees in the FP64 form (n <= 10 basis functions) by the
@@ -738,7 +739,7 @@ __device__ void block_moments_tc(const double* cf, const double* cfd, const doub
 constexpr int kFp64MomentsMaxDeg = 3;
 template <int D, class TA, class OR>
 __device__ __forceinline__ void block_moments_any(
-    const double* cf, const double* cfd, const double* __restrict__ ru,
+    const double* cf, const double* cfd, const FxChart<D>& ch, int S, const double* __restrict__ ru,
     const double* __restrict__ rv, const double* __restrict__ rw, int Q, const SegMap* segs,
     int nseg, const TA& ta, int T, OR orow, const KernelParams& kp, unsigned char* smb,
     const double* cen, double R, double* eout, int form) {
@@ -754,8 +755,31 @@ __device__ __forceinline__ void block_moments_any(
       return;
     }
   }
-  block_moments_tc<D>(cf, cfd, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout,
-                      form);
+  block_moments_tc<D>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout, form);
+}
+
+// Exponent S of the fixed-point scale of positions relative to the centroid: the chart's (2^sx)
+// and the T targets' coordinates are below 2^(S - 1), so that differences are below 2^S.
+// Block-wide; slot: one int of shared memory; ends with a barrier.
+template <class TA>
+__device__ int block_scale(const TA& ta, int T, const double* cen, int sx, int* slot) {
+  __syncthreads();
+  if (threadIdx.x == 0) *slot = sx;
+  __syncthreads();
+  int m = -1000;
+  for (int i = threadIdx.x; i < T; i += blockDim.x) {
+    double x[3];
+    ta.pos(i, x);
+    for (int c = 0; c < 3; ++c) {
+      int e;
+      fx_mant(x[c] - cen[c], &e);
+      if (e <= 1024) m = max(m, e);  // not the exponent of an infinity or a NaN
+    }
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, m);
+  __syncthreads();
+  return *slot + 1;
 }
 
 // Shared-memory bytes of the moment workspace (either engine's).
@@ -859,15 +883,17 @@ __device__ __forceinline__ SegMap seg_T0() { return {0.0, 0.0, 1.0, 0.0, 0.0, 1.
 // two cross products).  Thread per node; targets staged through shared memory.
 // WARP_ACC: M is instead this warp's row of per-warp sums in shared memory; every lane
 // takes part (zeros for lanes without a node) and lane 0 adds the warp's sum.
+// scratch: 5 kGradTile doubles of shared memory.
+constexpr int kGradTile = 32;
 template <int D, bool WARP_ACC = false, class TA, class WF>
 __device__ void block_grad(const double* cf, const double* __restrict__ ru,
                            const double* __restrict__ rv, const double* __restrict__ rw, int Q,
                            const SegMap* segs, int nseg, const TA& ta, int T, WF wf,
                            const KernelParams& kp, const cplx* shat, const double* cen,
-                           double* M) {
-  constexpr int TG = 32;
-  __shared__ double gx[TG][3];
-  __shared__ cplx gwt[TG];
+                           double* M, double* scratch) {
+  constexpr int TG = kGradTile;
+  double (*gx)[3] = reinterpret_cast<double (*)[3]>(scratch);
+  cplx* gwt = reinterpret_cast<cplx*>(scratch + 3 * TG);
   const int total = nseg * Q;
   for (int c0 = 0; c0 < total; c0 += blockDim.x) {
     const int q = c0 + threadIdx.x;
@@ -1041,7 +1067,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
   long long my_tests = 0, my_nodes = 0, my_tree = 0;
   __shared__ int next_b, next_g;
   __shared__ KernelParams kps;
-  __shared__ double cfd[2 * 3 * (D * (D + 1) / 2)];  // derivative series of the chart
+  // derivative series of the chart, for the FP64 engine of the smallest degrees
+  __shared__ double cfd[D <= kFp64MomentsMaxDeg ? 2 * 3 * (D * (D + 1) / 2) : 1];
+  __shared__ FxChart<D> ch;
+  __shared__ int tsc;
   const double* cfdp = cfd;
 
   for (;;) {
@@ -1090,7 +1119,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
     load_coef<D>(dv.coef, dv.node_off[j], cf);
     if (threadIdx.x == 0) kps = patch_kp(dv, j, kp);  // read after block_moments' barrier
     __syncthreads();
-    load_coef_derivs<D>(cf, dv.duv[D], cfd);
+    if constexpr (D <= kFp64MomentsMaxDeg) load_coef_derivs<D>(cf, dv.duv[D], cfd);
+    load_fx_chart<D>(cf, dv.duv[D], &ch);
+    const int S2 = block_scale(TgtPairIdx{dv.tgt, dv.NT, dv.pair_tgt, apairs, dv.tnrm}, A,
+                               dv.cen + 3 * j, ch.sx, &tsc);
     if constexpr (GRAD) {
 #pragma unroll
       for (int e = 0; e < 3 * n; ++e) Mg[e] = 0.0;
@@ -1114,7 +1146,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
     __syncthreads();
     if (leaf_order > 0) {
       TgtPairIdx ta{dv.tgt, dv.NT, dv.pair_tgt, apairs, dv.tnrm};
-      block_moments_any<D>(cf, cfdp, ru, rv, rw, Q, segs, 1, ta, A,
+      block_moments_any<D>(cf, cfdp, ch, S2, ru, rv, rw, Q, segs, 1, ta, A,
                            [=] __device__(int i) { return lvlI + (int64_t)i * 4 * n; }, kps, smb,
                            dv.cen + 3 * j, Rj, tmpE, formj);
     }
@@ -1166,7 +1198,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
       __syncthreads();
       // children moments of every target in S
       TgtAdaptive ta{dv.tgt, dv.NT, dv.pair_tgt, apairs, ST, dv.tnrm};
-      block_moments_any<D>(cf, cfdp, ru, rv, rw, Q, segs, 4, ta, S,
+      block_moments_any<D>(cf, cfdp, ch, S2, ru, rv, rw, Q, segs, 4, ta, S,
                            [=] __device__(int i) { return tmp + (int64_t)i * 4 * n; }, kps, smb,
                            dv.cen + 3 * j, Rj, tmpE, formj);
       __syncthreads();
@@ -1219,7 +1251,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
                         const cplx c = gt[dv.pair_tgt[apairs[ST[i]]]];
                         return {c.re, -c.im};
                       },
-                      kps, shat, dv.cen + 3 * j, Mg);
+                      kps, shat, dv.cen + 3 * j, Mg, ws);
       }
       // stable compaction of the refining targets into level L+1
       int base = 0;

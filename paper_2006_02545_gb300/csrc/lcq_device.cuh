@@ -108,7 +108,9 @@ inline const FxHostTables& fx_host_tables() {
   return t;
 }
 
-// Fills c_kw, c_jac, c_kwexp, g_sct, g_sctf, g_fxcs and g_fxdec of the calling translation unit.
+// Fills c_kw, c_jac, c_kwexp, g_sct, g_sctf, g_fxcs, g_fxdec and the tables of the fixed-point
+// basis of the calling translation unit.
+static inline cudaError_t upload_fx_basis(const int* kwexp, cudaStream_t st);
 static inline cudaError_t upload_kw_tables(cudaStream_t st) {
   double c[kMaxBasis], jc[(kMaxDeg + 1) * (kMaxDeg + 1) * 3] = {};
   int ke[kMaxBasis];
@@ -154,6 +156,7 @@ static inline cudaError_t upload_kw_tables(cudaStream_t st) {
   if (e == cudaSuccess)
     e = cudaMemcpyToSymbolAsync(g_fxdec, fxt.dec.data(), sizeof(u64) * kFxTab, 0,
                                 cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = upload_fx_basis(ke, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the sources live on this stack
   return e;
 }
@@ -810,3 +813,5 @@ __device__ __forceinline__ void cross3(const double* a, const double* b, double*
 }
 
 }  // namespace lcq
+
+#include "lcq_fxgeom.cuh"

@@ -59,6 +59,12 @@ LCQ_HD i64 fx_smul(FxS a, FxS b) {
   const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h);
   return fx_swide(a.h, b.h) + (t >> 31);
 }
+// a b / 2^(64 - K), the extra bits kept
+template <int K>
+LCQ_HD i64 fx_smul_sl(FxS a, FxS b) {
+  const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h);
+  return fx_swide(a.h, b.h) * (1ll << K) + (t >> (31 - K));
+}
 // (a b + c d) / 2^61, |a|, |c| < 2^62.3, |b|, |d| < 2^61
 LCQ_HD i64 fx_dot2(FxS a, FxS b, FxS c, FxS d) {
   const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h) + fx_swide(c.h, d.l) + fx_swide(c.l, d.h);
@@ -121,6 +127,7 @@ struct FxKernel {
   int neg;       // kr < 0: the phase's sign
   int single;    // the single layer alone (alpha = 0, beta = 1)
   int cplx;      // Im(alpha) or p not zero
+  int has;       // 1: Re(beta) not zero, 2: Im(beta) not zero, 4: Re(alpha) = 1
 };
 
 // kind, k, alpha, beta as KernelParams holds them (kind 0: S, 1 and 3: D form, 2: CFIE).
@@ -163,6 +170,7 @@ LCQ_HD FxKernel fx_kernel(int kind, double kr, double ki, double ar, double ai, 
   f.br = fx_split(fx_fix(br, f.eb));
   f.bi = fx_split(fx_fix(bi, f.eb));
   f.cplx = ai != 0.0 || p != 0.0;
+  f.has = (br != 0.0 ? 1 : 0) | (bi != 0.0 ? 2 : 0) | (ar == 1.0 && ai == 0.0 ? 4 : 0);
   return f;
 }
 
@@ -267,60 +275,57 @@ LCQ_HD double fx_pack(i64 v, int e) {
   return fx_double(b);
 }
 
-// The kernel value of one pair from d = x - X (FP64).  False (and nothing written) for
-// arguments that it does not cover: |d| outside [2^-300, 2^300] (zero among them), a phase
-// above 2^24 turns, a decay above 2^9 halvings, values that are not finite.  With env the
-// rounding envelope |G| Jw (eb + ea |1 - ikr| R / r^2) in FP32 (fk: |kr|, fki: ki, fe = eb, fa =
-// ea R, fw = W in FP32).
-template <bool INT>
-LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1, double d2,
-                    const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
-                    float fki, float feb, float feaR, float fw) {
-  const u64 b0 = fx_bits(d0), b1 = fx_bits(d1), b2 = fx_bits(d2);
-  const int x0 = (int)(fx_hi(b0) & 0x7fffffffu) >> 20, x1 = (int)(fx_hi(b1) & 0x7fffffffu) >> 20,
-            x2 = (int)(fx_hi(b2) & 0x7fffffffu) >> 20;
-  const int ex = fx_max(x0, fx_max(x1, x2));
-  const int sh = ex - 1022 + K.ek + 8;
-  if ((unsigned)(ex - 723) > 600u || sh > 30 || ew > kFxBad) return false;
-  const int E = ex - 1022;
-  // d = D 2^(E - 62)
-  i64 D[3];
-  {
-    const u64 b[3] = {b0, b1, b2};
-    const int xs[3] = {x0, x1, x2};
-#ifdef __CUDACC__
-#pragma unroll
+LCQ_HD int fx_clz(u64 v) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)v);
+#else
+  return v == 0 ? 64 : __builtin_clzll(v);
 #endif
-    for (int c = 0; c < 3; ++c) {
-      const u64 m = ((b[c] & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
-      const int s = fx_min(ex - xs[c], 63);
-      const i64 v = (i64)(m >> s);
-      const i64 g = (i64)b[c] >> 63;
-      D[c] = v ^ g;
-    }
-  }
-  const FxS D0 = fx_split(D[0]), D1 = fx_split(D[1]), D2 = fx_split(D[2]);
-  // r^2 = r2 2^(2E - 60), r2 in [2^58, 3 2^60]
+}
+
+// Length of the vector D 2^(E - 62), 2^61 <= max |D_c| < 2^62: R 2^(E - 62) with its inverse
+// RI 2^(-61 - E); 2^61 <= R < 2^62.8, 2^60.2 < RI <= 2^62.  r2 = |D|^2 / 2^64 in [2^58, 3 2^60];
+// f = r2 2^-32 and y = f^(-1/2) to 22 bits from the special function unit; then Y = y 2^44,
+// the residual e = 1 - r2 Y^2 2^-120 exactly enough, and RI = Y 2^31 (1 + e/2 + 3 e^2 / 8).
+struct FxRoot {
+  u64 RI, R;
+  float f, y;
+};
+LCQ_HD FxRoot fx_root(FxS D0, FxS D1, FxS D2) {
   const i64 cr = fx_swide(D0.h, D0.l) + fx_swide(D1.h, D1.l) + fx_swide(D2.h, D2.l);
   const u64 r2 = (u64)(fx_swide(D0.h, D0.h) + fx_swide(D1.h, D1.h) + fx_swide(D2.h, D2.h) +
                        (cr >> 30));
-  // 1/r = RI 2^(-61 - E): Y = 2^60 / sqrt(r2) to 22 bits from the special function unit, its
-  // residual e = 1 - r2 Y^2 exactly enough, and RI = Y 2^31 (1 + e/2 + 3 e^2 / 8)
-  const float f = (float)fx_hi(r2);
+  FxRoot o;
+  o.f = (float)fx_hi(r2);
 #ifdef __CUDA_ARCH__
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
-  const uint32_t Y = __float2uint_rz(y * 17592186044416.0f);
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(o.y) : "f"(o.f));
+  const uint32_t Y = __float2uint_rz(o.y * 17592186044416.0f);
 #else
-  const float y = 1.0f / sqrtf(f);
-  const uint32_t Y = (uint32_t)(y * 17592186044416.0f);
+  o.y = 1.0f / sqrtf(o.f);
+  const uint32_t Y = (uint32_t)(o.y * 17592186044416.0f);
 #endif
-  const u64 G = fx_umul32(r2, Y);                       // sqrt(r2) 2^28
+  const u64 G = fx_umul32(r2, Y);                        // sqrt(r2) 2^28
   const i64 e1 = (i64)((1ull << 56) - fx_umul32(G, Y));  // unit 2^-56
   const int e2 = (int)(e1 >> 8);
   const i64 c1 = (e1 + (i64)(((int)(fx_swide(e2, e2) >> 32) * 3) >> 10)) >> 1;
-  const u64 RI = ((u64)Y << 31) + (u64)(((i64)(Y >> 4) * c1) >> 21);
-  const u64 R = fx_umul(r2 << 1, RI) << 4;              // r = R 2^(E - 62)
+  o.RI = ((u64)Y << 31) + (u64)(((i64)(Y >> 4) * c1) >> 21);
+  o.R = fx_umul(r2 << 1, o.RI) << 4;
+  return o;
+}
+
+// The kernel value of one pair from d = x - X = D 2^(E - 62), 2^61 <= max |D_c| < 2^62.  False
+// (and nothing written) for arguments that it does not cover: a phase above 2^22 turns, a decay
+// above 2^9 halvings, a node that is not finite (ew above kFxBad).  With env the rounding
+// envelope |G| Jw (eb + ea |1 - ikr| R / r^2) in FP32 (fk: |kr|, fki: ki, feb = eb, feaR = ea R,
+// fw = W in FP32).
+template <bool INT>
+LCQ_HD bool fx_core(const FxKernel& K, const FxTables& tab, FxS D0, FxS D1, FxS D2, int E,
+                    const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
+                    float fki, float feb, float feaR, float fw) {
+  const int sh = E + K.ek + 8;
+  if (sh > 30 || ew > kFxBad) return false;
+  const FxRoot rt = fx_root(D0, D1, D2);
+  const u64 RI = rt.RI, R = rt.R;
   // the phase in turns 2^-64 and e^{ikr}
   u64 ph = fx_umul(R, K.kt);                            // kr / 2 pi = ph 2^(E + ek - 60)
   ph = sh >= 4 ? ph << (sh - 4) : ph >> fx_min(4 - sh, 63);
@@ -355,7 +360,7 @@ LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1
 #else
     const float sc = ldexpf(1.0f, -eb), rs = ldexpf(1.0f, eb);
 #endif
-    const float fri = y * 16384.0f * sc, fr = f * y * rs * 6.103515625e-05f * 1.0f;
+    const float fri = rt.y * 16384.0f * sc, fr = rt.f * rt.y * rs * 6.103515625e-05f;
     const float fo = fki * fr + 1.0f, f1 = fk * fr;
     const float fab = sqrtf(fo * fo + f1 * f1);
     float g = fri * fw;
@@ -384,9 +389,11 @@ LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1
   const int eb = K.eb + E, ep = K.ep + E;
   const int eA = fx_max(K.ea, fx_max(eb, ep));
   const int sb = eA - eb, sa = eA - K.ea, sp = eA - ep;
-  i64 A = fx_sra(fx_smul(K.br, Rs), sb) + fx_sra(fx_smul(K.ar, c), sa);
-  i64 B = fx_sra(fx_smul(K.bi, Rs), sb) +
-          fx_sra(fx_smul(fx_split(fx_smul(K.q, Rs) << 2), c), sp);
+  // (branches on the constants are uniform; alpha = 1 has ea = 1)
+  i64 A = fx_sra((K.has & 4) ? ((i64)c.h << 29) + (c.l >> 2) : fx_smul(K.ar, c), sa);
+  i64 B = fx_sra(fx_smul(fx_split(fx_smul(K.q, Rs) << 2), c), sp);
+  if (K.has & 1) A += fx_sra(fx_smul(K.br, Rs), sb);
+  if (K.has & 2) B += fx_sra(fx_smul(K.bi, Rs), sb);
   if (K.cplx) {
     A += fx_sra(fx_smul(fx_split(fx_smul(K.p, Rs) << 2), c), sp);
     B += fx_sra(fx_smul(K.ai, c), sa);
@@ -396,6 +403,40 @@ LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1
   *re = fx_pack<INT>(fx_dot2(As, ec, Bn, es), ev);
   *im = fx_pack<INT>(fx_dot2(As, es, Bs, ec), ev);
   return true;
+}
+
+// The same from FP64 coordinates of d; also false for |d| outside [2^-300, 2^300], zero among them.
+template <bool INT>
+LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1, double d2,
+                    const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
+                    float fki, float feb, float feaR, float fw) {
+  const u64 b[3] = {fx_bits(d0), fx_bits(d1), fx_bits(d2)};
+  int xs[3];
+  for (int c = 0; c < 3; ++c) xs[c] = (int)(fx_hi(b[c]) & 0x7fffffffu) >> 20;
+  const int ex = fx_max(xs[0], fx_max(xs[1], xs[2]));
+  if ((unsigned)(ex - 723) > 600u) return false;
+  FxS D[3];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+  for (int c = 0; c < 3; ++c) {
+    const u64 m = ((b[c] & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
+    D[c] = fx_split((i64)(m >> fx_min(ex - xs[c], 63)) ^ ((i64)b[c] >> 63));
+  }
+  return fx_core<INT>(K, tab, D[0], D[1], D[2], ex - 1022, n, w, ew, re, im, env, fk, fki, feb,
+                      feaR, fw);
+}
+
+// The same from d = (d0, d1, d2) 2^(S - 62), |d_c| < 2^62; also false for d = 0.
+template <bool INT>
+LCQ_HD bool fx_eval_int(const FxKernel& K, const FxTables& tab, i64 d0, i64 d1, i64 d2, int S,
+                        const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
+                        float fki, float feb, float feaR, float fw) {
+  const int sh = fx_clz((u64)((d0 ^ (d0 >> 63)) | (d1 ^ (d1 >> 63)) | (d2 ^ (d2 >> 63)))) - 2;
+  const int E = S - sh;
+  if (sh > 61 || (unsigned)(E + 300) > 600u) return false;
+  return fx_core<INT>(K, tab, fx_split(d0 << sh), fx_split(d1 << sh), fx_split(d2 << sh), E, n, w,
+                      ew, re, im, env, fk, fki, feb, feaR, fw);
 }
 
 }  // namespace lcq

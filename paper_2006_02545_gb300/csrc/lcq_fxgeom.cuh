@@ -1,0 +1,311 @@
+// The chart and the Koornwinder basis at the leaf nodes in 64-bit fixed point.
+//
+// The moment engine needs, at every node of every subtriangle of the refinement trees, the
+// basis values as 7-bit slices of a 56-bit integer (block_moments_tc), the point X and the
+// normal X_u x X_v.  In FP64 that is about 170 instructions of 64 cycles a node and 250 a rule
+// row.  The basis is bounded on the triangle by construction (|L_m| <= 1, |K_nm| < 2^E_nm) and the
+// chart by the sum of its coefficients, so the same recurrences run on 62-bit integers: a
+// product is three 32 x 32 multiply-adds of 4 cycles, and the basis slices come out of the
+// integers directly.  A basis value carries 2^-57 of its bound 2^E_nm, X 2^-56 of the chart's
+// coefficient sum and the unit normal 2^-55: below FP64's rounding of the same recurrences.
+#pragma once
+
+#include "lcq_device.cuh"
+
+namespace lcq {
+
+// A value as its high word and 28 bits of the low one, v = h 2^32 + 16 l: sums of up to 16
+// cross products of such pairs stay below 2^63.
+__device__ __forceinline__ u64 fx_join28(i64 v) {
+  return ((u64)(v >> 32) << 32) | ((uint32_t)v >> 4);
+}
+__device__ __forceinline__ FxS fx_28(FxS a) { return {a.h, a.l >> 3}; }
+
+// Jacobi recurrences of the scaled basis factors (fx_row_factors), filled by upload_kw_tables:
+// [m][a]: g1, g0, g2 2^60, and the first factor 2^62 of each m.
+static __constant__ i64 c_fxj[(kMaxDeg + 1) * (kMaxDeg + 1) * 3];
+static __constant__ i64 c_fxj0[kMaxDeg + 1];
+// (m - 1) / m (2 / a_m) (2 / a_{m-1}), a_j = (2j - 1) / j: coefficient of (1 - v)^2 in the
+// recurrence of the scaled L_m
+static __constant__ double c_fxq[kMaxDeg + 1];
+
+// Host values of the three tables.  kwexp: E_nm.
+struct FxBasisTables {
+  i64 j[(kMaxDeg + 1) * (kMaxDeg + 1) * 3];
+  i64 j0[kMaxDeg + 1];
+  double q[kMaxDeg + 1];
+};
+inline FxBasisTables fx_basis_tables(const int* kwexp) {
+  FxBasisTables t{};
+  auto idx = [](int n, int m) { return n * (n + 1) / 2 + m; };
+  auto root = [](double p, double q) {  // sqrt(p / q)
+    const HostDD x = dd_div({p, 0.0}, q);
+    const double h = sqrt(x.h);
+    return HostDD{h, (fma(-h, h, x.h) + x.l) / (2.0 * h)};
+  };
+  auto fix = [](HostDD a, int e) {  // a 2^e rounded
+    const double f = ldexp(1.0, e), x = a.h * f;
+    const i64 i = (i64)x;
+    return i + llrint((x - (double)i) + a.l * f);
+  };
+  auto rat = [&](double p, double q, HostDD r) { return dd_div(dd_mul({p, 0.0}, r), q); };
+  HostDD kappa = {1.0, 0.0};
+  for (int m = 0; m <= kMaxDeg; ++m) {
+    if (m >= 2) kappa = rat(2.0 * m - 1.0, 2.0 * m, kappa);
+    t.q[m] = m < 2 ? 0.0 : (m - 1.0) / m * (2.0 * m / (2.0 * m - 1.0)) *
+                               (m == 2 ? 1.0 : 2.0 * (m - 1) / (2.0 * m - 3.0));
+    auto E = [&](int a) { return kwexp[idx(m + a, m)]; };
+    t.j0[m] = fix(dd_mul(kappa, root(2.0 * (2 * m + 1) * (m + 1), 1.0)), 62 - E(0));
+    const int b = 2 * m + 1;
+    for (int a = 0; m + a < kMaxDeg; ++a) {
+      // jacobi_coef times the ratios of c_nm 2^-E_nm
+      const double den = 2.0 * (a + 1) * (a + b + 1) * (2 * a + b);
+      const HostDD r1 = root(m + a + 2, m + a + 1), r2 = root(m + a + 2, a > 0 ? m + a : 1);
+      i64* g = t.j + (m * (kMaxDeg + 1) + a) * 3;
+      g[0] = fix(rat((2.0 * a + b + 1) * (2 * a + b + 2) * (2 * a + b), den, r1), 60 + E(a) - E(a + 1));
+      g[1] = -fix(rat((2.0 * a + b + 1) * b * b, den, r1), 60 + E(a) - E(a + 1));
+      g[2] = a == 0 ? 0 : fix(rat(2.0 * a * (a + b) * (2 * a + b + 2), den, r2),
+                              60 + E(a - 1) - E(a + 1));
+    }
+  }
+  return t;
+}
+
+static inline cudaError_t upload_fx_basis(const int* kwexp, cudaStream_t st) {
+  const FxBasisTables t = fx_basis_tables(kwexp);
+  cudaError_t e = cudaMemcpyToSymbolAsync(c_fxj, t.j, sizeof(t.j), 0, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyToSymbolAsync(c_fxj0, t.j0, sizeof(t.j0), 0, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyToSymbolAsync(c_fxq, t.q, sizeof(t.q), 0, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // t lives on this stack
+  return e;
+}
+
+// A patch's chart in fixed point: coefficients x_nm 2^(E_nm + 62 - sx) and the derivative
+// series' with their own scales su and sv, each scale above the sum of the magnitudes, so that
+// every partial sum stays below 1.  bad: a coefficient is not finite.
+template <int D>
+struct FxChart {
+  static constexpr int n = (D + 1) * (D + 2) / 2, nd = D * (D + 1) / 2;
+  u64 x[3 * n];
+  u64 d[6 * nd];   // X_u then X_v
+  int sx, su, sv, bad;
+};
+
+// By the block's threads, from the coefficients cf and the projections duv (load_coef_derivs);
+// begins and ends with a barrier.
+template <int D>
+__device__ void load_fx_chart(const double* cf, const double* __restrict__ duv, FxChart<D>* ch) {
+  constexpr int n = FxChart<D>::n, nd = FxChart<D>::nd;
+  __syncthreads();
+  load_coef_derivs<D>(cf, duv, reinterpret_cast<double*>(ch->d));
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int c = 0; c < 3; ++c) {
+      double a = 0.0, b = 0.0, e = 0.0;
+      for (int i = threadIdx.x; i < n; i += 32) {
+        const double p2 = __longlong_as_double((long long)(c_kwexp[i] + 1023) << 52);
+        a += fabs(cf[3 * i + c]) * p2;
+        if (i < nd) {
+          b += fabs(reinterpret_cast<const double*>(ch->d)[3 * i + c]) * p2;
+          e += fabs(reinterpret_cast<const double*>(ch->d)[3 * (nd + i) + c]) * p2;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+        e += __shfl_xor_sync(0xffffffffu, e, o);
+      }
+      s[0] = fmax(s[0], a);
+      s[1] = fmax(s[1], b);
+      s[2] = fmax(s[2], e);
+      if (!isfinite(a + b + e)) s[0] = s[1] = s[2] = a + b + e;
+    }
+    if (threadIdx.x == 0) {
+      int e[3];
+      for (int k = 0; k < 3; ++k) {
+        fx_mant(s[k], &e[k]);
+        e[k] = max(e[k], -1000);
+      }
+      ch->sx = e[0];
+      ch->su = e[1];
+      ch->sv = e[2];
+      ch->bad = !(s[0] < 1e300 && s[1] < 1e300 && s[2] < 1e300);
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 3 * n; i += blockDim.x)
+    ch->x[i] = fx_join28(fx_fix(cf[i], ch->sx - c_kwexp[i / 3]));
+  for (int i = threadIdx.x; i < 6 * nd; i += blockDim.x) {
+    const int k = i / 3;
+    const double v = reinterpret_cast<const double*>(ch->d)[i];
+    ch->d[i] = k < nd ? fx_join28(fx_fix(v, ch->su - c_kwexp[k]))
+                      : fx_join28(fx_fix(v, ch->sv - c_kwexp[k - nd]));
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ void fx_mac28(i64& hh, i64& t, FxS a, FxS b) {
+  hh += fx_swide(a.h, b.h);
+  t += fx_swide(a.h, b.l) + fx_swide(a.l, b.h);
+}
+
+// A rule row (nodes of one v): [Q (D+1), J (n), BX (3 (D+1)), BU (3 D), BV (3 D)], 62-bit values:
+// Q[m] the (1 - v)^2 term of the L recurrence, J_nm 2^-E_nm times the scale of L_m (split with 31
+// bits), BX, BU, BV the chart's sums over n at fixed m (28 bits).
+template <int D>
+struct FxRow {
+  static constexpr int n = (D + 1) * (D + 2) / 2;
+  static constexpr int Q = 0, J = Q + D + 1, BX = J + n, BU = BX + 3 * (D + 1), BV = BU + 3 * D;
+  static constexpr int size = BV + 3 * D;
+};
+
+// The part of the row factors that belongs to one m (Q too when m = 0), so that a block
+// spreads a row over D + 1 threads.
+template <int D>
+__device__ __forceinline__ void fx_row_factors(double v, int m, const FxChart<D>& ch, u64* row) {
+  using RW = FxRow<D>;
+  constexpr int nd = FxChart<D>::nd;
+  if (m == 0) {
+    const double q2 = (1.0 - v) * (1.0 - v);
+#pragma unroll 1
+    for (int mm = 2; mm <= D; ++mm) row[RW::Q + mm] = fx_join(fx_split(fx_fix(c_fxq[mm] * q2, 0)));
+  }
+  const FxS y = fx_split(fx_fix(1.0 - 2.0 * v, 0));
+  const i64* g = c_fxj + m * (kMaxDeg + 1) * 3;
+  i64 J = c_fxj0[m], Jp = 0;
+  i64 h[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, t[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+  for (int a = 0; a <= D - m; ++a) {
+    const int nn = m + a, idx = nn * (nn + 1) / 2 + m;
+    const FxS Js = fx_split(J), J8 = fx_28(Js);
+    row[RW::J + idx] = fx_join(Js);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) fx_mac28(h[c], t[c], J8, fx_unjoin(ch.x[idx * 3 + c]));
+    if (nn < D) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        fx_mac28(h[3 + c], t[3 + c], J8, fx_unjoin(ch.d[idx * 3 + c]));
+        fx_mac28(h[6 + c], t[6 + c], J8, fx_unjoin(ch.d[(nd + idx) * 3 + c]));
+      }
+      // J_{a+1} = (g1 y + g0) J_a - g2 J_{a-1}
+      const FxS f = fx_split((fx_smul(fx_split(g[3 * a]), y) << 2) + g[3 * a + 1]);
+      const FxS g2 = fx_split(g[3 * a + 2]), Jq = fx_split(Jp);
+      const i64 tt = fx_swide(f.h, Js.l) + fx_swide(f.l, Js.h) - fx_swide(g2.h, Jq.l) -
+                     fx_swide(g2.l, Jq.h);
+      Jp = J;
+      J = (i64)((u64)(fx_swide(f.h, Js.h) - fx_swide(g2.h, Jq.h)) << 4) + (tt >> 27);
+    }
+  }
+  auto out = [&](int o, int k) { row[o] = fx_join28((h[k] << 2) + (t[k] >> 26)); };
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    out(RW::BX + 3 * m + c, c);
+    if (m < D) {
+      out(RW::BU + 3 * m + c, 3 + c);
+      out(RW::BV + 3 * m + c, 6 + c);
+    }
+  }
+}
+
+// Next of the scaled L_m (|L| < 2.84, unit 2^-61): 2 s L - Q Lp, s 2^62 and Q 2^62.
+__device__ __forceinline__ i64 fx_next_L(FxS s, FxS L, FxS Q, FxS Lp) {
+  const i64 ta = fx_swide(s.h, L.l) + fx_swide(s.l, L.h);
+  const i64 tb = fx_swide(Q.h, Lp.l) + fx_swide(Q.l, Lp.h);
+  return (i64)(((u64)fx_swide(s.h, L.h) << 3) - ((u64)fx_swide(Q.h, Lp.h) << 2) +
+               (u64)((ta >> 28) - (tb >> 29)));
+}
+
+// X (2^(59 - sx)), and the normal X_u x X_v (2^(61 - su - sv)) of the node at s = 2u + v - 1 of a row.
+template <int D>
+__device__ __forceinline__ void fx_chart_point(FxS s, const u64* row, i64* X, i64* N) {
+  using RW = FxRow<D>;
+  i64 h[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, t[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  FxS L = {1 << 29, 0}, Lp = {0, 0};
+#pragma unroll
+  for (int m = 0; m <= D; ++m) {
+    if (m == 1) {
+      Lp = L;
+      L = {s.h >> 1, (int)(((uint32_t)(s.h & 1) << 30) | ((uint32_t)s.l >> 1))};
+    } else if (m > 1) {
+      const FxS Ln = fx_split(fx_next_L(s, L, fx_unjoin(row[RW::Q + m]), Lp));
+      Lp = L;
+      L = Ln;
+    }
+    const FxS L8 = fx_28(L);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      fx_mac28(h[c], t[c], L8, fx_unjoin(row[RW::BX + 3 * m + c]));
+      if (m < D) {
+        fx_mac28(h[3 + c], t[3 + c], L8, fx_unjoin(row[RW::BU + 3 * m + c]));
+        fx_mac28(h[6 + c], t[6 + c], L8, fx_unjoin(row[RW::BV + 3 * m + c]));
+      }
+    }
+  }
+  FxS d[6];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) X[c] = h[c] + (t[c] >> 28);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) d[c] = fx_split((h[3 + c] << 3) + (t[3 + c] >> 25));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const FxS a = d[(c + 1) % 3], b = d[3 + (c + 2) % 3], e = d[(c + 2) % 3], f = d[3 + (c + 1) % 3];
+    const i64 tt = fx_swide(a.h, b.l) + fx_swide(a.l, b.h) - fx_swide(e.h, f.l) - fx_swide(e.l, f.h);
+    N[c] = (i64)((u64)(fx_swide(a.h, b.h) - fx_swide(e.h, f.h)) << 1) + (tt >> 30);
+  }
+}
+
+// Basis values of the node: emit(idx, K_nm 2^(59 - E_nm)) for the m of one part of `parts`.
+template <int D, class F>
+__device__ __forceinline__ void fx_basis_point(FxS s, const u64* row, int part, int parts, F&& emit) {
+  using RW = FxRow<D>;
+  FxS L = {1 << 29, 0}, Lp = {0, 0};
+#pragma unroll
+  for (int m = 0; m <= D; ++m) {
+    if (m == 1) {
+      Lp = L;
+      L = {s.h >> 1, (int)(((uint32_t)(s.h & 1) << 30) | ((uint32_t)s.l >> 1))};
+    } else if (m > 1) {
+      const FxS Ln = fx_split(fx_next_L(s, L, fx_unjoin(row[RW::Q + m]), Lp));
+      Lp = L;
+      L = Ln;
+    }
+    if (parts > 1 && m % parts != part) continue;
+#pragma unroll
+    for (int a = 0; a <= D - m; ++a) {
+      const int nn = m + a, idx = nn * (nn + 1) / 2 + m;
+      emit(idx, fx_smul(L, fx_unjoin(row[RW::J + idx])));
+    }
+  }
+}
+
+// The node for fx_eval from the integer normal N 2^(sn - 62) and the rule weight wt (area of the
+// subtriangle included): unit normal 2^62, W = |N| wt / (4 pi) = wm 2^(ew - 62).
+__device__ __forceinline__ void fx_node_from_normal(const i64* N, int sn, double wt, FxS* n, u64* wm,
+                                                    int* ew) {
+  const int sh =
+      fx_clz((u64)((N[0] ^ (N[0] >> 63)) | (N[1] ^ (N[1] >> 63)) | (N[2] ^ (N[2] >> 63)))) - 2;
+  if (sh > 60) {  // no area
+    n[0] = n[1] = n[2] = {0, 0};
+    *wm = 0;
+    *ew = 0;
+    return;
+  }
+  const FxS a = fx_split(N[0] << sh), b = fx_split(N[1] << sh), c = fx_split(N[2] << sh);
+  const FxRoot rt = fx_root(a, b, c);
+  const FxS ri = fx_split((i64)rt.RI);
+  n[0] = fx_split(fx_smul_sl<3>(a, ri));
+  n[1] = fx_split(fx_smul_sl<3>(b, ri));
+  n[2] = fx_split(fx_smul_sl<3>(c, ri));
+  int e;
+  const u64 m = (u64)fx_mant(wt * 0.07957747154594767, &e);
+  const u64 p = fx_umul(rt.R, m);  // |N| W = p 2^(sn - sh + e - 60)
+  const int z = fx_clz(p) - 2;
+  *wm = z >= 0 && p != 0 ? p << z : p;
+  *ew = sn - sh + e + 2 - (p != 0 ? z : 0);
+}
+
+}  // namespace lcq

@@ -46,12 +46,12 @@ __global__ void __launch_bounds__(256) k_check_tc(int nq, unsigned long long see
   using C = TcCfg<D>;
   constexpr int n = C::n;
   extern __shared__ __align__(128) unsigned char smb[];
-  uint16_t* Bsl = reinterpret_cast<uint16_t*>(smb + C::OFF_BS);
-  cplx* Gs = reinterpret_cast<cplx*>(smb + C::OFF_G);
-  uint16_t* Asl = reinterpret_cast<uint16_t*>(smb + C::OFF_G);
-  int* rowE = reinterpret_cast<int*>(smb + C::OFF_ROWE);
-  __shared__ cplx A0[C::TT][C::CH];
-  __shared__ double Bref[C::CH][n];
+  uint2* Bs = reinterpret_cast<uint2*>(smb + C::OFF_B);
+  uint4* G = reinterpret_cast<uint4*>(smb + C::OFF_G);
+  int* rowE = reinterpret_cast<int*>(smb + C::OFF_RE);
+  constexpr int NQ = D <= 6 ? 128 : 64;  // nq at most
+  __shared__ cplx A0[C::TT][NQ];
+  __shared__ double Bref[NQ][n];
   __shared__ cplx res[C::TT][n];
   const int ncp = (nq + 15) & ~15;
   auto rnd = [&](unsigned long long k) {  // splitmix64 of (seed, k) -> [0, 1)
@@ -61,20 +61,17 @@ __global__ void __launch_bounds__(256) k_check_tc(int nq, unsigned long long see
     z ^= z >> 31;
     return (double)(z >> 11) * (1.0 / 9007199254740992.0);
   };
-  for (int e = threadIdx.x; e < C::CH * C::NP; e += blockDim.x) {
-    const int q = e / C::NP, nm = e - q * C::NP;
+  for (int e = threadIdx.x; e < NQ * C::NTILE * 8; e += blockDim.x) {
+    const int q = e / (C::NTILE * 8), nm = e - q * C::NTILE * 8;
     double b = 0.0;
     if (q < nq && nm < n) b = (2.0 * rnd(4 * e) - 1.0) * ldexp(1.0, c_kwexp[nm]) * rnd(4 * e + 1);
     if (nm < n) {
       Bref[q][nm] = b;
-      store_basis_slices<D>(Bsl, nm, q, b);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) Bsl[(size_t)i * C::NP * C::CH + C::swz(nm, q)] = 0;
+      Bs[nm * C::BST + q] = slice_bytes(fix_mag<8>(b, c_kwexp[nm]), b < 0.0);
     }
   }
-  for (int e = threadIdx.x; e < C::TT * C::CH; e += blockDim.x) {
-    const int t = e / C::CH, q = e - t * C::CH;
+  for (int e = threadIdx.x; e < C::TT * NQ; e += blockDim.x) {
+    const int t = e / NQ, q = e - t * NQ;
     cplx a = {0.0, 0.0};
     if (q < nq) {
       const double mag = pow(10.0, 12.0 * rnd(1000003 + 3 * e) - 6.0);
@@ -82,25 +79,28 @@ __global__ void __launch_bounds__(256) k_check_tc(int nq, unsigned long long see
       a = {mag * cos(ang), mag * sin(ang)};
     }
     A0[t][q] = a;
-    Gs[t * C::CH + q] = a;
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int VPL = C::CH / 32;
-  const int q0 = lane * VPL;
-  double re[VPL], im[VPL];
-#pragma unroll
-  for (int v = 0; v < VPL; ++v) {
-    const cplx g = (q0 + v < ncp) ? Gs[warp * C::CH + q0 + v] : cplx{0.0, 0.0};
-    re[v] = g.re;
-    im[v] = g.im;
+  const int warp = threadIdx.x >> 5;
+  if (threadIdx.x < 2 * C::TT) {
+    int f = 0;
+    for (int q = 0; q < nq; ++q) {
+      const cplx a = A0[threadIdx.x >> 1][q];
+      f = max(f, exp_field((threadIdx.x & 1) ? a.im : a.re));
+    }
+    rowE[threadIdx.x] = f;
   }
   __syncthreads();
-  split_row_pair<D, 8, VPL>(re, im, true, Asl, warp, q0, rowE);
+  for (int e = threadIdx.x; e < C::TT * NQ; e += blockDim.x) {
+    const int t = e / NQ, q = e - t * NQ;
+    const uint2 x = row_slices(A0[t][q].re, exp_bound(rowE[2 * t], 0.0));
+    const uint2 y = row_slices(A0[t][q].im, exp_bound(rowE[2 * t + 1], 0.0));
+    G[t * C::GST + q] = make_uint4(x.x, x.y, y.x, y.y);
+  }
   __syncthreads();
   for (int ct = warp; ct < C::NTILE; ct += blockDim.x >> 5)
-    tc_tile<D, 8, 9>(Bsl, Asl, rowE, ct, 0, ncp, C::TT, 0, 0, true,
-                     [&](int t) { return &res[t][0]; });
+    tc_tile<D, 8, 9, 0x7ff>(Bs, G, rowE, ct, 0, ncp, C::TT, 0, 0, true,
+                            [&](int t) { return &res[t][0]; });
   __syncthreads();
   for (int e = threadIdx.x; e < C::TT * n; e += blockDim.x) {
     const int t = e / n, nm = e - t * n;

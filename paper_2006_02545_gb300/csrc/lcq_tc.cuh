@@ -28,39 +28,30 @@ namespace lcq {
 constexpr int kSliceBits = 7;
 constexpr int kPoisonExp = 0x40000000;  // row exponent marking a non-finite kernel value
 
-// Shared-memory layout of the tensor-core moment engine for degree D (byte offsets).  The
-// f16 slice arrays are [slice][row][CH] with the 16-byte chunks of each row XOR-swizzled by
-// the row index (swz), so that ldmatrix reads 8 rows of one chunk without bank conflicts.
+// Shared-memory layout of the tensor-core moment engine for degree D (byte offsets).  An operand
+// value is eight bytes, one 7-bit slice each (slice_bytes): basis values B[n][BST], kernel values
+// G[TT][GST] (two operands, Re and Im; the FP64 or FP32 values before they are sliced).  The row
+// strides keep the fragment loads of the MMA (128 bits a lane) free of bank conflicts.
 template <int D>
 struct TcCfg {
   static constexpr int n = (D + 1) * (D + 2) / 2;
-  static constexpr int NP = (n + 7) / 8 * 8;       // basis columns padded to MMA n-tiles of 8
-  static constexpr int NTILE = NP / 8;
-  static constexpr int CH = D <= 6 ? 128 : 64;     // padded nodes per chunk (multiple of 16)
+  static constexpr int NTILE = (n + 7) / 8;        // MMA n-tiles of 8 basis columns
+  static constexpr int CH = D <= 6 ? 256 : 128;    // padded nodes per chunk (two blocks fit an SM)
+  static constexpr int CHG = CH / 2;               // columns that share a row scale in the FP32 tier
+  static constexpr int PARTS = 256 / CH;           // threads per node
   static constexpr int TT = 8;                     // targets per tile: 16 MMA rows (Re, then Im)
-  static constexpr int NSMAX = 8;                  // slices per FP64 operand
   static constexpr int MAXP = CH / 16;             // pieces (segment parts) per chunk at most
-  static constexpr int OFF_X = 0;                                  // Xs[3][CH] double
-  static constexpr int OFF_N = OFF_X + 3 * CH * 8;                 // Ns[3][CH] double (N w)
-  static constexpr int OFF_J = OFF_N + 3 * CH * 8;                 // Js[CH] double (J w)
-  static constexpr int OFF_K = OFF_J + CH * 8;                     // Ks[CH] double (folded)
-  static constexpr int OFF_BS = OFF_K + CH * 8;                    // Bsl[NSMAX][NP][CH] f16
-  static constexpr int OFF_G = OFF_BS + NSMAX * NP * CH * 2;       // Gs + Ef / Asl / row factors
-  static constexpr int G_EVAL = TT * CH * 16 + TT * CH * 4;        // Gs[TT][CH] cplx, Ef[TT][CH]
-  static constexpr int G_A = NSMAX * 16 * CH * 2;                  // Asl[NSMAX][16][CH] f16
-  static constexpr int G_BYTES = G_A > G_EVAL ? G_A : G_EVAL;
-  static constexpr int OFF_EF = OFF_G + TT * CH * 16;              // Ef, after Gs
-  static constexpr int OFF_JF = OFF_G + G_BYTES;                   // Jf[CH] float
-  static constexpr int OFF_NF = OFF_JF + CH * 4;                   // Nf[3][CH] float (mixed)
-  static constexpr int OFF_ROWE = OFF_NF + 3 * CH * 4;             // rowE[16] int
-  static constexpr int OFF_TX = (OFF_ROWE + 16 * 4 + 15) / 16 * 16;  // tx[3 TT], tn[3 TT] double
-  static constexpr int OFF_CI = OFF_TX + 6 * TT * 8;               // colinfo[CH] int
-  static constexpr int OFF_PC = OFF_CI + CH * 4;                   // pieces[MAXP][8] int
-  static constexpr int BYTES = OFF_PC + MAXP * 8 * 4;
-  // element (row, k) of a [rows][CH] f16 array, 16-byte chunks XOR-swizzled by row
-  static __device__ __forceinline__ int swz(int row, int k) {
-    return row * CH + ((((k >> 3) ^ (row & 7)) << 3) | (k & 7));
-  }
+  static constexpr int BST = CH + 8;               // B row stride (8-byte values)
+  static constexpr int GST = CH + 1;               // G row stride (16-byte values)
+  static constexpr int OFF_G = 0;                              // G; before it the row factors
+  static constexpr int G_BYTES = TT * GST * 16;
+  static constexpr int OFF_B = (OFF_G + G_BYTES + 15) / 16 * 16;
+  static constexpr int OFF_TX = OFF_B + n * BST * 8;           // tx[3 TT], tn[3 TT]
+  static constexpr int OFF_EP = OFF_TX + 6 * TT * 8;           // Ep[TT][MAXP] float
+  static constexpr int OFF_RE = OFF_EP + TT * MAXP * 4;        // rowE[MAXP][TT][2] int
+  static constexpr int OFF_PC = OFF_RE + MAXP * TT * 2 * 4;    // pieces[MAXP][8] int
+  static constexpr int OFF_TE = OFF_PC + MAXP * 8 * 4;         // te[TT] int: target not finite
+  static constexpr int BYTES = OFF_TE + TT * 4;
 };
 
 // |x| 2^(7 NS - E) rounded to the nearest integer, for |x| < 2^E: below 2^(7 NS).  Zero,
@@ -110,35 +101,28 @@ __device__ __forceinline__ int exp_bound(int field, float) { return field - 126;
 __device__ __forceinline__ bool exp_nonfinite(int field, double) { return field == 0x7ff; }
 __device__ __forceinline__ bool exp_nonfinite(int field, float) { return field == 0xff; }
 
-// Slice i (0: most significant) of M, 7 bits.
-template <int NS>
-__device__ __forceinline__ unsigned slice_of(unsigned long long M, int i) {
-  return (unsigned)(M >> (kSliceBits * (NS - 1 - i))) & 0x7fu;
+// The eight 7-bit slices of a 56-bit magnitude M with a sign, one a byte: slices 0-3 (the most
+// significant) in the low word of the pair, slice i in byte 3 - i % 4, as 128 +- c.
+__device__ __forceinline__ uint32_t spread_28(uint32_t h) {
+  return h + (h & ~0x7fu) + ((h & ~0x3fffu) << 1) + ((h & ~0x1fffffu) << 2);
 }
-
-// Two f16 values (low half first) holding the integers c0, c1 in [0, 128) with the given
-// signs: 1024 + c is the f16 bit pattern 0x6400 | c, and subtracting 1024 is exact.
-__device__ __forceinline__ uint32_t half2_ints(unsigned c0, unsigned c1, uint32_t signs) {
-  const uint32_t w = (0x6400u | c0) | ((0x6400u | c1) << 16);
-  uint32_t r;
-  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0x64006400u));
-  return r ^ signs;
+constexpr uint32_t kZeroSlices = 0x80808080u;
+__device__ __forceinline__ uint2 slice_bytes(unsigned long long M, bool neg) {
+  const uint32_t a = spread_28((uint32_t)(M >> 28)), b = spread_28((uint32_t)M & 0xfffffffu);
+  return neg ? make_uint2(kZeroSlices - a, kZeroSlices - b)
+             : make_uint2(kZeroSlices + a, kZeroSlices + b);
 }
-// Slices i and i + 1 of one value as two f16 values (low half: slice i), negative when neg:
-// -(1024 + c) is 0xE400 | c, and subtracting -1024 leaves -c.
-__device__ __forceinline__ uint32_t half2_pair(unsigned c0, unsigned c1, bool neg) {
-  const uint32_t base = neg ? 0xE400E400u : 0x64006400u;
-  const uint32_t w = base | c0 | (c1 << 16);
+// Slice i of two values as two f16 (the low half: of x0): the f16 with bits 0x6400 | u is 1024 + u,
+// and subtracting 1152 leaves u - 128 = +- c exactly.
+template <int I>
+__device__ __forceinline__ uint32_t half2_slice(uint2 x0, uint2 x1) {
+  constexpr uint32_t j = 3 - (I & 3);
+  const uint32_t p = __byte_perm(I < 4 ? x0.x : x0.y, I < 4 ? x1.x : x1.y,
+                                 j | (j << 4) | ((4 + j) << 8) | ((4 + j) << 12));
+  const uint32_t w = (p & 0x00ff00ffu) | 0x64006400u;
   uint32_t r;
-  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(base));
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0x64806480u));
   return r;
-}
-
-__device__ __forceinline__ uint32_t sign_bits(double a, double b) {
-  return ((uint32_t)(__double2hiint(a) < 0) << 15) | ((uint32_t)(__double2hiint(b) < 0) << 31);
-}
-__device__ __forceinline__ uint32_t sign_bits(float a, float b) {
-  return ((__float_as_uint(a) >> 31) << 15) | ((__float_as_uint(b) >> 31) << 31);
 }
 
 // D += A B for one m16n8k16 tile: A row-major f16 (4 registers), B column-major f16 (2),
@@ -149,15 +133,6 @@ __device__ __forceinline__ void mma_f16_16816(float* d, const uint32_t* a, const
       "{%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// The four 8x8 f16 matrices of an m16n8k16 A operand from shared memory; p is this lane's row
-// address (rows (lane & 7) + 8 ((lane >> 3) & 1), columns 8 (lane >> 4) of the 16x16 tile).
-__device__ __forceinline__ void ldsm_x4(uint32_t* r, const void* p) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(a));
 }
 
 // FP64 value of one accumulator element: the diagonals d = 0..ND-1 (exact integers in FP32)
