@@ -143,15 +143,21 @@ __global__ void k_grad_v2c(const int* __restrict__ plist, int count, const int64
 }
 
 
-// A^H per patch: out_l = (V^T K z)_l over the rule q_j, plus conj(c) g over the patch's
-// near pairs and self pairs in patch-major order (deterministic, no atomics), plus
-// jump * g_t at the node of each on-surface target t.
+// A^H per patch: out_l = (V^T K z)_l over the rule q_j (z the sum of its parts), plus conj(c) g
+// over the patch's near pairs and self pairs in patch-major order (deterministic, no atomics),
+// plus jump * g_t at the node of each on-surface target t.  The basis values of 64 nodes at a
+// time go through shared memory: a thread per node forms them, a thread per basis function sums.
+constexpr int kAdjThreads = 64;
 template <int D>
-__global__ void k_adj_patch(const int* __restrict__ plist, int count, Dev dv,
-                            const double* __restrict__ Vt, const int64_t* __restrict__ src_off,
-                            const cplx* __restrict__ z, const double* __restrict__ val,
-                            const cplx* __restrict__ g, double jump, cplx* __restrict__ out) {
+__global__ void __launch_bounds__(kAdjThreads) k_adj_patch(
+    const int* __restrict__ plist, int count, Dev dv, const double* __restrict__ Vt,
+    const int64_t* __restrict__ src_off, const cplx* __restrict__ z, int parts, int64_t n_over,
+    const double* __restrict__ val, const cplx* __restrict__ g, double jump,
+    cplx* __restrict__ out) {
   constexpr int n = (D + 1) * (D + 2) / 2;
+  constexpr int NR = (n + kAdjThreads - 1) / kAdjThreads;  // basis functions per thread
+  __shared__ double Ks[kAdjThreads * (n + 1)];
+  __shared__ cplx zs[kAdjThreads];
   __shared__ cplx kz[n];
   for (int b = blockIdx.x; b < count; b += gridDim.x) {
     const int j = plist[b];
@@ -159,18 +165,39 @@ __global__ void k_adj_patch(const int* __restrict__ plist, int count, Dev dv,
     const int m = dv.q[j], Q = m * m;
     const double* ru = dv.ru + dv.roff[m];
     const double* rv = dv.rv + dv.roff[m];
-    __syncthreads();
-    // (K z)_nm: thread per basis function, nodes in order
-    for (int nm = threadIdx.x; nm < n; nm += blockDim.x) {
-      double re = 0.0, im = 0.0;
-      for (int q = 0; q < Q; ++q) {
-        double K[n];
-        kw_values<D>(ru[q], rv[q], K, 1);
-        const cplx zq = z[src_off[j] + q];
-        re = fma(K[nm], zq.re, re);
-        im = fma(K[nm], zq.im, im);
+    cplx acc[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) acc[r] = {0.0, 0.0};
+    for (int q0 = 0; q0 < Q; q0 += kAdjThreads) {
+      const int q = q0 + threadIdx.x;
+      __syncthreads();
+      if (q < Q) {
+        kw_values<D>(ru[q], rv[q], Ks + threadIdx.x * (n + 1), 1);
+        cplx s = {0.0, 0.0};
+        for (int k = 0; k < parts; ++k) {
+          const cplx zq = z[k * n_over + src_off[j] + q];
+          s.re += zq.re;
+          s.im += zq.im;
+        }
+        zs[threadIdx.x] = s;
       }
-      kz[nm] = {re, im};
+      __syncthreads();
+      const int cnt = min(kAdjThreads, Q - q0);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int nm = threadIdx.x + r * kAdjThreads;
+        if (nm < n)
+          for (int i = 0; i < cnt; ++i) {
+            const double kv = Ks[i * (n + 1) + nm];
+            acc[r].re = fma(kv, zs[i].re, acc[r].re);
+            acc[r].im = fma(kv, zs[i].im, acc[r].im);
+          }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int nm = threadIdx.x + r * kAdjThreads;
+      if (nm < n) kz[nm] = acc[r];
     }
     __syncthreads();
     for (int l = threadIdx.x; l < n; l += blockDim.x) {
@@ -200,6 +227,7 @@ __global__ void k_adj_patch(const int* __restrict__ plist, int count, Dev dv,
       }
       out[off + l] = {re, im};
     }
+    __syncthreads();
   }
 }
 
@@ -250,12 +278,12 @@ void GradV2cL<D>::run(const LaunchCommon& lc, const int* plist, int count, const
 
 template <int D>
 void AdjPatchL<D>::run(const LaunchCommon& lc, const int* plist, int count, const Dev& dv,
-                  const double* Vt, const int64_t* src_off, const void* z, const double* val,
-                  const void* g, double jump, void* out) {
+                  const double* Vt, const int64_t* src_off, const void* z, int parts,
+                  int64_t n_over, const double* val, const void* g, double jump, void* out) {
     ++*lc.launches;
-    k_adj_patch<D><<<grid_of(lc, count), 64, 0, lc.stream>>>(plist, count, dv, Vt, src_off,
-                                                             (const cplx*)z, val, (const cplx*)g,
-                                                             jump, (cplx*)out);
+    k_adj_patch<D><<<count, kAdjThreads, 0, lc.stream>>>(plist, count, dv, Vt, src_off,
+                                                         (const cplx*)z, parts, n_over, val,
+                                                         (const cplx*)g, jump, (cplx*)out);
   }
 
 }  // namespace lcq

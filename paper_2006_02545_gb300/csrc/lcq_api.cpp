@@ -1443,15 +1443,17 @@ lcq_status lcq_apply_corrected_Sp(lcq_ctx* ctx, const lcq_surface* surf, const l
 }
 
 // Oversampled far sources of every patch (positions, weighted normals, J w, interpolated
-// density if sigma is given) into a new buffer [9][n_over].
+// density if sigma is given; fx: in the form of the fixed-point kernel values) into a new
+// buffer [10][n_over].
 static lcq_status far_sources(lcq_ctx* ctx, const lcq_near* nr, lcq_corr* c, const Dev& dv,
-                              const LaunchCommon& lc, const double* sigma, double** src_out) {
+                              const LaunchCommon& lc, const double* sigma, bool fx,
+                              double** src_out) {
   double* src;
-  CK(dalloc(ctx->stream, &src, (size_t)9 * std::max<int64_t>(c->n_over, 1)));
+  CK(dalloc(ctx->stream, &src, (size_t)10 * std::max<int64_t>(c->n_over, 1)));
   for (int d = 1; d <= kMaxDeg; ++d) {
     if (!nr->plist_count[d]) continue;
     launch_far_src(d, lc, nr->plist_dev[d], nr->plist_count[d], dv, ctx->deg[d].dV, c->q,
-                   c->src_off, sigma, src, c->n_over, false);
+                   c->src_off, sigma, src, c->n_over, fx);
   }
   *src_out = src;
   return LCQ_OK;
@@ -1475,15 +1477,16 @@ lcq_status lcq_apply_adjoint(lcq_ctx* ctx, const lcq_surface* surf, const lcq_ne
     dfree(st, src);
     dfree(st, z);
   });
-  s = far_sources(ctx, nr, c, dv, lc, nullptr, &src);
+  s = far_sources(ctx, nr, c, dv, lc, nullptr, true, &src);
   if (s != LCQ_OK) return s;
-  CK(dalloc(st, &z, (size_t)2 * std::max<int64_t>(c->n_over, 1)));
+  const int parts = far_sum_T_parts(ctx->num_sms, nr->n_targets, c->n_over);
+  CK(dalloc(st, &z, (size_t)2 * parts * std::max<int64_t>(c->n_over, 1)));
   launch_far_sum_T(lc, dv, nr->n_patches, src, c->n_over, c->src_off, c->kp,
-                   c->grp ? nr->tgroup : nullptr, g, z);
+                   c->grp ? nr->tgroup : nullptr, g, z, parts);
   for (int d = 1; d <= kMaxDeg; ++d) {
     if (!nr->plist_count[d]) continue;
     launch_adj_patch(d, lc, nr->plist_dev[d], nr->plist_count[d], dv, ctx->deg[d].dV, c->src_off, z,
-                     c->val, g, jump, out);
+                     parts, c->n_over, c->val, g, jump, out);
   }
   CK(cudaGetLastError());
   return LCQ_OK;
@@ -1529,7 +1532,7 @@ lcq_status lcq_shape_gradient(lcq_ctx* ctx, const lcq_surface* surf, const lcq_n
     launch_shat(d, lc, nr->plist_dev[d], nr->plist_count[d], nr->node_off, ctx->deg[d].dV, sigma,
                 shat);
   }
-  s = far_sources(ctx, nr, c, dv, lc, nullptr, &src);
+  s = far_sources(ctx, nr, c, dv, lc, nullptr, false, &src);
   if (s != LCQ_OK) return s;
   // 1. far pairs through the rules q_j; 2. annulus pairs (both write M)
   launch_far_grad_sum(lc, dv, P, src, c->n_over, c->src_off, c->kp, c->grp ? nr->tgroup : nullptr,

@@ -895,6 +895,7 @@ __device__ void block_grad(const double* cf, const double* __restrict__ ru,
   double (*gx)[3] = reinterpret_cast<double (*)[3]>(scratch);
   cplx* gwt = reinterpret_cast<cplx*>(scratch + 3 * TG);
   const int total = nseg * Q;
+  const GradCoef co = grad_coef(kp);
   for (int c0 = 0; c0 < total; c0 += blockDim.x) {
     const int q = c0 + threadIdx.x;
     const bool on = q < total;
@@ -914,7 +915,10 @@ __device__ void block_grad(const double* cf, const double* __restrict__ ru,
         sg.im = fma(shat[idx].im, k0, sg.im);
       });
     }
-    cplx SX[3] = {{0, 0}, {0, 0}, {0, 0}}, SN[3] = {{0, 0}, {0, 0}, {0, 0}};
+    const double nN = sqrt(Nn[0] * Nn[0] + Nn[1] * Nn[1] + Nn[2] * Nn[2]);
+    const cplx bN = {co.be.re * nN, co.be.im * nN};
+    GradSum gs;
+    grad_clear(gs);
     for (int t0 = 0; t0 < T; t0 += TG) {
       const int nt = min(TG, T - t0);
       __syncthreads();
@@ -931,19 +935,12 @@ __device__ void block_grad(const double* cf, const double* __restrict__ ru,
         for (int i = 0; i < nt; ++i) {
           const cplx c = gwt[i];
           if (c.re == 0.0 && c.im == 0.0) continue;
-          cplx dX[3], dN[3];
-          kernel_grad(kp, gx[i], X, Nn, dX, dN);
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const cplx a = cmul(c, dX[k]), b = cmul(c, dN[k]);
-            SX[k].re += a.re;
-            SX[k].im += a.im;
-            SN[k].re += b.re;
-            SN[k].im += b.im;
-          }
+          grad_add(gs, kp, co, bN, gx[i], X, Nn, c);
         }
     }
     if (WARP_ACC || on) {
+      cplx SX[3], SN[3];
+      grad_finish(gs, co, Nn, nN, SX, SN);
       double aX[3], aN[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) {

@@ -100,7 +100,8 @@ struct GradV2cL {
 template <int D>
 struct AdjPatchL {
   static void run(const LaunchCommon& lc, const int* plist, int count, const Dev& dv,
-                  const double* Vt, const int64_t* src_off, const void* z, const double* val,
+                  const double* Vt, const int64_t* src_off, const void* z, int parts,
+                  int64_t n_over, const double* val,
                   const void* g, double jump, void* out);
 };
 

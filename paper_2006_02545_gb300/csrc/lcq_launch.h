@@ -193,9 +193,10 @@ bool launch_grad_v2c(int d, const LaunchCommon& lc, const int* plist, int count,
                      double* out);
 void launch_far_sum_T(const LaunchCommon& lc, const Dev& dv, int64_t P, const double* src,
                       int64_t n_over, const int64_t* src_off, const KernelParams& kp,
-                      const int32_t* tgroup, const void* g, void* z);
+                      const int32_t* tgroup, const void* g, void* z, int parts);
+int far_sum_T_parts(int num_sms, int64_t NT, int64_t n_over);
 bool launch_adj_patch(int d, const LaunchCommon& lc, const int* plist, int count, const Dev& dv,
-                      const double* Vt, const int64_t* src_off, const void* z, const double* val,
-                      const void* g, double jump, void* out);
+                      const double* Vt, const int64_t* src_off, const void* z, int parts,
+                      int64_t n_over, const double* val, const void* g, double jump, void* out);
 
 }  // namespace lcq
