@@ -807,8 +807,9 @@ static Dev make_dev(lcq_ctx* ctx, const lcq_near* nr, const int32_t* q, int ldI,
 }
 
 // Per-block workspace of the adaptive kernel (sized by the largest work item and the depth
-// cap) and its grid.
-static void adaptive_stride(lcq_ctx* ctx, const lcq_near* nr, int64_t A, int levels,
+// cap) and its grid: as many blocks as fit the device, no more than one degree's work items, and
+// within 64 GB of workspace.
+static void adaptive_stride(lcq_ctx* ctx, const lcq_near* nr, int64_t A, int levels, int64_t items,
                             int64_t* stride_out, int* grid_out) {
   const int64_t n = nr->n_max;
   int64_t stride = A * n * 16 + A * 4 * n * 16 + (int64_t)levels * A * 4 * n * 16 +
@@ -817,14 +818,16 @@ static void adaptive_stride(lcq_ctx* ctx, const lcq_near* nr, int64_t A, int lev
   int bps = 1;
   for (int d = 1; d <= kMaxDeg; ++d)
     if (nr->ad_count[d]) bps = std::max(bps, adaptive_blocks_per_sm(d));
-  *grid_out = ctx->num_sms * bps;
+  int64_t grid = std::min<int64_t>((int64_t)ctx->num_sms * bps, std::max<int64_t>(items, 1));
+  grid = std::min(grid, std::max<int64_t>(ctx->num_sms, (int64_t(64) << 30) / *stride_out));
+  *grid_out = (int)grid;
 }
 // The same in the context's workspace, grown when needed.
 static cudaError_t adaptive_work(lcq_ctx* ctx, const lcq_near* nr, int64_t A, int levels,
-                                 int64_t* stride_out, int* grid_out) {
+                                 int64_t items, int64_t* stride_out, int* grid_out) {
   int64_t stride = 0;
   int agrid = 0;
-  adaptive_stride(ctx, nr, A, levels, &stride, &agrid);
+  adaptive_stride(ctx, nr, A, levels, items, &stride, &agrid);
   const size_t need = (size_t)stride * agrid;
   if (ctx->work_bytes < need) {
     if (ctx->work) {
@@ -1001,6 +1004,7 @@ static lcq_status gen_scratch(lcq_ctx* ctx, const lcq_near* nr, lcq_kernel kerne
     for (int d = 1; d <= kMaxDeg; ++d)
       if (nr->ad_count[d]) bps = std::max(bps, adaptive_blocks_per_sm(d));
     const int64_t slots = (int64_t)ctx->num_sms * bps;
+    int64_t items = 1;  // of the degree with the most
     for (int d = 1; d <= kMaxDeg; ++d) {
       gs->tune_meas[d] = -1;
       if (!nr->ad_count[d]) continue;
@@ -1018,13 +1022,16 @@ static lcq_status gen_scratch(lcq_ctx* ctx, const lcq_near* nr, lcq_kernel kerne
       }
       gs->A_eff = std::max<int64_t>(gs->A_eff, gs->gsz[d]);
       ctx->last_group_size = std::max(ctx->last_group_size, gs->gsz[d]);
-      for (int64_t a : nr->ad_nad_h[d]) ctx->last_items += (a + gs->gsz[d] - 1) / gs->gsz[d];
+      int64_t it = 0;
+      for (int64_t a : nr->ad_nad_h[d]) it += (a + gs->gsz[d] - 1) / gs->gsz[d];
+      ctx->last_items += it;
+      items = std::max(items, it);
     }
     if (gs->own_work) {
-      adaptive_stride(ctx, nr, gs->A_eff, gs->levels, &gs->astride, &gs->agrid);
+      adaptive_stride(ctx, nr, gs->A_eff, gs->levels, items, &gs->astride, &gs->agrid);
       CK(cudaMallocAsync(&gs->work, (size_t)gs->astride * gs->agrid, st));
     } else {
-      CK(adaptive_work(ctx, nr, gs->A_eff, gs->levels, &gs->astride, &gs->agrid));
+      CK(adaptive_work(ctx, nr, gs->A_eff, gs->levels, items, &gs->astride, &gs->agrid));
       gs->work = ctx->work;
     }
     int maxc = 0;
@@ -1548,7 +1555,9 @@ lcq_status lcq_shape_gradient(lcq_ctx* ctx, const lcq_surface* surf, const lcq_n
     const int levels = pr.max_depth;
     int64_t stride;
     int agrid;
-    CK(adaptive_work(ctx, nr, nr->max_adaptive, levels, &stride, &agrid));
+    int64_t items = 1;
+    for (int d = 1; d <= kMaxDeg; ++d) items = std::max<int64_t>(items, nr->ad_count[d]);
+    CK(adaptive_work(ctx, nr, nr->max_adaptive, levels, items, &stride, &agrid));
     const int64_t npr = std::max<int64_t>(nr->n_pairs, 1);
     CK(dalloc(st, &Is, (size_t)2 * npr * ldI));
     CK(dalloc(st, &In, (size_t)2 * npr * ldI));

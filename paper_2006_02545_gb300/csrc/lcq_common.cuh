@@ -312,7 +312,8 @@ template <int V>
 struct IntC {
   static constexpr int value = V;
 };
-template <int D, int NS, int ND, int FMAX, class OR>
+// BST: row stride of Bs (values).
+template <int D, int NS, int ND, int FMAX, int BST = TcCfg<D>::BST, class OR>
 __device__ __forceinline__ void tc_tile(const uint2* Bs, const uint4* G, const int* rowE, int ct,
                                         int kbeg, int kend, int nt, int t0, int sg, bool first,
                                         OR orow) {
@@ -323,16 +324,17 @@ __device__ __forceinline__ void tc_tile(const uint2* Bs, const uint4* G, const i
   float acc[ND][4];
 #pragma unroll
   for (int d = 0; d < ND; ++d) acc[d][0] = acc[d][1] = acc[d][2] = acc[d][3] = 0.0f;
-  const uint4* gp = G + g * C::GST + 2 * c;
-  const uint2* bp = Bs + (nb < n ? nb : 0) * C::BST + 2 * c;
+  const uint4 z = make_uint4(kZeroSlices, kZeroSlices, kZeroSlices, kZeroSlices);
+  // rows and columns beyond the operands are zero
+  const bool ga = g < nt, gb = nb < n;
+  const uint4* gp = G + (ga ? g : 0) * C::GST + 2 * c;
+  const uint2* bp = Bs + (gb ? nb : 0) * BST + 2 * c;
 #pragma unroll 1
   for (int k0 = kbeg; k0 < kend; k0 += 16) {
-    uint4 b0 = *reinterpret_cast<const uint4*>(bp + k0);
-    uint4 b1 = *reinterpret_cast<const uint4*>(bp + k0 + 8);
-    if (nb >= n) b0 = b1 = make_uint4(kZeroSlices, kZeroSlices, kZeroSlices, kZeroSlices);
-    const uint4 z = make_uint4(kZeroSlices, kZeroSlices, kZeroSlices, kZeroSlices);
-    const uint4 v0 = g < nt ? gp[k0] : z, v1 = g < nt ? gp[k0 + 1] : z;
-    const uint4 v2 = g < nt ? gp[k0 + 8] : z, v3 = g < nt ? gp[k0 + 9] : z;
+    const uint4 b0 = gb ? *reinterpret_cast<const uint4*>(bp + k0) : z;
+    const uint4 b1 = gb ? *reinterpret_cast<const uint4*>(bp + k0 + 8) : z;
+    const uint4 v0 = ga ? gp[k0] : z, v1 = ga ? gp[k0 + 1] : z;
+    const uint4 v2 = ga ? gp[k0 + 8] : z, v3 = ga ? gp[k0 + 9] : z;
     uint32_t bf[NS][2];
     auto bslice = [&](auto I) {
       constexpr int i = decltype(I)::value;
@@ -435,6 +437,27 @@ __device__ __forceinline__ void block_moments_form(
   const int mr = (int)lrintf(sqrtf((float)Q));
   using RW = FxRow<D>;
   constexpr int kRowMax = C::G_BYTES / 8 / RW::size;
+  // targets of a tile; up to TT targets in all are loaded once, in the shadow of the first rows
+  auto load_targets = [&](int t0, int nt) {
+    if (threadIdx.x < nt) {
+      double xp[3];
+      ta.pos(t0 + threadIdx.x, xp);
+      bool fin = true;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        xp[c] -= cen[c];
+        fin = fin && isfinite(xp[c]);
+        if (fixed) txi[3 * threadIdx.x + c] = fx_fix(xp[c], S);
+        else tx[3 * threadIdx.x + c] = xp[c];
+      }
+      te[threadIdx.x] = fin ? -100000 : kFxBad + 1;
+      if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
+    }
+  };
+  if (T <= C::TT) {
+    __syncthreads();
+    load_targets(0, T);
+  }
   int sg_next = 0, l_next = 0;
   while (sg_next < nseg) {
     // plan the chunk (uniform across the block); thread 0 records it for indexed lookups.  A
@@ -526,8 +549,8 @@ __device__ __forceinline__ void block_moments_form(
       const u64* row = rows + (pc[5] + l / mr - pc[4]) * RW::size;
       fx_basis_point<D>(s, row, part, C::PARTS, [&](int idx, i64 kv) {
         const u64 sgn = (u64)(kv >> 63);
-        const u64 M = ((((u64)kv ^ sgn) - sgn) + 4) >> 3;  // 56 bits, rounded
-        Bs[idx * C::BST + col] = slice_bytes(M < (1ull << 56) ? M : (1ull << 56) - 1, kv < 0);
+        // 56 bits, rounded; below 2^56, since |K_nm| (1 + 1e-12) < 2^E_nm
+        Bs[idx * C::BST + col] = slice_bytes(((((u64)kv ^ sgn) - sgn) + 4) >> 3, kv < 0);
       });
       i64 X[3], N[3];
       fx_chart_point<D>(s, row, X, N);
@@ -571,20 +594,7 @@ __device__ __forceinline__ void block_moments_form(
     for (int t0 = 0; t0 < T; t0 += C::TT) {
       const int nt = min(C::TT, T - t0);
       for (int e = threadIdx.x; e < C::MAXP * C::TT * 2; e += blockDim.x) rowE[e] = 0;
-      if (threadIdx.x < nt) {
-        double xp[3];
-        ta.pos(t0 + threadIdx.x, xp);
-        bool fin = true;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          xp[c] -= cen[c];
-          fin = fin && isfinite(xp[c]);
-          if (fixed) txi[3 * threadIdx.x + c] = fx_fix(xp[c], S);
-          else tx[3 * threadIdx.x + c] = xp[c];
-        }
-        te[threadIdx.x] = fin ? -100000 : kFxBad + 1;
-        if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
-      }
+      if (T > C::TT) load_targets(t0, nt);
       __syncthreads();
       // (3) the column's kernel values; zeros in padding columns
       if (in) {  // whole half-warps: pieces are multiples of 16 columns
@@ -1250,22 +1260,37 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
                       },
                       kps, shat, dv.cen + 3 * j, Mg, ws);
       }
-      // stable compaction of the refining targets into level L+1
+      // stable compaction of the refining targets into level L+1; up to 32 of them by one warp's
+      // ballot (cnt[L + 1] carries the count through the barrier below)
       int base = 0;
       int* DT = lvlT + (int64_t)(L + 1) * A_max;
       cplx* DI = lvlI + (int64_t)(L + 1) * A_max * 4 * n;
-      for (int s0 = 0; s0 < S; s0 += blockDim.x) {
-        const int s = s0 + threadIdx.x;
-        const int f = s < S ? flags[s] : 0;
-        int tot;
-        const int pos = block_flag_scan(f, ism, &tot);
-        if (f) {
-          flags[s] = -(base + pos) - 1;  // remember destination
-          DT[base + pos] = ST[s];
+      if (S <= 32) {
+        if (threadIdx.x < 32) {
+          const int f = lane < S ? flags[lane] : 0;
+          const unsigned bal = __ballot_sync(0xffffffffu, f);
+          if (f) {
+            const int pos = __popc(bal & ((1u << lane) - 1u));
+            flags[lane] = -pos - 1;  // remember destination
+            DT[pos] = ST[lane];
+          }
+          if (lane == 0) ism[0] = __popc(bal);
         }
-        base += tot;
+      } else {
+        for (int s0 = 0; s0 < S; s0 += blockDim.x) {
+          const int s = s0 + threadIdx.x;
+          const int f = s < S ? flags[s] : 0;
+          int tot;
+          const int pos = block_flag_scan(f, ism, &tot);
+          if (f) {
+            flags[s] = -(base + pos) - 1;  // remember destination
+            DT[base + pos] = ST[s];
+          }
+          base += tot;
+        }
       }
       __syncthreads();
+      if (S <= 32) base = ism[0];
       for (int e = threadIdx.x; e < S * 4 * n; e += blockDim.x) {
         const int s = e / (4 * n);
         const int f = flags[s];

@@ -219,6 +219,16 @@ __device__ __forceinline__ i64 fx_next_L(FxS s, FxS L, FxS Q, FxS Lp) {
                (u64)((ta >> 28) - (tb >> 29)));
 }
 
+// X_u x X_v (2^61) of d = (X_u, X_v) (2^62).
+__device__ __forceinline__ void fx_cross(const FxS* d, i64* N) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const FxS a = d[(c + 1) % 3], b = d[3 + (c + 2) % 3], e = d[(c + 2) % 3], f = d[3 + (c + 1) % 3];
+    const i64 tt = fx_swide(a.h, b.l) + fx_swide(a.l, b.h) - fx_swide(e.h, f.l) - fx_swide(e.l, f.h);
+    N[c] = (i64)((u64)(fx_swide(a.h, b.h) - fx_swide(e.h, f.h)) << 1) + (tt >> 30);
+  }
+}
+
 // X (2^(59 - sx)), and the normal X_u x X_v (2^(61 - su - sv)) of the node at s = 2u + v - 1 of a row.
 template <int D>
 __device__ __forceinline__ void fx_chart_point(FxS s, const u64* row, i64* X, i64* N) {
@@ -245,17 +255,12 @@ __device__ __forceinline__ void fx_chart_point(FxS s, const u64* row, i64* X, i6
       }
     }
   }
-  FxS d[6];
 #pragma unroll
   for (int c = 0; c < 3; ++c) X[c] = h[c] + (t[c] >> 28);
+  FxS d[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) d[c] = fx_split((h[3 + c] << 3) + (t[3 + c] >> 25));
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const FxS a = d[(c + 1) % 3], b = d[3 + (c + 2) % 3], e = d[(c + 2) % 3], f = d[3 + (c + 1) % 3];
-    const i64 tt = fx_swide(a.h, b.l) + fx_swide(a.l, b.h) - fx_swide(e.h, f.l) - fx_swide(e.l, f.h);
-    N[c] = (i64)((u64)(fx_swide(a.h, b.h) - fx_swide(e.h, f.h)) << 1) + (tt >> 30);
-  }
+  fx_cross(d, N);
 }
 
 // Basis values of the node: emit(idx, K_nm 2^(59 - E_nm)) for the m of one part of `parts`.
@@ -306,6 +311,98 @@ __device__ __forceinline__ void fx_node_from_normal(const i64* N, int sn, double
   const int z = fx_clz(p) - 2;
   *wm = z >= 0 && p != 0 ? p << z : p;
   *ew = sn - sh + e + 2 - (p != 0 ? z : 0);
+}
+
+// The basis at a point that shares no row with others: emit(idx, K_nm 2^(62 - E_nm)), and the normal
+// X_u x X_v (2^(61 - su - sv)) from the chart's derivative series.  The recurrence in n runs on
+// K_nm itself, started at L_m.
+template <int D, class F>
+__device__ __forceinline__ void fx_basis_normal(double u, double v, const FxChart<D>& ch, i64* N,
+                                                F&& emit) {
+  constexpr int nd = FxChart<D>::nd;
+  const FxS s = fx_split(fx_fix(2.0 * u + v - 1.0, 0)), y = fx_split(fx_fix(1.0 - 2.0 * v, 0));
+  const double q2 = (1.0 - v) * (1.0 - v);
+  i64 h[6] = {0, 0, 0, 0, 0, 0}, t[6] = {0, 0, 0, 0, 0, 0};
+  FxS L = {1 << 29, 0}, Lp = {0, 0};
+#pragma unroll 1
+  for (int m = 0; m <= D; ++m) {
+    if (m == 1) {
+      Lp = L;
+      L = {s.h >> 1, (int)(((uint32_t)(s.h & 1) << 30) | ((uint32_t)s.l >> 1))};
+    } else if (m > 1) {
+      const FxS Ln = fx_split(fx_next_L(s, L, fx_split(fx_fix(c_fxq[m] * q2, 0)), Lp));
+      Lp = L;
+      L = Ln;
+    }
+    const i64* g = c_fxj + m * (kMaxDeg + 1) * 3;
+    i64 K = fx_smul_sl<3>(L, fx_split(c_fxj0[m])), Kp = 0;
+#pragma unroll 1
+    for (int a = 0; a <= D - m; ++a) {
+      const int nn = m + a, idx = nn * (nn + 1) / 2 + m;
+      emit(idx, K);
+      if (nn < D) {
+        const FxS Ks = fx_split(K), K8 = fx_28(Ks);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          fx_mac28(h[c], t[c], K8, fx_unjoin(ch.d[idx * 3 + c]));
+          fx_mac28(h[3 + c], t[3 + c], K8, fx_unjoin(ch.d[(nd + idx) * 3 + c]));
+        }
+        const FxS f = fx_split((fx_smul(fx_split(g[3 * a]), y) << 2) + g[3 * a + 1]);
+        const FxS g2 = fx_split(g[3 * a + 2]), Kq = fx_split(Kp);
+        const i64 tt = fx_swide(f.h, Ks.l) + fx_swide(f.l, Ks.h) - fx_swide(g2.h, Kq.l) -
+                       fx_swide(g2.l, Kq.h);
+        Kp = K;
+        K = (i64)((u64)(fx_swide(f.h, Ks.h) - fx_swide(g2.h, Kq.h)) << 4) + (tt >> 27);
+      }
+    }
+  }
+  FxS d[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) d[c] = fx_split((h[c] << 2) + (t[c] >> 26));
+  fx_cross(d, N);
+}
+
+// The chord of chart_taylor's coefficients tX 2^(62 - st) (28 bits of the low word; st above the
+// sum of their magnitudes) at (du, dv) = (da, db) 2^e: dX = du A + dv B with A and B polynomials,
+// so that the chord keeps its relative precision as the point approaches the node.
+// dX = out 2^(e + st - 61).
+template <int D>
+__device__ __forceinline__ void fx_chord(const u64* tX, double du, double dv, i64* out, int* eout) {
+  constexpr int n = (D + 1) * (D + 2) / 2;
+  const FxS u = fx_split(fx_fix(du, 0)), v = fx_split(fx_fix(dv, 0));
+  i64 h[6] = {0, 0, 0, 0, 0, 0}, t[6] = {0, 0, 0, 0, 0, 0};  // A, then B
+  FxS pj = {1 << 30, 0};  // dv^j
+#pragma unroll
+  for (int j = 0; j <= D; ++j) {
+    FxS q = pj;           // du^(i-1) dv^j
+#pragma unroll
+    for (int i = 1; i <= D - j; ++i) {
+      const int gg = i + j, e = gg * (gg + 1) / 2 + j;
+      const FxS q8 = fx_28(q);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) fx_mac28(h[c], t[c], q8, fx_unjoin(tX[c * n + e]));
+      if (i < D - j) q = fx_split(fx_smul_sl<2>(q, u));
+    }
+    if (j < D) {
+      const int gg = j + 1, e = gg * (gg + 1) / 2 + gg;
+      const FxS q8 = fx_28(pj);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) fx_mac28(h[3 + c], t[3 + c], q8, fx_unjoin(tX[c * n + e]));
+      pj = fx_split(fx_smul_sl<2>(pj, v));
+    }
+  }
+  int e0, e1;
+  fx_mant(du, &e0);
+  fx_mant(dv, &e1);
+  const int e = max(max(e0, e1), -1000);
+  const FxS a = fx_split(fx_fix(du, e)), b = fx_split(fx_fix(dv, e));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const FxS A = fx_split((h[c] << 2) + (t[c] >> 26)), B = fx_split((h[3 + c] << 2) + (t[3 + c] >> 26));
+    const i64 tt = fx_swide(a.h, A.l) + fx_swide(a.l, A.h) + fx_swide(b.h, B.l) + fx_swide(b.l, B.h);
+    out[c] = ((fx_swide(a.h, A.h) + fx_swide(b.h, B.h)) << 1) + (tt >> 30);
+  }
+  *eout = e;
 }
 
 }  // namespace lcq

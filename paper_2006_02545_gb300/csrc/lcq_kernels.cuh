@@ -383,25 +383,69 @@ struct SelfSeg {
 };
 
 // Block per self target: the self rule above applied to the chart, contracted with the
-// basis into the target's self weights (Sec. 4).
+// basis into the target's self weights (Sec. 4).  About 2000 nodes a target at eps = 1e-9, none
+// sharing a row with another: in FP64 a node took 430 instructions of 64 cycles (basis 130, tangents
+// 126, chord 105, parameters 50) and 64 more in the contraction.  Here the rule's radial and angular
+// factors are formed once per (panel, angle) instead of per node, basis, tangents and chord are
+// fixed-point (lcq_fxgeom.cuh), and the contraction runs on the tensor cores (tc_tile with one
+// target: the chunk's 128 kernel values are one row).
+constexpr int kSelfThreads = 128;
+constexpr int kSelfTab = 384;  // (panel, angle) entries kept; longer rules form them per node
 template <int D>
-__global__ void __launch_bounds__(128) k_self(Dev dv, const int32_t* __restrict__ deg_of_patch,
+struct SelfCfg {
+  static constexpr int n = (D + 1) * (D + 2) / 2;
+  static constexpr int BST = kSelfThreads + 8;
+  static constexpr size_t taylor = ((D + 1) * n + 2 * n * n) * sizeof(double);
+  static constexpr size_t basis = (size_t)n * BST * 8;
+  static constexpr size_t OFF_G = ((taylor > basis ? taylor : basis) + 15) / 16 * 16;
+  static constexpr size_t OFF_TAB = OFF_G + kSelfThreads * 16;
+  static constexpr size_t BYTES = OFF_TAB + kSelfTab * 3 * sizeof(double);
+};
+// The direction and weight of angle entry e = (segment, panel, angle): (du, dv) = s (out[0],
+// out[1]) and node weight w_s s out[2] for the radial node s.
+__device__ __forceinline__ void self_entry(const SelfSeg* sg, int nseg, int ns, int nt,
+                                           const double* __restrict__ glx, const double* __restrict__ glw,
+                                           const double* Mm, int e, double* out) {
+  int k = 0;
+  while (k + 1 < nseg && e * ns >= sg[k + 1].off) ++k;
+  const SelfSeg& g = sg[k];
+  const int loc = e - g.off / ns;
+  const int p = loc / nt, ti = loc - p * nt;
+  const double lo = g.xi_max * p / g.npan, hi = g.xi_max * (p + 1) / g.npan;
+  const double xi = lo + (hi - lo) * glx[ti];
+  // sinh and cosh from one exponential (xi >= 0: the difference loses at most a few
+  // 1e-16 absolute near xi = 0, which moves the node by mu times that)
+  const double ex = exp(xi), exi = 1.0 / ex;
+  const double tpar = g.t0 + g.side * g.mu * (0.5 * (ex - exi));
+  const double zx = g.E0x + tpar * g.Dx, zy = g.E0y + tpar * g.Dy;
+  out[0] = Mm[0] * zx + Mm[1] * zy;
+  out[1] = Mm[2] * zx + Mm[3] * zy;
+  out[2] = glw[ti] * (hi - lo) * g.mu * (0.5 * (ex + exi)) * g.area2 * Mm[4];
+}
+
+template <int D>
+__global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t* __restrict__ deg_of_patch,
                                               const KernelParams kp, int order,
                                               cplx* __restrict__ out_self) {
-  constexpr int n = (D + 1) * (D + 2) / 2;
+  using SC = SelfCfg<D>;
+  constexpr int n = SC::n;
   __shared__ double cf[3 * n];
   __shared__ SelfSeg sg[6];
   __shared__ double Mm[5];  // M00 M01 M10 M11 detM
   __shared__ double P[2];
   __shared__ int nseg, total;
-  __shared__ cplx red[4][n];
   __shared__ KernelParams kps;
   __shared__ int ord;
   __shared__ double nP[3];  // unit chart normal at the target node (S')
-  __shared__ double cfd[2 * 3 * (D * (D + 1) / 2)];  // derivative series of the chart
-  __shared__ cplx gbuf[128];                          // kernel values of a chunk's nodes
-  __shared__ double tX[3 * n];                        // Taylor coefficients of the chord at P
-  extern __shared__ double krows[];                   // [128][n + 1] basis rows of a chunk
+  __shared__ FxChart<D> ch;
+  __shared__ double tX[3 * n];  // Taylor coefficients of the chord at P, then in fixed point
+  __shared__ int st;
+  __shared__ int rowE[2];
+  __shared__ cplx acc[n];
+  extern __shared__ __align__(16) unsigned char ssm[];
+  uint2* Bs = reinterpret_cast<uint2*>(ssm);
+  uint4* G = reinterpret_cast<uint4*>(ssm + SC::OFF_G);
+  double* tabl = reinterpret_cast<double*>(ssm + SC::OFF_TAB);
   long long my_nodes = 0;
   for (int64_t s = blockIdx.x; s < dv.n_self; s += gridDim.x) {
     const int t = dv.self_tgt[s];
@@ -414,13 +458,10 @@ __global__ void __launch_bounds__(128) k_self(Dev dv, const int32_t* __restrict_
       kps = patch_kp(dv, j, kp);
       ord = dv.pgroup ? dv.grp[dv.pgroup[j]].self_order : order;
     }
-    __syncthreads();
-    load_coef_derivs<D>(cf, dv.duv[D], cfd);
+    load_fx_chart<D>(cf, dv.duv[D], &ch);
     const int ns = ord, nt = ord;
-    const double* glx_s = dv.gl_x + dv.gl_off[ns];
-    const double* glw_s = dv.gl_w + dv.gl_off[ns];
-    const double* glx_t = dv.gl_x + dv.gl_off[nt];
-    const double* glw_t = dv.gl_w + dv.gl_off[nt];
+    const double* glx = dv.gl_x + dv.gl_off[ord];
+    const double* glw = dv.gl_w + dv.gl_off[ord];
     if (threadIdx.x == 0) {
       const double pu = dv.nodes_uv[D][i], pv = dv.nodes_uv[D][n + i];
       P[0] = pu;
@@ -484,87 +525,84 @@ __global__ void __launch_bounds__(128) k_self(Dev dv, const int32_t* __restrict_
     const FxTables tab = fx_tables();
     FxS nPx[3];  // S': the source's normal replaced by -n_x
     for (int c = 0; c < 3; ++c) nPx[c] = fx_split(fx_fix(-nP[c], 0));
-    chart_taylor<D>(P[0], P[1], cf, krows, tX);  // krows is free until the first chunk
-    // the target is the chart's value at the node: x - X(P + delta) = -(dX)
-    // chunks of 128 nodes: each thread forms one node's kernel value and basis row in
-    // shared memory, then the block contracts them, thread (nm, quarter of the chunk)
+    const int nent = total / ns;
+    for (int e = threadIdx.x; e < nent && e < kSelfTab; e += blockDim.x)
+      self_entry(sg, nseg, ns, nt, glx, glw, Mm, e, tabl + 3 * e);
+    // the basis area is free until the first chunk
+    chart_taylor<D>(P[0], P[1], cf, reinterpret_cast<double*>(ssm), tX);
+    if (threadIdx.x == 0) {
+      double mx = 0.0;
+      for (int c = 0; c < 3; ++c) {
+        double a = 0.0;
+        for (int e = 1; e < n; ++e) a += fabs(tX[c * n + e]);
+        mx = fmax(mx, a);
+      }
+      fx_mant(mx, &st);
+      st = max(st, -1000);
+    }
+    __syncthreads();
+    u64* tXf = reinterpret_cast<u64*>(tX);
+    for (int e = threadIdx.x; e < 3 * n; e += blockDim.x) tXf[e] = fx_join28(fx_fix(tX[e], st));
+    for (int e = threadIdx.x; e < n; e += blockDim.x) acc[e] = {0.0, 0.0};
     const int tot = total;
-    constexpr int NR = (n + 31) / 32;  // basis indices per thread in the contraction
-    const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
-    double are[NR], aim[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) are[r] = aim[r] = 0.0;
-    for (int c0 = 0; c0 < tot; c0 += 128) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int c0 = 0; c0 < tot; c0 += kSelfThreads) {
+      if (threadIdx.x < 2) rowE[threadIdx.x] = 0;
+      __syncthreads();
       const int idx = c0 + threadIdx.x;
       cplx gk = {0.0, 0.0};
-      double* Kq = krows + threadIdx.x * (n + 1);
       if (idx < tot) {
-        int k = 0;
-        while (k + 1 < nseg && idx >= sg[k + 1].off) ++k;
-        const SelfSeg& g = sg[k];
-        const int loc = idx - g.off;
-        const int p = loc / (nt * ns);
-        const int rem = loc - p * nt * ns;
-        const int ti = rem / ns, si = rem - ti * ns;
-        const double lo = g.xi_max * p / g.npan, hi = g.xi_max * (p + 1) / g.npan;
-        const double xi = lo + (hi - lo) * glx_t[ti];
-        // sinh and cosh from one exponential (xi >= 0: the difference loses at most a few
-        // 1e-16 absolute near xi = 0, which moves the node by mu times that)
-        const double ex = exp(xi), exi = 1.0 / ex;
-        const double tpar = g.t0 + g.side * g.mu * (0.5 * (ex - exi));
-        const double wt = glw_t[ti] * (hi - lo) * g.mu * (0.5 * (ex + exi));
-        const double sv = glx_s[si];
-        const double w = glw_s[si] * wt * sv * g.area2 * Mm[4];
-        const double zx = sv * (g.E0x + tpar * g.Dx), zy = sv * (g.E0y + tpar * g.Dy);
-        const double du = Mm[0] * zx + Mm[1] * zy;
-        const double dvv = Mm[2] * zx + Mm[3] * zy;
-        double dX[3], Xu[3], Xv[3], Nn[3];
-        kw_geometry_proj<D, false>(P[0] + du, P[1] + dvv, cf, cfd, nullptr, Xu, Xv, Kq);
-        chart_chord<D>(tX, du, dvv, dX);
-        cross3(Xu, Xv, Nn);
+        const int e = idx / ns, si = idx - e * ns;
+        double direct[3];
+        const double* en = tabl + 3 * e;
+        if (e >= kSelfTab) {
+          self_entry(sg, nseg, ns, nt, glx, glw, Mm, e, direct);
+          en = direct;
+        }
+        const double sv = glx[si], du = sv * en[0], dvv = sv * en[1];
+        const double w = glw[si] * sv * en[2];
+        i64 N[3], d[3];
+        fx_basis_normal<D>(P[0] + du, P[1] + dvv, ch, N, [&](int k, i64 kv) {
+          const u64 sgn = (u64)(kv >> 63);
+          Bs[k * SC::BST + threadIdx.x] = slice_bytes(((((u64)kv ^ sgn) - sgn) + 32) >> 6, kv < 0);
+        });
+        int ed;
+        fx_chord<D>(tXf, du, dvv, d, &ed);
         FxS nn[3];
         u64 wm;
         int ew;
-        fx_make_node(Nn, w, nn, &wm, &ew);
-        const FxS* nu = kps.kind == 3 ? nPx : nn;
-        if (!fx_eval<false>(kps.fx, tab, -dX[0], -dX[1], -dX[2], nu, wm, ew, &gk.re, &gk.im, nullptr,
-                            0.0f, 0.0f, 0.0f, 0.0f, 0.0f))
-          gk = fx_fallback(kps, -dX[0], -dX[1], -dX[2], nu[0], nu[1], nu[2], wm, ew, 0.0, nullptr);
+        fx_node_from_normal(N, ch.su + ch.sv + 1, w, nn, &wm, &ew);
+        if (ch.bad) ew = kFxBad + 1;
+        // the target is the chart's value at the node: x - X(P + delta) = -dX
+        const int S = ed + st + 1;
+        const FxS nu[3] = {kps.kind == 3 ? nPx[0] : nn[0], kps.kind == 3 ? nPx[1] : nn[1],
+                           kps.kind == 3 ? nPx[2] : nn[2]};
+        if (!fx_eval_int<false>(kps.fx, tab, -d[0], -d[1], -d[2], S, nu, wm, ew, &gk.re, &gk.im,
+                                nullptr, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f))
+          gk = fx_fallback(kps, fx_pack<false>(-d[0], S - 62), fx_pack<false>(-d[1], S - 62),
+                           fx_pack<false>(-d[2], S - 62), nu[0], nu[1], nu[2], wm, ew, 0.0, nullptr);
       } else {
-        for (int e = 0; e < n; ++e) Kq[e] = 0.0;
+        for (int k = 0; k < n; ++k) Bs[k * SC::BST + threadIdx.x] = make_uint2(kZeroSlices, kZeroSlices);
       }
-      gbuf[threadIdx.x] = gk;
+      const int fr = __reduce_max_sync(0xffffffffu, exp_field(gk.re));
+      const int fi = __reduce_max_sync(0xffffffffu, exp_field(gk.im));
+      if (lane == 0) {
+        atomicMax(rowE, fr);
+        atomicMax(rowE + 1, fi);
+      }
       __syncthreads();
-      const int qa = part * 32, qb = min(qa + 32, tot - c0);
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const int nm = lane + 32 * r;
-        if (nm < n)
-          for (int q = qa; q < qb; ++q) {
-            const cplx gq = gbuf[q];
-            const double kv = krows[q * (n + 1) + nm];
-            are[r] = fma(gq.re, kv, are[r]);
-            aim[r] = fma(gq.im, kv, aim[r]);
-          }
-      }
+      const uint2 a = row_slices(gk.re, exp_bound(rowE[0], 0.0));
+      const uint2 b = row_slices(gk.im, exp_bound(rowE[1], 0.0));
+      G[threadIdx.x] = make_uint4(a.x, a.y, b.x, b.y);
+      __syncthreads();
+      const int kend = (min(kSelfThreads, tot - c0) + 15) & ~15;
+      for (int ct = warp; ct < TcCfg<D>::NTILE; ct += kSelfThreads / 32)
+        tc_tile<D, 8, 9, 0x7ff, SC::BST>(Bs, G, rowE, ct, 0, kend, 1, 0, 0, false,
+                                         [&](int) { return acc; });
       __syncthreads();
     }
     my_nodes += tot;
-    // the four quarters, in a fixed order
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const int nm = lane + 32 * r;
-      if (nm < n) red[part][nm] = {are[r], aim[r]};
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      cplx sum = red[0][k];
-      for (int q = 1; q < 4; ++q) {
-        sum.re += red[q][k].re;
-        sum.im += red[q][k].im;
-      }
-      out_self[s * dv.ldI + k] = sum;
-    }
+    for (int k = threadIdx.x; k < n; k += blockDim.x) out_self[s * dv.ldI + k] = acc[k];
   }
   if (threadIdx.x == 0)
     atomicAdd(reinterpret_cast<unsigned long long*>(dv.counters + 2), (unsigned long long)my_nodes);
@@ -802,11 +840,8 @@ void SelfL<D>::run(const LaunchCommon& lc, const Dev& dv, const int32_t* deg, co
     const int64_t g = dv.n_self < (int64_t)0x7fffffff ? dv.n_self : (int64_t)0x7fffffff;
     if (g <= 0) return;
     ++*lc.launches;
-    constexpr size_t n = (D + 1) * (D + 2) / 2;
-    constexpr size_t rows = 128 * (n + 1), taylor = (D + 1) * n + 2 * n * n;
-    const size_t sm = (rows > taylor ? rows : taylor) * sizeof(double);
-    set_smem(k_self<D>, sm);
-    k_self<D><<<(int)g, 128, sm, lc.stream>>>(dv, deg, kp, order, (cplx*)out);
+    set_smem(k_self<D>, SelfCfg<D>::BYTES);
+    k_self<D><<<(int)g, kSelfThreads, SelfCfg<D>::BYTES, lc.stream>>>(dv, deg, kp, order, (cplx*)out);
   }
 
 template <int D>
