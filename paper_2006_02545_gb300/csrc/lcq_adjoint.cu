@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(kThreads) k_far_grad_sum(
 // q's patch (the far sum of apply includes near pairs; their smooth-rule term is part of A).
 // As k_far_sum with the roles exchanged: a thread per source (its node in registers) and part of
 // the targets, fixed-point kernel values; z[part][n_over], which k_adj_patch adds in order.
-// 34,839 sources x 14,000 targets, CFIE: 72.6 ms with FP64 values and CUDA's sincos in one part.
+// 34,839 sources x 14,000 targets, CFIE: 72.6 ms with FP64 values and CUDA's sincos in
+// one part, 14 ms so.
 __global__ void __launch_bounds__(kSumTThreads) k_far_sum_T(
     Dev dv, int64_t P, const double* __restrict__ src, int64_t n_over,
     const int64_t* __restrict__ src_off, const KernelParams kp, const int32_t* __restrict__ tgroup,

@@ -401,7 +401,7 @@ __device__ __forceinline__ void tc_tile(const uint2* Bs, const uint4* G, const i
 // mma.sync on fragments built from the slice bytes.  Storing an operand as 8 bytes (not as 8
 // f16) lets a chunk hold 256 columns where it held 128, so that every thread has a node and the
 // barriers come half as often; they, not the pipes, bounded the kernel (1280-patch CFIE, eps
-// 1e-9: issue slots 32% busy before).
+// 1e-9: adaptive walk 295 ms at 32% of the issue slots before, 180 ms at 47% since).
 // S: exponent of the fixed-point positions (block_scale).  form: 0 FP64 (fixed point); 1 FP32
 // kernel values (the mixed form for eps >= kMixedMinEps); 2 two-float ones (kernel_eval_ff; the
 // mixed form below that) where the constants fold, else FP64.
@@ -468,7 +468,7 @@ __device__ __forceinline__ void block_moments_form(
     int np = 0, ncp = 0, nrow = 0, gcp = 0, g0 = 0;
     __syncthreads();
     while (sg_next < nseg && np < C::MAXP && ncp < C::CH) {
-      int nq = Q - l_next;
+      int nq = min(Q - l_next, 128);  // the slice sums of 128 nodes are exact in FP32
       const int room = C::CH - ncp;
       if (mixed) {
         const int nparts = (Q + C::CHG - 1) / C::CHG;
@@ -745,7 +745,9 @@ __device__ void block_moments_tc(const FxChart<D>& ch, int S, const double* __re
 // The moments of the smallest degrees in the FP64 form (n <= 10 basis functions) by the
 // plain FP64 engine (16-target tiles, one thread per output): there the contraction is too
 // small to pay for the tensor-core pipeline's fixed cost per 8-target tile (barriers, the
-// slice split).  Every other case: block_moments_tc.  smb holds either engine's workspace.
+// slices).  2400 patches, S, generation with this engine and with the tensor one: degree 1 eps
+// 5e-3 12.6 and 17.9 ms, degree 2 eps 5e-7 43.3 and 46.4, degree 3 eps 5e-3 22.6 and 26.8, eps 5e-7
+// 77.7 and 76.1 (the smooth rules alone: 5.8 and 14.6).  Every other case: block_moments_tc.  smb holds either engine's workspace.
 constexpr int kFp64MomentsMaxDeg = 3;
 template <int D, class TA, class OR>
 __device__ __forceinline__ void block_moments_any(

@@ -249,9 +249,8 @@ __device__ __forceinline__ void kw_geometry(double u, double v, const double* __
 // cfd = (X_u coefficients [nd][3], X_v coefficients [nd][3]) in the degree D-1 basis
 // (nd its size: the first nd basis functions, those with n < D).  Only the values
 // recurrence runs; K (stride 1, written first and read back) receives the basis values.
-// Same polynomials as kw_geometry at about half its cost.  WITH_X = false: X is not
-// formed (nor written).
-template <int D, bool WITH_X = true>
+// Same polynomials as kw_geometry at about half its cost.
+template <int D>
 __device__ __forceinline__ void kw_geometry_proj(double u, double v, const double* cf,
                                                  const double* cfd, double* X, double* Xu,
                                                  double* Xv, double* K) {
@@ -263,11 +262,9 @@ __device__ __forceinline__ void kw_geometry_proj(double u, double v, const doubl
 #pragma unroll 1
   for (int idx = 0; idx < nd; ++idx) {
     const double k = K[idx];
-    if (WITH_X) {
-      x0 = fma(cf[idx * 3], k, x0);
-      x1 = fma(cf[idx * 3 + 1], k, x1);
-      x2 = fma(cf[idx * 3 + 2], k, x2);
-    }
+    x0 = fma(cf[idx * 3], k, x0);
+    x1 = fma(cf[idx * 3 + 1], k, x1);
+    x2 = fma(cf[idx * 3 + 2], k, x2);
     u0 = fma(cfd[idx * 3], k, u0);
     u1 = fma(cfd[idx * 3 + 1], k, u1);
     u2 = fma(cfd[idx * 3 + 2], k, u2);
@@ -275,18 +272,16 @@ __device__ __forceinline__ void kw_geometry_proj(double u, double v, const doubl
     v1 = fma(cfd[(nd + idx) * 3 + 1], k, v1);
     v2 = fma(cfd[(nd + idx) * 3 + 2], k, v2);
   }
-  if (WITH_X) {
 #pragma unroll 1
-    for (int idx = nd; idx < n; ++idx) {
-      const double k = K[idx];
-      x0 = fma(cf[idx * 3], k, x0);
-      x1 = fma(cf[idx * 3 + 1], k, x1);
-      x2 = fma(cf[idx * 3 + 2], k, x2);
-    }
-    X[0] = x0;
-    X[1] = x1;
-    X[2] = x2;
+  for (int idx = nd; idx < n; ++idx) {
+    const double k = K[idx];
+    x0 = fma(cf[idx * 3], k, x0);
+    x1 = fma(cf[idx * 3 + 1], k, x1);
+    x2 = fma(cf[idx * 3 + 2], k, x2);
   }
+  X[0] = x0;
+  X[1] = x1;
+  X[2] = x2;
   Xu[0] = u0;
   Xu[1] = u1;
   Xu[2] = u2;
@@ -361,11 +356,10 @@ __device__ __forceinline__ void kw_row_factors(double v, int m, const double* cf
   }
 }
 
-// X, X_u, X_v at (u, v) from the row factors of v; each basis value K_nm is handed to
-// emit(idx, K_nm) as it is formed (idx = n(n+1)/2 + m).
-template <int D, class F>
-__device__ __forceinline__ void kw_geometry_row_emit(double u, const double* row, double* X,
-                                                     double* Xu, double* Xv, F&& emit) {
+// X, X_u, X_v and the basis values K (stride 1) at (u, v) from the row factors of v.
+template <int D>
+__device__ __forceinline__ void kw_geometry_row(double u, const double* row, double* X,
+                                                double* Xu, double* Xv, double* K) {
   using RW = KwRow<D>;
   const double v = row[0];
   const double s = 2.0 * u + v - 1.0;
@@ -394,7 +388,7 @@ __device__ __forceinline__ void kw_geometry_row_emit(double u, const double* row
 #pragma unroll
     for (int a = 0; a <= D - m; ++a) {
       const int nn = m + a, idx = nn * (nn + 1) / 2 + m;
-      emit(idx, L * row[RW::J + idx]);
+      K[idx] = L * row[RW::J + idx];
     }
   }
   X[0] = x0;
@@ -406,13 +400,6 @@ __device__ __forceinline__ void kw_geometry_row_emit(double u, const double* row
   Xv[0] = v0;
   Xv[1] = v1;
   Xv[2] = v2;
-}
-
-// X, X_u, X_v and the basis values K (stride 1) at (u, v) from the row factors of v.
-template <int D>
-__device__ __forceinline__ void kw_geometry_row(double u, const double* row, double* X,
-                                                double* Xu, double* Xv, double* K) {
-  kw_geometry_row_emit<D>(u, row, X, Xu, Xv, [&](int idx, double k) { K[idx] = k; });
 }
 
 // cfd for kw_geometry_proj from cf and the projections duv (Du [n][nd], then Dv), by
@@ -528,28 +515,6 @@ __device__ void chart_taylor(double pu, double pv, const double* cf, double* scr
     tX[o] = acc;
   }
   __syncthreads();
-}
-
-// The chord dX(d) from the coefficients of chart_taylor: Horner in du inside Horner in dv.
-template <int D>
-__device__ __forceinline__ void chart_chord(const double* tX, double du, double dv, double* dX) {
-  constexpr int n = (D + 1) * (D + 2) / 2;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const double* t = tX + c * n;
-    double acc = 0.0;
-#pragma unroll
-    for (int j = D; j >= 0; --j) {
-      double in = 0.0;
-#pragma unroll
-      for (int i = D - j; i >= 0; --i) {
-        const int g = i + j;
-        in = fma(in, du, t[g * (g + 1) / 2 + j]);
-      }
-      acc = fma(acc, dv, in);
-    }
-    dX[c] = acc;
-  }
 }
 
 // f(idx, K_nm, dK_nm/du, dK_nm/dv) for every basis function at (u, v): the recurrences of

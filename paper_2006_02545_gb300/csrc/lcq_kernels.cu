@@ -1,4 +1,5 @@
-// CUDA kernels of the correction path (sm_103a).  FP64 throughout.
+// CUDA kernels of the correction path (sm_103a), FP64 precision throughout (kernel values in
+// 64-bit fixed point).
 //
 //   k_geom         chart coefficients, centroid, radius, d_j        (Sec. 3.2, Sec. 4)
 //   (near lists: lcq_nearlist.cu)
@@ -75,7 +76,7 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
 // The kernel values are fixed-point (fx_eval): of FP64 there are only the difference x - X and
 // the four multiply-adds of the density (448 cycles of the FP64 pipe a pair and warp, beside
 // about 440 integer instructions for the single layer).  35,840 targets x 127,606 sources, CFIE:
-// 407 ms with FP64 kernel values (41 FP64 instructions a pair), 129 ms so; 8,960 x 25,920, S: 15.7
+// 407 ms with FP64 kernel values (41 FP64 instructions a pair), 126 ms so; 8,960 x 25,920, S: 15.7
 // and 4.4 ms.  More warps per SM (128, 96, 80, 64 registers) and two sources a step: within 3%.
 // The sources of an on-surface target's own patch are skipped (their contribution is
 // carried entirely by the self correction).  In a batch of independent surfaces a target

@@ -1,20 +1,21 @@
-// Building blocks of the split-precision tensor-core contraction and the lean FP64 kernel
-// evaluation used by the adaptive near integration (Sec. 4.3).
+// Building blocks of the split-precision tensor-core contraction, of the two-float kernel values
+// and of the lean FP64 gradients used by the adaptive near integration (Sec. 4.3).
 //
 // On GB300 the FP64 pipe retires 2 FMA per clock per SM (measured 1.26 TFLOP/s), the FP32
 // pipe 128 and the warp-level f16 tensor-core MMA about 0.47 m16n8k16 per clock per SM
 // (measured 602 TFLOP/s).  The dense part of the adaptive integration, the contraction of
 // kernel values (targets x leaf nodes) with basis values (leaf nodes x n), is therefore
-// done exactly on the tensor cores: each FP64 operand is written as a sum of NS slices of
+// done exactly on the tensor cores: each operand is written as a sum of NS slices of
 // 7 bits on a common power-of-two scale (the row's for the kernel values, a fixed per-column
 // bound for the basis values; the Ozaki splitting of Ozaki, Ogita, Oishi and Rump,
 // Numer. Algorithms 59, 2012), every product of two slices (< 2^14) and every sum of them
-// over a chunk of at most 128 nodes and over the at most 8 slice pairs of one diagonal stays
+// over a piece of at most 128 nodes and over the at most 8 slice pairs of one diagonal stays
 // below 2^24, so the f16 MMA with FP32 accumulators computes each diagonal exactly; the
-// diagonals are combined in 64-bit integers and converted to FP64 once per chunk.  With
+// diagonals are combined in 64-bit integers and converted to FP64 once per piece.  With
 // NS = 8 (56 bits per operand) and the diagonals i + j <= 8 (43 MMAs per 16-node step; the
 // dropped products are below 2^-60 of the operands' scales) the result matches an FP64
-// contraction to the FP64 rounding level of the sum of |products|.
+// contraction to the FP64 rounding level of the sum of |products|.  In shared memory an operand
+// is 8 bytes, one slice each, and becomes f16 pairs in registers (half2_slice).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -225,8 +226,8 @@ __device__ __forceinline__ void sincos_tab(double th, const double2* __restrict_
   *sn = fma(e.y, c, e.x * s);
 }
 
-// kernel_eval_tc for real k, kinds S, D and CFIE with a real alpha, with the constants folded
-// into the per-node source data: N' = N w alpha / (4 pi) (alpha = 1 for D), Js = beta_r Jw /
+// Kernel value for real k, kinds S, D and CFIE with a real alpha in lean FP64, the constants folded
+// into the per-node source data (the arguments that kernel_eval_ff does not cover): N' = N w alpha / (4 pi) (alpha = 1 for D), Js = beta_r Jw /
 // (4 pi) (Jw / (4 pi) for S), Ks = beta_i Jw / (4 pi), fJ = FP32 Jw / (4 pi).  Then
 //   S: e^{ikr}/r Js,   D and CFIE: e^{ikr}/r ((1 - ikr) N'.d / r^2 + Js + i Ks),
 // about 39 FP64 instructions for the CFIE.  r = 0 gives 0.
@@ -322,57 +323,6 @@ __device__ __forceinline__ cplx kernel_eval_ff(int kind, double kr, ff krf, cons
     im = ff_add(ff_mul(ec, mi), ff_mul(es, mr));
   }
   return {dbl_of(re), dbl_of(im)};
-}
-
-// kernel_eval (lcq_device.cuh) with the table sincos, the Newton-refined FP32 reciprocal
-// square root and the rounding envelope formed in FP32 from the FP64 quantities' bits: the
-// same kernel value to a few ulps.  fJw: FP32 copy of Jw; fR: FP32 patch radius; has_ki:
-// Im k != 0.  r = 0 gives 0.
-__device__ __forceinline__ cplx kernel_eval_tc(const KernelParams& kp, const KernelParamsF& kf,
-                                               const double2* __restrict__ sct, double x0,
-                                               double x1, double x2, double X0, double X1,
-                                               double X2, double N0, double N1, double N2,
-                                               double Jw, float fJw, float fR, float* env,
-                                               const double* nx, bool has_ki) {
-  if (kp.kind == 3) {
-    N0 = -nx[0] * Jw;
-    N1 = -nx[1] * Jw;
-    N2 = -nx[2] * Jw;
-  }
-  const double d0 = x0 - X0, d1 = x1 - X1, d2 = x2 - X2;
-  const double r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
-  if ((__double_as_longlong(r2) << 1) == 0) {
-    *env = 0.0f;
-    return {0.0, 0.0};
-  }
-  const double rinv = rsqrt_nr(r2);
-  const double r = r2 * rinv;
-  const double th = kp.kr * r;
-  double sn, cs;
-  sincos_tab(th, sct, &sn, &cs);
-  double ex = 0.07957747154594767 * rinv;  // 1/(4 pi r)
-  if (has_ki) ex *= exp(-kp.ki * r);
-  {
-    // |G| Jw (|beta| + |alpha| |1 - ik r| R / r^2) in FP32
-    const float fr = f32_bits(r), fri = 1.0f / fr;
-    const float f0 = fmaf(kf.ki, fr, 1.0f), f1 = kf.kr * fr;
-    const float fa = sqrtf(fmaf(f0, f0, f1 * f1));
-    *env = f32_bits(ex) * fJw * fmaf(kf.ea * fa * fR, fri * fri, kf.eb);
-  }
-  const double ec = ex * cs, es = ex * sn;
-  if (kp.kind == 0) return {ec * Jw, es * Jw};
-  const double rinv2 = rinv * rinv;
-  const double ndx = fma(N0, d0, fma(N1, d1, N2 * d2)) * rinv2;
-  // (1 - ikr) ndx with k = kr + i ki: ((1 + ki r) ndx, -kr r ndx)
-  double cr = has_ki ? fma(kp.ki, r, 1.0) * ndx : ndx;
-  double ci = -th * ndx;
-  if (kp.kind == 2) {
-    const double tr = fma(kp.ar, cr, fma(-kp.ai, ci, kp.br * Jw));
-    const double ti = fma(kp.ar, ci, fma(kp.ai, cr, kp.bi * Jw));
-    cr = tr;
-    ci = ti;
-  }
-  return {fma(ec, cr, -es * ci), fma(ec, ci, es * cr)};
 }
 
 // Kernel gradients summed over the targets of one source (or the reverse of k_far_sum): with d =
