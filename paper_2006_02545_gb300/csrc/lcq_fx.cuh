@@ -154,6 +154,9 @@ LCQ_HD FxKernel fx_kernel(int kind, double kr, double ki, double ar, double ai, 
   f.kd = m;
   const double p = ar * ki + ai * kr, q = ai * ki - ar * kr;
   int e1, e2;
+  // a product of the constants that overflows: no phase counts as covered, so that every pair
+  // takes the FP64 kernel
+  if (!(fabs(p) < 1e300 && fabs(q) < 1e300)) f.ek = 100000;
   fx_mant(ar, &e1);
   fx_mant(ai, &e2);
   f.ea = fx_max(e1, e2);

@@ -117,6 +117,7 @@ def test_range(fx):
     assert fx(2, kp, [np.inf, 0.0, 1.0], n, 1.0, True) is None
     assert fx(0, (1e9, 0, 0, 0, 0, 0), [1.0, 0.0, 0.0], n, 1.0, True) is None   # phase
     assert fx(0, (1.0, 1e5, 0, 0, 0, 0), [1.0, 0.0, 0.0], n, 1.0, True) is None  # decay
+    assert fx(2, (1e200, 0, 1e200, 0, 0, 0), [1.0, 0.0, 0.0], n, 1.0, True) is None  # alpha k
     for r in (1e-90, 1e-30, 1e30, 1e89):                             # inside: S, k = 0
         got = fx(0, (0.0, 0, 0, 0, 0, 0), [0.0, r, 0.0], n, 1.0, True)
         assert abs(got - 1.0 / r) <= 4 * U / r
