@@ -212,7 +212,8 @@ TUNING_GENERATIONS = 6
 MIXED_DTYPE = {"fp64": "f64", "fp32": "f32+f64", "two-float": "f32x2+f64",
                "fp32+two-float": "f32+f32x2+f64"}
 FORM_NAMES = {0: "fp64", 1: "fp32", 2: "two-float", 3: "fp32+two-float"}  # lcq_counters [7]
-KERNEL_SOURCES = ("lcq_common.cuh", "lcq_device.cuh", "lcq_tc.cuh")  # k_adaptive and its helpers
+KERNEL_SOURCES = ("lcq_common.cuh", "lcq_device.cuh", "lcq_fx.cuh", "lcq_fxgeom.cuh",
+                  "lcq_tc.cuh")  # k_adaptive and its helpers
 
 
 def kernel_source_sha():
@@ -696,10 +697,10 @@ def run_ours(args, rank, world, local_rank):
     achieved = flops / (a_ms / 1e3) / 1e12
     peak = peaks["fp64_fma_tflops"]
     roofline = {"bound": "alu",
-                "kernel": ("k_adaptive<6>: " + {"fp64": "FP64", "fp32": "FP32",
+                "kernel": ("k_adaptive<6>: " + {"fp64": "64-bit fixed-point", "fp32": "FP32",
                                                  "two-float": "two-float"}.get(
                                FORM_NAMES[main_forms], "mixed") +
-                           " kernel values, FP64 geometry; contraction on the f16 tensor "
+                           " kernel values, fixed-point geometry; contraction on the f16 tensor "
                            "cores by an exact slice split"),
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": traffic_for("k_adaptive"),
