@@ -402,12 +402,15 @@ __device__ __forceinline__ void tc_tile(const uint2* Bs, const uint4* G, const i
 // f16) lets a chunk hold 256 columns where it held 128, so that every thread has a node and the
 // barriers come half as often; they, not the pipes, bounded the kernel (1280-patch CFIE, eps
 // 1e-9: adaptive walk 295 ms at 32% of the issue slots before, 180 ms at 47% since).
-// S: exponent of the fixed-point positions (block_scale).  form: 0 FP64 (fixed point); 1 FP32
+// Positions in fixed point are relative to the centroid at the exponent S = sx + 3 of the patch's own
+// chart (|X_c| < 2^sx, no bit of it dropped); a target beyond 2^(S - 1) in some coordinate, over
+// four times the chart's bound away, takes the FP64 difference (nothing cancels there).  So a
+// target's values do not depend on the targets it shares the call with.  form: 0 FP64 (fixed point); 1 FP32
 // kernel values (the mixed form for eps >= kMixedMinEps); 2 two-float ones (kernel_eval_ff; the
 // mixed form below that) where the constants fold, else FP64.
 template <int D, int FORM, class TA, class OR>
 __device__ __forceinline__ void block_moments_form(
-    const FxChart<D>& ch, int S, const double* __restrict__ ru, const double* __restrict__ rv,
+    const FxChart<D>& ch, const double* __restrict__ ru, const double* __restrict__ rv,
     const double* __restrict__ rw, int Q, const SegMap* segs, int nseg, const TA& ta, int T, OR orow,
     const KernelParams& kp, unsigned char* smb, const double* cen, double R, double* eout) {
   using C = TcCfg<D>;
@@ -425,6 +428,7 @@ __device__ __forceinline__ void block_moments_form(
   int* te = reinterpret_cast<int*>(smb + C::OFF_TE);
   const KernelParamsF kf = to_f32(kp);
   const float fR = f32_bits(R);
+  const int S = ch.sx + 3;
   const FxKernel& fx = kp.fx;  // read at its uses: as a register copy it spills
   const FxTables tab = fx_tables();
   constexpr double kInv4Pi = 0.07957747154594767;
@@ -442,15 +446,20 @@ __device__ __forceinline__ void block_moments_form(
     if (threadIdx.x < nt) {
       double xp[3];
       ta.pos(t0 + threadIdx.x, xp);
-      bool fin = true;
+      bool near = fixed;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
+        int e;
         xp[c] -= cen[c];
-        fin = fin && isfinite(xp[c]);
-        if (fixed) txi[3 * threadIdx.x + c] = fx_fix(xp[c], S);
+        fx_mant(xp[c], &e);
+        near = near && e < S;
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (near) txi[3 * threadIdx.x + c] = fx_fix(xp[c], S);
         else tx[3 * threadIdx.x + c] = xp[c];
       }
-      te[threadIdx.x] = fin ? -100000 : kFxBad + 1;
+      te[threadIdx.x] = !near;
       if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
     }
   };
@@ -556,9 +565,8 @@ __device__ __forceinline__ void block_moments_form(
       fx_chart_point<D>(s, row, X, N);
       const double w = rw[l] * Sg.det;
       if (fixed) {
-        const int k = S - ch.sx;  // >= 1
 #pragma unroll
-        for (int c = 0; c < 3; ++c) Xi[c] = fx_sra(X[c] << 3, k);
+        for (int c = 0; c < 3; ++c) Xi[c] = X[c];  // unit 2^(S - 62)
         fx_node_from_normal(N, ch.su + ch.sv + 1, w, nn, &wm, &ew);
         if (ch.bad) ew = kFxBad + 1;
         const int e = min(max(ew, -120), 120);
@@ -626,13 +634,19 @@ __device__ __forceinline__ void block_moments_form(
                   nt3[1] = fx_unjoin(tn[3 * i + 1]);
                   nt3[2] = fx_unjoin(tn[3 * i + 2]);
                 }
-                const i64 d0 = txi[3 * i] - Xi[0], d1 = txi[3 * i + 1] - Xi[1],
-                          d2 = txi[3 * i + 2] - Xi[2];
-                const int e2 = max(ew, te[i]);
-                if (!fx_eval_int<false>(fx, tab, d0, d1, d2, S, nt3, wm, e2, &g.re, &g.im, &ev,
-                                        kf.kr, kf.ki, kf.eb, kf.ea * fR, Jf))
-                  g = fx_fallback(kp, fx_pack<false>(d0, S - 62), fx_pack<false>(d1, S - 62),
-                                  fx_pack<false>(d2, S - 62), nt3[0], nt3[1], nt3[2], wm, e2,
+                auto diff = [&](int c) {  // x - X in FP64
+                  return te[i] ? tx[3 * i + c] - fx_pack<false>(Xi[c], S - 62)
+                               : fx_pack<false>(txi[3 * i + c] - Xi[c], S - 62);
+                };
+                FxS dm[3];
+                int de;
+                const bool ok =
+                    te[i] ? fx_vector(diff(0), diff(1), diff(2), dm, &de)
+                          : fx_vector_int(txi[3 * i] - Xi[0], txi[3 * i + 1] - Xi[1],
+                                          txi[3 * i + 2] - Xi[2], S, dm, &de);
+                if (!ok || !fx_core<false>(fx, tab, dm[0], dm[1], dm[2], de, nt3, wm, ew, &g.re,
+                                           &g.im, &ev, kf.kr, kf.ki, kf.eb, kf.ea * fR, Jf))
+                  g = fx_fallback(kp, diff(0), diff(1), diff(2), nt3[0], nt3[1], nt3[2], wm, ew,
                                   (double)fR, &ev);
               }
             }
@@ -727,7 +741,7 @@ __device__ __forceinline__ void block_moments_form(
 }
 
 template <int D, class TA, class OR>
-__device__ void block_moments_tc(const FxChart<D>& ch, int S, const double* __restrict__ ru,
+__device__ void block_moments_tc(const FxChart<D>& ch, const double* __restrict__ ru,
                                  const double* __restrict__ rv, const double* __restrict__ rw,
                                  int Q, const SegMap* segs, int nseg, const TA& ta, int T, OR orow,
                                  const KernelParams& kp, unsigned char* smb, const double* cen,
@@ -735,11 +749,11 @@ __device__ void block_moments_tc(const FxChart<D>& ch, int S, const double* __re
   // two-float kernel values: real k, kinds S, D and CFIE with a real alpha, whose constants are
   // folded into the node data
   if (form == 1)
-    block_moments_form<D, 1>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+    block_moments_form<D, 1>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
   else if (form == 2 && kp.ki == 0.0 && kp.kind <= 2 && kp.ai == 0.0)
-    block_moments_form<D, 2>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+    block_moments_form<D, 2>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
   else
-    block_moments_form<D, 0>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+    block_moments_form<D, 0>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
 }
 
 // The moments of the smallest degrees in the FP64 form (n <= 10 basis functions) by the
@@ -751,7 +765,7 @@ __device__ void block_moments_tc(const FxChart<D>& ch, int S, const double* __re
 constexpr int kFp64MomentsMaxDeg = 3;
 template <int D, class TA, class OR>
 __device__ __forceinline__ void block_moments_any(
-    const double* cf, const double* cfd, const FxChart<D>& ch, int S, const double* __restrict__ ru,
+    const double* cf, const double* cfd, const FxChart<D>& ch, const double* __restrict__ ru,
     const double* __restrict__ rv, const double* __restrict__ rw, int Q, const SegMap* segs,
     int nseg, const TA& ta, int T, OR orow, const KernelParams& kp, unsigned char* smb,
     const double* cen, double R, double* eout, int form) {
@@ -767,31 +781,7 @@ __device__ __forceinline__ void block_moments_any(
       return;
     }
   }
-  block_moments_tc<D>(ch, S, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout, form);
-}
-
-// Exponent S of the fixed-point scale of positions relative to the centroid: the chart's (2^sx)
-// and the T targets' coordinates are below 2^(S - 1), so that differences are below 2^S.
-// Block-wide; slot: one int of shared memory; ends with a barrier.
-template <class TA>
-__device__ int block_scale(const TA& ta, int T, const double* cen, int sx, int* slot) {
-  __syncthreads();
-  if (threadIdx.x == 0) *slot = sx;
-  __syncthreads();
-  int m = -1000;
-  for (int i = threadIdx.x; i < T; i += blockDim.x) {
-    double x[3];
-    ta.pos(i, x);
-    for (int c = 0; c < 3; ++c) {
-      int e;
-      fx_mant(x[c] - cen[c], &e);
-      if (e <= 1024) m = max(m, e);  // not the exponent of an infinity or a NaN
-    }
-  }
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0) atomicMax(slot, m);
-  __syncthreads();
-  return *slot + 1;
+  block_moments_tc<D>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout, form);
 }
 
 // Shared-memory bytes of the moment workspace (either engine's).
@@ -1079,7 +1069,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
   // derivative series of the chart, for the FP64 engine of the smallest degrees
   __shared__ double cfd[D <= kFp64MomentsMaxDeg ? 2 * 3 * (D * (D + 1) / 2) : 1];
   __shared__ FxChart<D> ch;
-  __shared__ int tsc;
   const double* cfdp = cfd;
 
   for (;;) {
@@ -1130,8 +1119,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
     __syncthreads();
     if constexpr (D <= kFp64MomentsMaxDeg) load_coef_derivs<D>(cf, dv.duv[D], cfd);
     load_fx_chart<D>(cf, dv.duv[D], &ch);
-    const int S2 = block_scale(TgtPairIdx{dv.tgt, dv.NT, dv.pair_tgt, apairs, dv.tnrm}, A,
-                               dv.cen + 3 * j, ch.sx, &tsc);
     if constexpr (GRAD) {
 #pragma unroll
       for (int e = 0; e < 3 * n; ++e) Mg[e] = 0.0;
@@ -1155,7 +1142,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
     __syncthreads();
     if (leaf_order > 0) {
       TgtPairIdx ta{dv.tgt, dv.NT, dv.pair_tgt, apairs, dv.tnrm};
-      block_moments_any<D>(cf, cfdp, ch, S2, ru, rv, rw, Q, segs, 1, ta, A,
+      block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, Q, segs, 1, ta, A,
                            [=] __device__(int i) { return lvlI + (int64_t)i * 4 * n; }, kps, smb,
                            dv.cen + 3 * j, Rj, tmpE, formj);
     }
@@ -1207,7 +1194,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
       __syncthreads();
       // children moments of every target in S
       TgtAdaptive ta{dv.tgt, dv.NT, dv.pair_tgt, apairs, ST, dv.tnrm};
-      block_moments_any<D>(cf, cfdp, ch, S2, ru, rv, rw, Q, segs, 4, ta, S,
+      block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, Q, segs, 4, ta, S,
                            [=] __device__(int i) { return tmp + (int64_t)i * 4 * n; }, kps, smb,
                            dv.cen + 3 * j, Rj, tmpE, formj);
       __syncthreads();

@@ -408,17 +408,14 @@ LCQ_HD bool fx_core(const FxKernel& K, const FxTables& tab, FxS D0, FxS D1, FxS 
   return true;
 }
 
-// The same from FP64 coordinates of d; also false for |d| outside [2^-300, 2^300], zero among them.
-template <bool INT>
-LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1, double d2,
-                    const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
-                    float fki, float feb, float feaR, float fw) {
+// d = x - X as fx_core takes it, D 2^(E - 62) with 2^61 <= max |D_c| < 2^62, from FP64 coordinates;
+// false for |d| outside [2^-300, 2^300], zero among them.
+LCQ_HD bool fx_vector(double d0, double d1, double d2, FxS* D, int* E) {
   const u64 b[3] = {fx_bits(d0), fx_bits(d1), fx_bits(d2)};
   int xs[3];
   for (int c = 0; c < 3; ++c) xs[c] = (int)(fx_hi(b[c]) & 0x7fffffffu) >> 20;
   const int ex = fx_max(xs[0], fx_max(xs[1], xs[2]));
   if ((unsigned)(ex - 723) > 600u) return false;
-  FxS D[3];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
@@ -426,20 +423,39 @@ LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1
     const u64 m = ((b[c] & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
     D[c] = fx_split((i64)(m >> fx_min(ex - xs[c], 63)) ^ ((i64)b[c] >> 63));
   }
-  return fx_core<INT>(K, tab, D[0], D[1], D[2], ex - 1022, n, w, ew, re, im, env, fk, fki, feb,
-                      feaR, fw);
+  *E = ex - 1022;
+  return true;
 }
 
 // The same from d = (d0, d1, d2) 2^(S - 62), |d_c| < 2^62; also false for d = 0.
+LCQ_HD bool fx_vector_int(i64 d0, i64 d1, i64 d2, int S, FxS* D, int* E) {
+  const int sh = fx_clz((u64)((d0 ^ (d0 >> 63)) | (d1 ^ (d1 >> 63)) | (d2 ^ (d2 >> 63)))) - 2;
+  *E = S - sh;
+  if (sh > 61 || (unsigned)(*E + 300) > 600u) return false;
+  D[0] = fx_split(d0 << sh);
+  D[1] = fx_split(d1 << sh);
+  D[2] = fx_split(d2 << sh);
+  return true;
+}
+
+// fx_core from FP64 coordinates of d, and from integers at one exponent.
+template <bool INT>
+LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1, double d2,
+                    const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
+                    float fki, float feb, float feaR, float fw) {
+  FxS D[3];
+  int E;
+  return fx_vector(d0, d1, d2, D, &E) &&
+         fx_core<INT>(K, tab, D[0], D[1], D[2], E, n, w, ew, re, im, env, fk, fki, feb, feaR, fw);
+}
 template <bool INT>
 LCQ_HD bool fx_eval_int(const FxKernel& K, const FxTables& tab, i64 d0, i64 d1, i64 d2, int S,
                         const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
                         float fki, float feb, float feaR, float fw) {
-  const int sh = fx_clz((u64)((d0 ^ (d0 >> 63)) | (d1 ^ (d1 >> 63)) | (d2 ^ (d2 >> 63)))) - 2;
-  const int E = S - sh;
-  if (sh > 61 || (unsigned)(E + 300) > 600u) return false;
-  return fx_core<INT>(K, tab, fx_split(d0 << sh), fx_split(d1 << sh), fx_split(d2 << sh), E, n, w,
-                      ew, re, im, env, fk, fki, feb, feaR, fw);
+  FxS D[3];
+  int E;
+  return fx_vector_int(d0, d1, d2, S, D, &E) &&
+         fx_core<INT>(K, tab, D[0], D[1], D[2], E, n, w, ew, re, im, env, fk, fki, feb, feaR, fw);
 }
 
 }  // namespace lcq

@@ -141,7 +141,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_rule_moments(
   // derivative series of the chart, for the FP64 engine of the smallest degrees
   __shared__ double cfd[D <= kFp64MomentsMaxDeg ? 2 * 3 * (D * (D + 1) / 2) : 1];
   __shared__ FxChart<D> ch;
-  __shared__ int tsc;
   const double* cfdp = cfd;
   const int64_t ld = dv.ldI;
   for (int b = blockIdx.x; b < count; b += gridDim.x) {
@@ -168,8 +167,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_rule_moments(
         const int64_t p0 = dv.pair_ptr[j], np = dv.pair_ptr[j + 1] - p0;
         TgtIdx ta{dv.tgt, dv.NT, dv.pair_tgt + p0, dv.tnrm};
         cplx* base = out_smooth + p0 * ld;
-        const int S = block_scale(ta, (int)np, dv.cen + 3 * j, ch.sx, &tsc);
-        block_moments_any<D>(cf, cfdp, ch, S, ru, rv, rw, m * m, segs, 1, ta, (int)np,
+        block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, m * m, segs, 1, ta, (int)np,
                              [=] __device__(int i) { return base + (int64_t)i * ld; }, kps, smb,
                              dv.cen + 3 * j, 0.0, nullptr, formj);
         evals += np * m * m;
@@ -177,8 +175,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_rule_moments(
         const int64_t a0 = dv.an_ptr[j], na = dv.an_ptr[j + 1] - a0;
         const int32_t* pl = dv.an_pair + a0;
         TgtPairIdx ta{dv.tgt, dv.NT, dv.pair_tgt, pl, dv.tnrm};
-        const int S = block_scale(ta, (int)na, dv.cen + 3 * j, ch.sx, &tsc);
-        block_moments_any<D>(cf, cfdp, ch, S, ru, rv, rw, m * m, segs, 1, ta, (int)na,
+        block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, m * m, segs, 1, ta, (int)na,
                              [=] __device__(int i) { return out_ann + (int64_t)pl[i] * ld; }, kps,
                              smb, dv.cen + 3 * j, 0.0, nullptr, formj);
         evals += na * m * m;

@@ -51,7 +51,7 @@ struct TcCfg {
   static constexpr int OFF_EP = OFF_TX + 6 * TT * 8;           // Ep[TT][MAXP] float
   static constexpr int OFF_RE = OFF_EP + TT * MAXP * 4;        // rowE[MAXP][TT][2] int
   static constexpr int OFF_PC = OFF_RE + MAXP * TT * 2 * 4;    // pieces[MAXP][8] int
-  static constexpr int OFF_TE = OFF_PC + MAXP * 8 * 4;         // te[TT] int: target not finite
+  static constexpr int OFF_TE = OFF_PC + MAXP * 8 * 4;         // te[TT] int: target far off
   static constexpr int BYTES = OFF_TE + TT * 4;
 };
 

@@ -1,0 +1,87 @@
+"""The fixed-point arithmetic of the moment engine, the self rules and the sums where its scales
+could show in the results."""
+import numpy as np
+import pytest
+
+from paper_2006_02545_gb300 import workloads as W
+from .gpu_helpers import run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import __graft_entry__ as g
+    g.build()
+    from paper_2006_02545_gb300 import lcq
+    c = lcq.Context(0)
+    yield c
+    c.close()
+
+
+def one_patch(deg):
+    s = W.ellipsoid(2, deg, axes=(1.0, 1.2, 0.9))
+    n = W.n_nodes(deg)
+    return W.Surface("one", s.deg[:1].copy(), s.node_off[:2].copy(),
+                     np.ascontiguousarray(s.xyz[:, :n]), {})
+
+
+def near_points(s, nt, seed=1):
+    """Points 1e-3 to 0.3 off the patch, above its nodes."""
+    rng = np.random.default_rng(seed)
+    i = np.arange(nt) % s.n_points
+    return np.ascontiguousarray(s.xyz[:, i] * (1.0 + 10.0 ** rng.uniform(-3, -0.5, nt)))
+
+
+@pytest.mark.parametrize("deg", [3, 4, 6, 7, 8])
+@pytest.mark.parametrize("far", [1e3, 1e9, 1e18])
+def test_a_distant_target_leaves_the_others_alone(ctx, deg, far):
+    """A target's corrections do not depend on the targets it shares the patch with: the
+    allocation-free entry with its last target 2 away and far away gives the same rows of the
+    others bit for bit; so does a generation (the far order at its cap, so that it is the same)."""
+    import torch
+    from paper_2006_02545_gb300 import lcq
+    s, nt = one_patch(deg), 21
+    x = near_points(s, nt)
+    n = W.n_nodes(deg)
+    y = torch.from_numpy(s.xyz).cuda()
+    rows, vals = [], []
+    for dist in (2.0, far):
+        x[:, -1] = x[:, 0] * dist
+        out = torch.zeros((nt, n), dtype=torch.complex128, device="cuda")
+        st = lcq.adaptive_corrections_noalloc(deg, y, torch.from_numpy(x).cuda(), "CFIE", 2.0, 8, 1e-6,
+                                              out, 1.0, -2j, max_depth=6)
+        assert st in (0, 4)                       # the depth cap is reported
+        rows.append(out.cpu().numpy())
+        g = run_gpu(ctx, s, x, -np.ones(nt, np.int64), "CFIE", 2.0, 1e-12, eta=4 * far, alpha=1.0,
+                    beta=-2j, eta1=4 * far, m_max=6, leaf_order=8, max_depth=5, eps_loosen=1e6)
+        assert g["status"] in (0, 4) and g["q"][0] == 6
+        vals.append(g["val"].reshape(nt, n))
+    assert np.isfinite(rows[1]).all() and np.abs(rows[0]).max() > 0
+    assert np.array_equal(rows[0][:-1], rows[1][:-1])
+    assert np.array_equal(vals[0][:-1], vals[1][:-1])
+
+
+def test_group_size_with_targets_far_beyond_the_patch():
+    """The group size stays without effect on the results when adaptive targets lie well outside
+    their patch's coordinate range (a large eta1)."""
+    from paper_2006_02545_gb300 import lcq
+    s = W.ellipsoid(2, 4, axes=(1.0, 1.5, 2.0))
+    rng = np.random.default_rng(4)
+    x = rng.standard_normal((3, 300))
+    x *= 10.0 ** rng.uniform(0.35, 2.0, 300) / np.linalg.norm(x, axis=0)
+    tn = -np.ones(300, np.int64)
+    c = lcq.Context(0)
+    try:
+        runs, sizes = [], []
+        for _ in range(6):
+            g = run_gpu(c, s, x, tn, "CFIE", 1.0, 1e-8, 400.0, alpha=1.0, beta=-1j, eta1=400.0)
+            assert g["status"] == 0
+            sizes.append(int(c.counters()[5]))
+            runs.append(g)
+        assert len(set(sizes)) >= 2, sizes
+        for g in runs[1:]:
+            assert np.array_equal(g["val"], runs[0]["val"])
+            assert np.array_equal(g["leaves"], runs[0]["leaves"])
+    finally:
+        c.close()
