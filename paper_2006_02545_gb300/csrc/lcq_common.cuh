@@ -99,6 +99,99 @@ struct Cfg {
   static constexpr int WS = CH * BS + 8 * CH + 3 * TT * CH + 6 * TT;
 };
 
+// Target accessors of block_moments: pos(i, x) the position of target i; nrm(i, xrel, n)
+// its unit normal for S' (the caller's normals tn, SoA [3][NT]; for bare test points the
+// radial direction from the centroid, xrel being the position relative to it).
+__device__ __forceinline__ void read_nrm(const double* tn, int64_t NT, int64_t t, double* n) {
+  n[0] = tn[t];
+  n[1] = tn[NT + t];
+  n[2] = tn[2 * NT + t];
+}
+// Output rows of targets: row i at base + i ld, or at base + idx[i] ld.
+struct RowsBy {
+  cplx* base;
+  const int32_t* idx;
+  int64_t ld;
+  __device__ __forceinline__ cplx* operator()(int i) const {
+    return base + (int64_t)(idx ? idx[i] : i) * ld;
+  }
+  __device__ __forceinline__ RowsBy any() const { return *this; }
+};
+struct RowsAt {
+  cplx* base;
+  int64_t ld;
+  __device__ __forceinline__ cplx* operator()(int i) const { return base + (int64_t)i * ld; }
+  __device__ __forceinline__ RowsBy any() const { return {base, nullptr, ld}; }
+};
+// Any of the target lists below: ids a[b[c[i]]], lists that are null left out.
+struct TgtAny {
+  const double* tgt;
+  int64_t NT;
+  const int32_t *a, *b, *c;
+  const double* tn;
+  __device__ int64_t id(int i) const {
+    if (c) i = c[i];
+    if (b) i = b[i];
+    return a[i];
+  }
+  __device__ void pos(int i, double* x) const {
+    const int64_t t = id(i);
+    x[0] = tgt[t];
+    x[1] = tgt[NT + t];
+    x[2] = tgt[2 * NT + t];
+  }
+  __device__ void nrm(int i, const double*, double* n) const { read_nrm(tn, NT, id(i), n); }
+};
+struct TgtIdx {  // targets by id list
+  const double* tgt;
+  int64_t NT;
+  const int32_t* ids;
+  const double* tn;
+  __device__ void pos(int i, double* x) const {
+    const int64_t t = ids[i];
+    x[0] = tgt[t];
+    x[1] = tgt[NT + t];
+    x[2] = tgt[2 * NT + t];
+  }
+  __device__ void nrm(int i, const double*, double* n) const { read_nrm(tn, NT, ids[i], n); }
+  __device__ TgtAny any() const { return {tgt, NT, ids, nullptr, nullptr, tn}; }
+};
+struct TgtPairIdx {  // targets of pair ids
+  const double* tgt;
+  int64_t NT;
+  const int32_t* pair_tgt;
+  const int32_t* pairs;
+  const double* tn;
+  __device__ void pos(int i, double* x) const {
+    const int64_t t = pair_tgt[pairs[i]];
+    x[0] = tgt[t];
+    x[1] = tgt[NT + t];
+    x[2] = tgt[2 * NT + t];
+  }
+  __device__ void nrm(int i, const double*, double* n) const {
+    read_nrm(tn, NT, pair_tgt[pairs[i]], n);
+  }
+  __device__ TgtAny any() const { return {tgt, NT, pair_tgt, pairs, nullptr, tn}; }
+};
+struct TgtAdaptive {  // targets of a union-tree node: local ids -> pairs -> targets
+  const double* tgt;
+  int64_t NT;
+  const int32_t* pair_tgt;
+  const int32_t* apairs;
+  const int* ST;
+  const double* tn;
+  __device__ void pos(int i, double* x) const {
+    const int64_t t = pair_tgt[apairs[ST[i]]];
+    x[0] = tgt[t];
+    x[1] = tgt[NT + t];
+    x[2] = tgt[2 * NT + t];
+  }
+  __device__ void nrm(int i, const double*, double* n) const {
+    read_nrm(tn, NT, pair_tgt[apairs[ST[i]]], n);
+  }
+  __device__ TgtAny any() const { return {tgt, NT, pair_tgt, apairs, ST, tn}; }
+};
+
 // Unit normal of a target (S') as fx_eval takes a node's, negated: S' is the double-layer
 // form with -n_x in the place of the source's normal.
 template <class TA>
@@ -407,8 +500,9 @@ __device__ __forceinline__ void tc_tile(const uint2* Bs, const uint4* G, const i
 // four times the chart's bound away, takes the FP64 difference (nothing cancels there).  So a
 // target's values do not depend on the targets it shares the call with.  form: 0 FP64 (fixed point); 1 FP32
 // kernel values (the mixed form for eps >= kMixedMinEps); 2 two-float ones (kernel_eval_ff; the
-// mixed form below that) where the constants fold, else FP64.
-template <int D, int FORM, class TA, class OR>
+// mixed form below that) where the constants fold, else FP64.  GEO64: a chart that the fixed-point
+// scales do not fit (FxChart::fp64), with FP64 nodes (the rows of kw_row_factors) and differences.
+template <int D, int FORM, bool GEO64, class TA, class OR>
 __device__ __forceinline__ void block_moments_form(
     const FxChart<D>& ch, const double* __restrict__ ru, const double* __restrict__ rv,
     const double* __restrict__ rw, int Q, const SegMap* segs, int nseg, const TA& ta, int T, OR orow,
@@ -440,13 +534,13 @@ __device__ __forceinline__ void block_moments_form(
   // midpoint descendants) keeps a function of the rule's v alone
   const int mr = (int)lrintf(sqrtf((float)Q));
   using RW = FxRow<D>;
-  constexpr int kRowMax = C::G_BYTES / 8 / RW::size;
+  constexpr int kRowSize = GEO64 ? KwRow<D>::size : RW::size, kRowMax = C::G_BYTES / 8 / kRowSize;
   // targets of a tile; up to TT targets in all are loaded once, in the shadow of the first rows
   auto load_targets = [&](int t0, int nt) {
     if (threadIdx.x < nt) {
       double xp[3];
       ta.pos(t0 + threadIdx.x, xp);
-      bool near = fixed;
+      bool near = fixed && !GEO64;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         int e;
@@ -530,7 +624,13 @@ __device__ __forceinline__ void block_moments_form(
       const int* pc = pcs + 8 * k;
       const SegMap& Sg = segs[pc[0]];
       const int l = (pc[4] + rr - pc[5]) * mr;
-      fx_row_factors<D>(Sg.ay + ru[l] * Sg.e1y + rv[l] * Sg.e2y, m, ch, rows + rr * RW::size);
+      const double v = Sg.ay + ru[l] * Sg.e1y + rv[l] * Sg.e2y;
+      if constexpr (GEO64)
+        kw_row_factors<D>(v, m, reinterpret_cast<const double*>(ch.x),
+                          reinterpret_cast<const double*>(ch.d),
+                          reinterpret_cast<double*>(rows) + rr * kRowSize);
+      else
+        fx_row_factors<D>(v, m, ch, rows + rr * kRowSize);
     }
     __syncthreads();
     // (2) this thread's node
@@ -540,11 +640,11 @@ __device__ __forceinline__ void block_moments_form(
     const int ql = col - pcs[8 * pk + 3];
     const bool in = col < ncp, real = in && ql < pcs[8 * pk + 2];
     const int pe = pcs[8 * pk + 7];  // the piece that holds its row scales
-    i64 Xi[3] = {0, 0, 0};   // fixed: point and node for fx_eval_int
+    i64 Xi[3] = {0, 0, 0};   // fixed: point (2^(62 - S)) and node for fx_core
     FxS nn[3] = {{0, 0}, {0, 0}, {0, 0}};
     u64 wm = 0;
     int ew = 0;
-    double Xd[3] = {0, 0, 0};  // two-float and FP32: point, weighted normal and area
+    double Xd[3] = {0, 0, 0};  // point in FP64; two-float and FP32: weighted normal and area
     ff Nff[3] = {{0, 0}, {0, 0}, {0, 0}}, Jff = {0, 0}, Kff = {0, 0};
     float Nf[3] = {0, 0, 0}, Jf = 0.0f;
     if (real) {
@@ -554,30 +654,43 @@ __device__ __forceinline__ void block_moments_form(
       const double r0 = ru[l], r1 = rv[l];
       const double u = Sg.ax + r0 * Sg.e1x + r1 * Sg.e2x;
       const double v = Sg.ay + r0 * Sg.e1y + r1 * Sg.e2y;
-      const FxS s = fx_split(fx_fix(2.0 * u + v - 1.0, 0));
-      const u64* row = rows + (pc[5] + l / mr - pc[4]) * RW::size;
-      fx_basis_point<D>(s, row, part, C::PARTS, [&](int idx, i64 kv) {
-        const u64 sgn = (u64)(kv >> 63);
-        // 56 bits, rounded; below 2^56, since |K_nm| (1 + 1e-12) < 2^E_nm
-        Bs[idx * C::BST + col] = slice_bytes(((((u64)kv ^ sgn) - sgn) + 4) >> 3, kv < 0);
-      });
-      i64 X[3], N[3];
-      fx_chart_point<D>(s, row, X, N);
+      const u64* row = rows + (pc[5] + l / mr - pc[4]) * kRowSize;
       const double w = rw[l] * Sg.det;
-      if (fixed) {
+      i64 X[3], N[3];
+      int sn = 0;
+      double Nn[3];  // of the FP64 nodes, and for the two-float and FP32 values
+      if constexpr (GEO64) {
+        double Xu[3], Xv[3];
+        kw_geometry_row_emit<D>(u, reinterpret_cast<const double*>(row), Xd, Xu, Xv,
+                                [&](int idx, double k) {
+          if (idx % C::PARTS == part)
+            Bs[idx * C::BST + col] = slice_bytes(fix_mag<8>(k, c_kwexp[idx]), __double2hiint(k) < 0);
+        });
+        cross3(Xu, Xv, Nn);
+        if (fixed) fx_make_node(Nn, w, nn, &wm, &ew);
+      } else {
+        const FxS s = fx_split(fx_fix(2.0 * u + v - 1.0, 0));
+        fx_basis_point<D>(s, row, part, C::PARTS, [&](int idx, i64 kv) {
+          const u64 sgn = (u64)(kv >> 63);
+          // 56 bits, rounded; below 2^56, since |K_nm| (1 + 1e-12) < 2^E_nm
+          Bs[idx * C::BST + col] = slice_bytes(((((u64)kv ^ sgn) - sgn) + 4) >> 3, kv < 0);
+        });
+        fx_chart_point<D>(s, row, ch.su, ch.sv, X, N, &sn);
+        if (fixed) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) Xi[c] = X[c];  // unit 2^(S - 62)
-        fx_node_from_normal(N, ch.su + ch.sv + 1, w, nn, &wm, &ew);
-        if (ch.bad) ew = kFxBad + 1;
+          for (int c = 0; c < 3; ++c) Xi[c] = X[c];  // unit 2^(S - 62)
+          fx_node_from_normal(N, sn + 1, w, nn, &wm, &ew);
+        }
+      }
+      if (fixed) {
         const int e = min(max(ew, -120), 120);
         Jf = (float)(uint32_t)(wm >> 32) * 9.31322575e-10f * __int_as_float((127 + e) << 23);
       } else {
-        double Nn[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          Xd[c] = ch.bad ? __longlong_as_double(0x7ff8000000000000ll)
-                         : fx_pack<false>(X[c], ch.sx - 59);
-          Nn[c] = fx_pack<false>(N[c], ch.su + ch.sv - 61);
+          if (GEO64) continue;
+          Xd[c] = fx_pack<false>(X[c], ch.sx - 59);
+          Nn[c] = fx_pack<false>(N[c], sn - 61);
         }
         const double N2 = fma(Nn[0], Nn[0], fma(Nn[1], Nn[1], Nn[2] * Nn[2]));
         const double Jw = N2 > 0.0 ? N2 * rsqrt_nr(N2) * w : 0.0;
@@ -635,13 +748,14 @@ __device__ __forceinline__ void block_moments_form(
                   nt3[2] = fx_unjoin(tn[3 * i + 2]);
                 }
                 auto diff = [&](int c) {  // x - X in FP64
-                  return te[i] ? tx[3 * i + c] - fx_pack<false>(Xi[c], S - 62)
-                               : fx_pack<false>(txi[3 * i + c] - Xi[c], S - 62);
+                  return GEO64   ? tx[3 * i + c] - Xd[c]
+                         : te[i] ? tx[3 * i + c] - fx_pack<false>(Xi[c], S - 62)
+                                 : fx_pack<false>(txi[3 * i + c] - Xi[c], S - 62);
                 };
                 FxS dm[3];
                 int de;
                 const bool ok =
-                    te[i] ? fx_vector(diff(0), diff(1), diff(2), dm, &de)
+                    GEO64 || te[i] ? fx_vector(diff(0), diff(1), diff(2), dm, &de)
                           : fx_vector_int(txi[3 * i] - Xi[0], txi[3 * i + 1] - Xi[1],
                                           txi[3 * i + 2] - Xi[2], S, dm, &de);
                 if (!ok || !fx_core<false>(fx, tab, dm[0], dm[1], dm[2], de, nt3, wm, ew, &g.re,
@@ -740,20 +854,44 @@ __device__ __forceinline__ void block_moments_form(
   }
 }
 
+// two-float kernel values: real k, kinds S, D and CFIE with a real alpha, whose constants are
+// folded into the node data
+template <int D, bool GEO64, class TA, class OR>
+__device__ __forceinline__ void block_moments_forms(
+    const FxChart<D>& ch, const double* __restrict__ ru, const double* __restrict__ rv,
+    const double* __restrict__ rw, int Q, const SegMap* segs, int nseg, const TA& ta, int T, OR orow,
+    const KernelParams& kp, unsigned char* smb, const double* cen, double R, double* eout, int form) {
+  if (form == 1)
+    block_moments_form<D, 1, GEO64>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+  else if (form == 2 && kp.ki == 0.0 && kp.kind <= 2 && kp.ai == 0.0)
+    block_moments_form<D, 2, GEO64>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+  else
+    block_moments_form<D, 0, GEO64>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+}
+
+// Out of line and for any accessors: few charts take it, so that it costs the others' kernels no
+// registers and is compiled once per degree.
+template <int D>
+__device__ __noinline__ void block_moments_fp64(
+    const FxChart<D>& ch, const double* __restrict__ ru, const double* __restrict__ rv,
+    const double* __restrict__ rw, int Q, const SegMap* segs, int nseg, const TgtAny& ta, int T,
+    const RowsBy& orow, const KernelParams& kp, unsigned char* smb, const double* cen, double R,
+    double* eout, int form) {
+  block_moments_forms<D, true>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout, form);
+}
+
 template <int D, class TA, class OR>
 __device__ void block_moments_tc(const FxChart<D>& ch, const double* __restrict__ ru,
                                  const double* __restrict__ rv, const double* __restrict__ rw,
                                  int Q, const SegMap* segs, int nseg, const TA& ta, int T, OR orow,
                                  const KernelParams& kp, unsigned char* smb, const double* cen,
                                  double R, double* eout, int form) {
-  // two-float kernel values: real k, kinds S, D and CFIE with a real alpha, whose constants are
-  // folded into the node data
-  if (form == 1)
-    block_moments_form<D, 1>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
-  else if (form == 2 && kp.ki == 0.0 && kp.kind <= 2 && kp.ai == 0.0)
-    block_moments_form<D, 2>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+  if (ch.fp64)
+    block_moments_fp64<D>(ch, ru, rv, rw, Q, segs, nseg, ta.any(), T, orow.any(), kp, smb, cen, R,
+                          eout, form);
   else
-    block_moments_form<D, 0>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout);
+    block_moments_forms<D, false>(ch, ru, rv, rw, Q, segs, nseg, ta, T, orow, kp, smb, cen, R, eout,
+                                  form);
 }
 
 // The moments of the smallest degrees in the FP64 form (n <= 10 basis functions) by the
@@ -798,43 +936,6 @@ __device__ __forceinline__ void load_coef(const double* __restrict__ coef, int64
   for (int e = threadIdx.x; e < 3 * n; e += blockDim.x) cf[e] = coef[off * 3 + e];
 }
 
-// Target accessors of block_moments: pos(i, x) the position of target i; nrm(i, xrel, n)
-// its unit normal for S' (the caller's normals tn, SoA [3][NT]; for bare test points the
-// radial direction from the centroid, xrel being the position relative to it).
-__device__ __forceinline__ void read_nrm(const double* tn, int64_t NT, int64_t t, double* n) {
-  n[0] = tn[t];
-  n[1] = tn[NT + t];
-  n[2] = tn[2 * NT + t];
-}
-struct TgtIdx {  // targets by id list
-  const double* tgt;
-  int64_t NT;
-  const int32_t* ids;
-  const double* tn;
-  __device__ void pos(int i, double* x) const {
-    const int64_t t = ids[i];
-    x[0] = tgt[t];
-    x[1] = tgt[NT + t];
-    x[2] = tgt[2 * NT + t];
-  }
-  __device__ void nrm(int i, const double*, double* n) const { read_nrm(tn, NT, ids[i], n); }
-};
-struct TgtPairIdx {  // targets of pair ids
-  const double* tgt;
-  int64_t NT;
-  const int32_t* pair_tgt;
-  const int32_t* pairs;
-  const double* tn;
-  __device__ void pos(int i, double* x) const {
-    const int64_t t = pair_tgt[pairs[i]];
-    x[0] = tgt[t];
-    x[1] = tgt[NT + t];
-    x[2] = tgt[2 * NT + t];
-  }
-  __device__ void nrm(int i, const double*, double* n) const {
-    read_nrm(tn, NT, pair_tgt[pairs[i]], n);
-  }
-};
 struct TgtPts {  // explicit points [i][3]
   const double* p;
   __device__ void pos(int i, double* x) const {
@@ -852,24 +953,6 @@ struct TgtPts {  // explicit points [i][3]
       n[0] = n[1] = 0.0;
       n[2] = 1.0;
     }
-  }
-};
-
-struct TgtAdaptive {  // targets of a union-tree node: local ids -> pairs -> targets
-  const double* tgt;
-  int64_t NT;
-  const int32_t* pair_tgt;
-  const int32_t* apairs;
-  const int* ST;
-  const double* tn;
-  __device__ void pos(int i, double* x) const {
-    const int64_t t = pair_tgt[apairs[ST[i]]];
-    x[0] = tgt[t];
-    x[1] = tgt[NT + t];
-    x[2] = tgt[2 * NT + t];
-  }
-  __device__ void nrm(int i, const double*, double* n) const {
-    read_nrm(tn, NT, pair_tgt[apairs[ST[i]]], n);
   }
 };
 
@@ -1143,7 +1226,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
     if (leaf_order > 0) {
       TgtPairIdx ta{dv.tgt, dv.NT, dv.pair_tgt, apairs, dv.tnrm};
       block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, Q, segs, 1, ta, A,
-                           [=] __device__(int i) { return lvlI + (int64_t)i * 4 * n; }, kps, smb,
+                           RowsAt{lvlI, 4 * n}, kps, smb,
                            dv.cen + 3 * j, Rj, tmpE, formj);
     }
     // DFS stack entries: level (8 bits) | child (2 bits) | path (2 bits per level) << 16
@@ -1195,7 +1278,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
       // children moments of every target in S
       TgtAdaptive ta{dv.tgt, dv.NT, dv.pair_tgt, apairs, ST, dv.tnrm};
       block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, Q, segs, 4, ta, S,
-                           [=] __device__(int i) { return tmp + (int64_t)i * 4 * n; }, kps, smb,
+                           RowsAt{tmp, 4 * n}, kps, smb,
                            dv.cen + 3 * j, Rj, tmpE, formj);
       __syncthreads();
       my_tests += S;

@@ -356,10 +356,11 @@ __device__ __forceinline__ void kw_row_factors(double v, int m, const double* cf
   }
 }
 
-// X, X_u, X_v and the basis values K (stride 1) at (u, v) from the row factors of v.
-template <int D>
-__device__ __forceinline__ void kw_geometry_row(double u, const double* row, double* X,
-                                                double* Xu, double* Xv, double* K) {
+// X, X_u, X_v at (u, v) from the row factors of v; each basis value K_nm is handed to emit(idx, K_nm)
+// as it is formed (idx = n(n+1)/2 + m).
+template <int D, class F>
+__device__ __forceinline__ void kw_geometry_row_emit(double u, const double* row, double* X,
+                                                     double* Xu, double* Xv, F&& emit) {
   using RW = KwRow<D>;
   const double v = row[0];
   const double s = 2.0 * u + v - 1.0;
@@ -388,7 +389,7 @@ __device__ __forceinline__ void kw_geometry_row(double u, const double* row, dou
 #pragma unroll
     for (int a = 0; a <= D - m; ++a) {
       const int nn = m + a, idx = nn * (nn + 1) / 2 + m;
-      K[idx] = L * row[RW::J + idx];
+      emit(idx, L * row[RW::J + idx]);
     }
   }
   X[0] = x0;
@@ -400,6 +401,13 @@ __device__ __forceinline__ void kw_geometry_row(double u, const double* row, dou
   Xv[0] = v0;
   Xv[1] = v1;
   Xv[2] = v2;
+}
+
+// X, X_u, X_v and the basis values K (stride 1) at (u, v) from the row factors of v.
+template <int D>
+__device__ __forceinline__ void kw_geometry_row(double u, const double* row, double* X,
+                                                double* Xu, double* Xv, double* K) {
+  kw_geometry_row_emit<D>(u, row, X, Xu, Xv, [&](int idx, double k) { K[idx] = k; });
 }
 
 // cfd for kw_geometry_proj from cf and the projections duv (Du [n][nd], then Dv), by

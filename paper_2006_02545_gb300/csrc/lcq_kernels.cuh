@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_rule_moments(
         TgtIdx ta{dv.tgt, dv.NT, dv.pair_tgt + p0, dv.tnrm};
         cplx* base = out_smooth + p0 * ld;
         block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, m * m, segs, 1, ta, (int)np,
-                             [=] __device__(int i) { return base + (int64_t)i * ld; }, kps, smb,
+                             RowsAt{base, ld}, kps, smb,
                              dv.cen + 3 * j, 0.0, nullptr, formj);
         evals += np * m * m;
       } else {
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_rule_moments(
         const int32_t* pl = dv.an_pair + a0;
         TgtPairIdx ta{dv.tgt, dv.NT, dv.pair_tgt, pl, dv.tnrm};
         block_moments_any<D>(cf, cfdp, ch, ru, rv, rw, m * m, segs, 1, ta, (int)na,
-                             [=] __device__(int i) { return out_ann + (int64_t)pl[i] * ld; }, kps,
+                             RowsBy{out_ann, pl, ld}, kps,
                              smb, dv.cen + 3 * j, 0.0, nullptr, formj);
         evals += na * m * m;
       }
@@ -416,6 +416,20 @@ __device__ __forceinline__ void self_entry(const SelfSeg* sg, int nseg, int ns, 
   out[2] = glw[ti] * (hi - lo) * g.mu * (0.5 * (ex + exi)) * g.area2 * Mm[4];
 }
 
+// Basis slices (column B, stride st) and normal X_u x X_v of a node of a chart that the fixed-point
+// scales do not fit.  Rare, so out of line.
+template <int D>
+__device__ __noinline__ void self_node_fp64(double u, double v, const FxChart<D>& ch, uint2* B, int st,
+                                            double* N) {
+  double K[(D + 1) * (D + 2) / 2], X[3], Xu[3], Xv[3];
+  kw_geometry_proj<D>(u, v, reinterpret_cast<const double*>(ch.x),
+                      reinterpret_cast<const double*>(ch.d), X, Xu, Xv, K);
+#pragma unroll 1
+  for (int k = 0; k < (D + 1) * (D + 2) / 2; ++k)
+    B[k * st] = slice_bytes(fix_mag<8>(K[k], c_kwexp[k]), __double2hiint(K[k]) < 0);
+  cross3(Xu, Xv, N);
+}
+
 template <int D>
 __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t* __restrict__ deg_of_patch,
                                               const KernelParams kp, int order,
@@ -555,17 +569,23 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
         const double sv = glx[si], du = sv * en[0], dvv = sv * en[1];
         const double w = glw[si] * sv * en[2];
         i64 N[3], d[3];
-        fx_basis_normal<D>(P[0] + du, P[1] + dvv, ch, N, [&](int k, i64 kv) {
-          const u64 sgn = (u64)(kv >> 63);
-          Bs[k * SC::BST + threadIdx.x] = slice_bytes(((((u64)kv ^ sgn) - sgn) + 32) >> 6, kv < 0);
-        });
-        int ed;
-        fx_chord<D>(tXf, du, dvv, d, &ed);
         FxS nn[3];
         u64 wm;
         int ew;
-        fx_node_from_normal(N, ch.su + ch.sv + 1, w, nn, &wm, &ew);
-        if (ch.bad) ew = kFxBad + 1;
+        if (ch.fp64) {
+          double Nd[3];
+          self_node_fp64<D>(P[0] + du, P[1] + dvv, ch, Bs + threadIdx.x, SC::BST, Nd);
+          fx_make_node(Nd, w, nn, &wm, &ew);
+        } else {
+          int sn;
+          fx_basis_normal<D>(P[0] + du, P[1] + dvv, ch, N, &sn, [&](int k, i64 kv) {
+            const u64 sgn = (u64)(kv >> 63);
+            Bs[k * SC::BST + threadIdx.x] = slice_bytes(((((u64)kv ^ sgn) - sgn) + 32) >> 6, kv < 0);
+          });
+          fx_node_from_normal(N, sn + 1, w, nn, &wm, &ew);
+        }
+        int ed;
+        fx_chord<D>(tXf, du, dvv, d, &ed);
         // the target is the chart's value at the node: x - X(P + delta) = -dX
         const int S = ed + st + 1;
         const FxS nu[3] = {kps.kind == 3 ? nPx[0] : nn[0], kps.kind == 3 ? nPx[1] : nn[1],
