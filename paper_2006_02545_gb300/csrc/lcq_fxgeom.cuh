@@ -16,12 +16,14 @@
 
 namespace lcq {
 
-// A value as its high word and 28 bits of the low one, v = h 2^32 + 16 l (rounded: a truncation
-// has one sign in every term of a sum): sums of up to 22 cross products of such pairs, |v| <
-// 2^62.5, stay below 2^63.
+// A value as a high word and 28 bits of the low one, v = h 2^32 + 16 l, rounded.  A stored one has l
+// of either sign (fx_join28), the other factor l >= 0 (fx_28): of their product h h' + (h l' + l h') /
+// 2^28 the part l l' is left out, which has no one sign that a sum would add up.  Sums of up to
+// 63 cross products h l', |v| < 2^62, stay below 2^63.
 __device__ __forceinline__ u64 fx_join28(i64 v) {
   v += 8;
-  return ((u64)(v >> 32) << 32) | ((uint32_t)v >> 4);
+  const u64 h = (u64)(v >> 32) + ((uint32_t)v >> 31);
+  return (h << 32) | (uint32_t)((int)(uint32_t)v >> 4);
 }
 __device__ __forceinline__ FxS fx_28(FxS a) { return {a.h, (int)(((uint32_t)a.l + 4u) >> 3)}; }
 
@@ -102,12 +104,13 @@ struct FxChart {
 // the bounds 2^E_nm are reached at a corner only: where the high coefficients are not small
 // beside the low ones (patches too coarse for their degree), the scales are far above the chart.
 // Largest errors of 120 points, X against R and the normal against its length, fixed and
-// FP64: scale / root mean square of up to 3 (1280-patch ellipsoid, degree 6) 1.2e-16 and 4.5e-16,
-// 7e-17 and 1e-15; up to 20 (242-patch torus, degree 8) 2.5e-16 and 4.8e-16, 6e-16 and 2e-15; up
-// to 33 and 60 (18-patch twisted torus, degree 8) 4.9e-16 and 4.9e-16, 1.3e-15 and 9e-16; 60 to 90
-// (54-patch torus, degree 6) 6e-16 and 5e-16, 2.6e-15 and 1.7e-15; 900 to 2800 (18-patch torus, degree
-// 8) 1.1e-14 and 4e-16, 7e-14 and 5e-15.
-constexpr double kFxChartMax = 24.0;
+// FP64: scale / root mean square of up to 3 (1280-patch ellipsoid, degree 6) 4.5e-17 and 4.5e-16,
+// 6e-17 and 1e-15; up to 20 (242-patch torus, degree 8) 1e-16 and 4.8e-16, 4e-16 and 2e-15; up to 50
+// (110-patch torus, degree 8; 128 patches) 1.2e-16 and 4.1e-16, 5e-16 to 9e-16 and 1.6e-15; 60 to 90
+// (54-patch torus, degree 6) 3e-16 and 5e-16, 1.7e-15 and 1.7e-15; 220 to 760 (30 patches, degree 8)
+// 1e-15 and 5e-16, 1.2e-14 and 1.7e-15; 900 to 2800 (18 patches, degree 8) 5e-15 and 4e-16, 1e-13 and
+// 5e-15.
+constexpr double kFxChartMax = 48.0;
 
 // Sums over the coefficients i0, i0 + step, ...: s[k][c] of |coefficient| 2^E_nm of component c of
 // (X, X_u, X_v)[k], s[9 + k] of the squared coefficients.

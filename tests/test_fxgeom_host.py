@@ -224,8 +224,8 @@ COARSE = [W.torus(3, 3, 8), W.torus(3, 5, 8), W.torus(3, 9, 6), W.torus(3, 3, 10
 def test_errors(probe, i):
     """Where the fixed point is taken it is as near to the exact chart as the FP64 recurrences.
     Its roundings are half units 2^-59 of the scale, n + 3 (D + 1) of them in X (the products of the
-    sums and of the stored factors): with the scale at most 24 times the root mean square and the
-    roundings adding in quadrature 5 (3 (n + 3 D + 3))^(1/2) 2^-60 24 < 8 u at the largest degree;
+    sums and of the stored factors): with the scale at most 48 times the root mean square and the
+    roundings adding in quadrature 2.5 (3 (n + 3 D + 3))^(1/2) 2^-60 48 < 8 u at the largest degree;
     twice that for the normal, which takes both derivatives.  The basis carries 2^-57."""
     s = (RESOLVED + COARSE)[i]
     e, flagged = probe(s)
