@@ -525,6 +525,29 @@ __device__ void chart_taylor(double pu, double pv, const double* cf, double* scr
   __syncthreads();
 }
 
+// The chord dX(d) from the coefficients of chart_taylor: Horner in du inside Horner in dv.  Out of
+// line: the self rules take it only where the fixed-point chord is not exact enough.
+template <int D>
+__device__ __noinline__ void chart_chord(const double* tX, double du, double dv, double* dX) {
+  constexpr int n = (D + 1) * (D + 2) / 2;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double* t = tX + c * n;
+    double acc = 0.0;
+#pragma unroll
+    for (int j = D; j >= 0; --j) {
+      double in = 0.0;
+#pragma unroll
+      for (int i = D - j; i >= 0; --i) {
+        const int g = i + j;
+        in = fma(in, du, t[g * (g + 1) / 2 + j]);
+      }
+      acc = fma(acc, dv, in);
+    }
+    dX[c] = acc;
+  }
+}
+
 // f(idx, K_nm, dK_nm/du, dK_nm/dv) for every basis function at (u, v): the recurrences of
 // kw_geometry, for callers that need the derivatives one by one (the adjoint).
 template <int D, class F>

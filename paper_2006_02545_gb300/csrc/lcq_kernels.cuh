@@ -438,15 +438,15 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
   constexpr int n = SC::n;
   __shared__ double cf[3 * n];
   __shared__ SelfSeg sg[6];
-  __shared__ double Mm[5];  // M00 M01 M10 M11 detM
+  __shared__ double Mm[6];  // M00 M01 M10 M11 detM, smallest singular value of DX at the node
   __shared__ double P[2];
   __shared__ int nseg, total;
   __shared__ KernelParams kps;
   __shared__ int ord;
   __shared__ double nP[3];  // unit chart normal at the target node (S')
   __shared__ FxChart<D> ch;
-  __shared__ double tX[3 * n];  // Taylor coefficients of the chord at P, then in fixed point
-  __shared__ int st;
+  __shared__ double tX[3 * n];  // Taylor coefficients of the chord at P, in fixed point unless cfp
+  __shared__ int st, cfp;
   __shared__ int rowE[2];
   __shared__ cplx acc[n];
   extern __shared__ __align__(16) unsigned char ssm[];
@@ -496,6 +496,8 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
       Mm[2] = -R01 / detR;
       Mm[3] = R00 / detR;
       Mm[4] = 1.0 / detR;
+      const double tr = R00 + R11;
+      Mm[5] = 2.0 * detR / (tr + sqrt(fmax(tr * tr - 4.0 * detR, 0.0)));
       double Z[3][2];
       const double VX[3] = {0.0, 1.0, 0.0}, VY[3] = {0.0, 0.0, 1.0};
       for (int k = 0; k < 3; ++k) {
@@ -546,10 +548,12 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
       }
       fx_mant(mx, &st);
       st = max(st, -1000);
+      cfp = !(mx < 1e150 && ldexp(1.0, st) <= kFxChordMax * Mm[5]);
     }
     __syncthreads();
     u64* tXf = reinterpret_cast<u64*>(tX);
-    for (int e = threadIdx.x; e < 3 * n; e += blockDim.x) tXf[e] = fx_join28(fx_fix(tX[e], st));
+    if (!cfp)
+      for (int e = threadIdx.x; e < 3 * n; e += blockDim.x) tXf[e] = fx_join28(fx_fix(tX[e], st));
     for (int e = threadIdx.x; e < n; e += blockDim.x) acc[e] = {0.0, 0.0};
     const int tot = total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -584,16 +588,31 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
           });
           fx_node_from_normal(N, sn + 1, w, nn, &wm, &ew);
         }
-        int ed;
-        fx_chord<D>(tXf, du, dvv, d, &ed);
         // the target is the chart's value at the node: x - X(P + delta) = -dX
-        const int S = ed + st + 1;
+        FxS dm[3];
+        int E = 0;
+        bool ok;
+        double dX[3];
+        if (cfp) {
+          chart_chord<D>(tX, du, dvv, dX);
+          ok = fx_vector(-dX[0], -dX[1], -dX[2], dm, &E);
+        } else {
+          fx_chord<D>(tXf, du, dvv, d, &E);
+          E += st + 1;
+          ok = fx_vector_int(-d[0], -d[1], -d[2], E, dm, &E);
+        }
         const FxS nu[3] = {kps.kind == 3 ? nPx[0] : nn[0], kps.kind == 3 ? nPx[1] : nn[1],
                            kps.kind == 3 ? nPx[2] : nn[2]};
-        if (!fx_eval_int<false>(kps.fx, tab, -d[0], -d[1], -d[2], S, nu, wm, ew, &gk.re, &gk.im,
-                                nullptr, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f))
-          gk = fx_fallback(kps, fx_pack<false>(-d[0], S - 62), fx_pack<false>(-d[1], S - 62),
-                           fx_pack<false>(-d[2], S - 62), nu[0], nu[1], nu[2], wm, ew, 0.0, nullptr);
+        if (!ok || !fx_core<false>(kps.fx, tab, dm[0], dm[1], dm[2], E, nu, wm, ew, &gk.re, &gk.im,
+                                   nullptr, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f)) {
+          if (!cfp) {
+            int e2;
+            fx_chord<D>(tXf, du, dvv, d, &e2);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) dX[c] = fx_pack<false>(d[c], e2 + st - 61);
+          }
+          gk = fx_fallback(kps, -dX[0], -dX[1], -dX[2], nu[0], nu[1], nu[2], wm, ew, 0.0, nullptr);
+        }
       } else {
         for (int k = 0; k < n; ++k) Bs[k * SC::BST + threadIdx.x] = make_uint2(kZeroSlices, kZeroSlices);
       }

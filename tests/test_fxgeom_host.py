@@ -176,6 +176,56 @@ struct Probe {
   }
 };
 
+// Largest error of the chord of random Taylor coefficients (order g: up to rho^g) against |d| times the
+// smallest singular value of the linear part, over cases up to kFxChordMax; their number.
+template <int D>
+void chord(int cases, double rho, unsigned seed, double* out) {
+  constexpr int n = (D + 1) * (D + 2) / 2;
+  srand48(seed);
+  for (int it = 0; it < cases; ++it) {
+    double t[3 * n], mx = 0.0, a = 0.0, b = 0.0, c = 0.0;
+    for (int k = 0; k < 3; ++k) {
+      double sum = 0.0;
+      for (int g = 0; g <= D; ++g)
+        for (int j = 0; j <= g; ++j)
+          t[k * n + g * (g + 1) / 2 + j] = g == 0 ? 0.0 : (2.0 * drand48() - 1.0) * pow(rho, g);
+      for (int e = 1; e < n; ++e) sum += fabs(t[k * n + e]);
+      mx = fmax(mx, sum);
+      a += t[k * n + 1] * t[k * n + 1];
+      b += t[k * n + 1] * t[k * n + 2];
+      c += t[k * n + 2] * t[k * n + 2];
+    }
+    const double smin = sqrt((a + c - sqrt((a - c) * (a - c) + 4.0 * b * b)) / 2.0);
+    int st;
+    fx_mant(mx, &st);
+    if (!(ldexp(1.0, st) <= kFxChordMax * smin)) continue;
+    u64 x[3 * n];
+    for (int e = 0; e < 3 * n; ++e) x[e] = fx_join28(fx_fix(t[e], st));
+    const double r = pow(10.0, -9.0 * drand48()), du = (2.0 * drand48() - 1.0) * r,
+                 dv = (2.0 * drand48() - 1.0) * r;
+    i64 o[3];
+    int e;
+    fx_chord<D>(x, du, dv, o, &e);
+    LD err = 0;
+    for (int k = 0; k < 3; ++k) {
+      LD w = 0;
+      for (int g = 1; g <= D; ++g)
+        for (int j = 0; j <= g; ++j)
+          w += (LD)t[k * n + g * (g + 1) / 2 + j] * powl(du, g - j) * powl(dv, j);
+      err += powl(ldexpl(o[k], e + st - 61) - w, 2);
+    }
+    out[0] = fmax(out[0], (double)(sqrtl(err) / (sqrtl((LD)du * du + (LD)dv * dv) * smin)));
+    out[1] += 1.0;
+  }
+}
+extern "C" void chords(int d, int cases, double rho, unsigned seed, double* out) {
+  out[0] = out[1] = 0.0;
+  switch (d) {
+#define CHORD(D) case D: chord<D>(cases, rho, seed, out); break;
+    CHORD(1) CHORD(2) CHORD(3) CHORD(4) CHORD(5) CHORD(6) CHORD(7) CHORD(8) CHORD(9) CHORD(10)
+  }
+}
+
 extern "C" void probe(int d, const double* xyz, int points, unsigned seed, double* out) {
   switch (d) {
 #define CASE(D) case D: { Probe<D> p(xyz); p.run(points, seed, out); break; }
@@ -199,7 +249,8 @@ def probe(tmp_path_factory):
                     os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include"),
                     str(d / "p.cpp"), os.path.join(csrc, "lcq_tables.cpp"), "-o", str(d / "p.so")],
                    check=True)
-    f = C.CDLL(str(d / "p.so")).probe
+    lib = C.CDLL(str(d / "p.so"))
+    f = lib.probe
 
     def surface(s, patches=24, points=40):
         """Worst errors over some patches that the fixed point takes, and the share that it does not."""
@@ -211,6 +262,12 @@ def probe(tmp_path_factory):
             rows.append(o)
         rows = np.array(rows)
         return rows[:, :7].max(axis=0), rows[:, 7].mean()
+
+    def chords(deg, rho):
+        o = np.zeros(2)
+        lib.chords(deg, 2000, C.c_double(rho), deg, o.ctypes.data_as(C.c_void_p))
+        return o
+    surface.chords = chords
     return surface
 
 
@@ -236,3 +293,13 @@ def test_errors(probe, i):
     assert e[0] <= 8 * U and e[1] <= 16 * U and e[3] <= 16 * U, e / U
     assert e[2] <= 2.0 ** -56 and e[4] <= 2.0 ** -56, e * 2.0 ** 56
     assert e[0] <= 2 * e[5] and e[1] <= 2 * e[6], e / U
+
+
+@pytest.mark.parametrize("deg", range(1, 11))
+@pytest.mark.parametrize("rho", [0.2, 0.4])
+def test_chord(probe, deg, rho):
+    """The self rules' chord: n coefficients rounded to 2^-59 of the scale and as many powers of d, in
+    quadrature below 2^-56 |d| times the scale, which is at most 32 times the smallest singular
+    value of the tangents: 8 u, near the node as away from it."""
+    err, cases = probe.chords(deg, rho)
+    assert cases > 200 and err <= 8 * U, (err / U, cases)

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 from paper_2006_02545_gb300 import workloads as W
-from .gpu_helpers import run_gpu
+from .gpu_helpers import leaves_by_pair, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +85,38 @@ def test_group_size_with_targets_far_beyond_the_patch():
             assert np.array_equal(g["leaves"], runs[0]["leaves"])
     finally:
         c.close()
+
+
+def coarse_patch(deg):
+    """A patch of a torus far too coarse for its degree: its nodes take the FP64 recurrences."""
+    s = W.torus(3, 3, deg)
+    n = W.n_nodes(deg)
+    return W.Surface("coarse", s.deg[:1].copy(), s.node_off[:2].copy(),
+                     np.ascontiguousarray(s.xyz[:, :n]), {})
+
+
+@pytest.mark.parametrize("deg,kind,precision,eps", [(6, "CFIE", "fp64", 1e-7), (8, "S", "fp64", 1e-7),
+                                                    (10, "D", "fp64", 1e-6), (6, "Sp", "fp64", 1e-6),
+                                                    (8, "CFIE", "mixed", 1e-7), (6, "D", "mixed", 1e-5)])
+def test_coarse_patches(ctx, deg, kind, precision, eps):
+    """Adaptive, smooth-rule and self integration on a chart that the fixed-point scales do not fit,
+    against the oracle: leaf counts and the potential at the parity bars (the tiers of the mixed form
+    keep FP64 values on such a chart, and their own rounding floors)."""
+    s = coarse_patch(deg)
+    rng = np.random.default_rng(deg)
+    i = rng.integers(0, s.n_points, 9)
+    x = s.xyz[:, i] + rng.standard_normal((3, 9)) * 0.2
+    xs, ts = W.onsurface_targets(s)
+    x = np.ascontiguousarray(np.concatenate([x, xs[:, :5]], axis=1))
+    tn = np.concatenate([-np.ones(9, np.int64), ts[:5]])
+    nrm = rng.standard_normal((3, 14)) if kind == "Sp" else None
+    a, b = (1.0, -1j) if kind == "CFIE" else (1.0, 0.0)
+    kw = dict(max_depth=7, eps_loosen=10.0)
+    g = run_gpu(ctx, s, x, tn, kind, 1.0, eps, alpha=a, beta=b, precision=precision, tgt_normal=nrm, **kw)
+    assert g["status"] in (0, 4)
+    oc, uo = run_oracle(s, x, tn, kind, 1.0, eps, alpha=a, beta=b, sigma=g["sigma"], tgt_normal=nrm, **kw)
+    assert np.array_equal(g["q"], oc.q)
+    if precision == "fp64":
+        assert all(p == q for p, q, _ in leaves_by_pair(g, oc))
+    tol = 1e-10 if precision == "fp64" else eps
+    assert np.linalg.norm(g["u"] - uo) <= tol * np.linalg.norm(uo)
