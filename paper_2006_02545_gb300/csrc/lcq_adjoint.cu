@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kSumTThreads) k_far_sum_T(
         const double d0 = sx[0][i] - X[0], d1 = sx[1][i] - X[1], d2 = sx[2][i] - X[2];
         cplx k;
         if (!fx_eval<true>(kf, tab, d0, d1, d2, m, w, ew, &k.re, &k.im, nullptr, 0.0f, 0.0f, 0.0f,
-                           0.0f, 0.0f))
+                           0.0f, 0.0f, &kq->fx))
           k = fx_fallback(*kq, d0, d1, d2, m[0], m[1], m[2], w, ew, 0.0, nullptr);
         // conj(k) * g
         re = fma(k.re, sg[i].re, re);

@@ -7,13 +7,14 @@
 // on a scale that is known beforehand (or one exponent per pair), where FP64 has 53.
 //
 // The value is written without the node's area element in it:
-//   K~ = W e^{-ki r} e^{i kr r} (A + iB) / r^2,   W = Jw / (4 pi),
-//   A = Re(beta) r + c (Re(alpha) + p r),  B = Im(beta) r + c (Im(alpha) + q r),
-//   c = n.d / r (n the unit normal, d = x - X),
-//   p = Re(alpha) ki + Im(alpha) kr,  q = Im(alpha) ki - Re(alpha) kr,
-// which is alpha (1 - ikr) n.d / r^2 + beta times W e^{ikr} / r, with every term bounded by
-// its own constant times max(1, r), so that A and B are fixed-point sums at one exponent per
-// pair.  The single layer alone is W e^{ikr} / r.
+//   K~ = W e^{-ki r} e^{i th} (A + iB) / r^2,   W = Jw / (4 pi),  th = kr r,
+//   A = T + th U + Re(beta) r + ki r T,  B = U - th T + Im(beta) r + ki r U,
+//   T = Re(alpha) c,  U = Im(alpha) c,  c = n.d / r  (n the unit normal, d = x - X),
+// which is alpha (1 - ikr) n.d / r^2 + beta times W e^{ikr} / r.  c, T and U are brought to full length
+// and A and B summed at the exponent of the largest term.  Below th = 2 pi / 256, where sin th ~ th and
+// g = sin th - th cos th ~ th^3 / 3, these come from their series to full length and every term has its
+// own exponent (fx_small_value), so that each part keeps its digits down to th = 0.  The single layer
+// alone is W e^{ikr} / r.
 //
 // Host and device code alike: the arithmetic is plain 64-bit integers, so a host program can
 // compare it with higher precision; only the start of the reciprocal square root differs.
@@ -24,8 +25,10 @@
 
 #ifdef __CUDACC__
 #define LCQ_HD __host__ __device__ __forceinline__
+#define LCQ_HD_NOINLINE static __host__ __device__ __noinline__
 #else
 #define LCQ_HD inline
+#define LCQ_HD_NOINLINE static
 #endif
 
 namespace lcq {
@@ -65,10 +68,12 @@ LCQ_HD i64 fx_smul_sl(FxS a, FxS b) {
   const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h);
   return fx_swide(a.h, b.h) * (1ll << K) + (t >> (31 - K));
 }
-// (a b + c d) / 2^61, |a|, |c| < 2^62.3, |b|, |d| < 2^61
+// (a b + c d) / 2^61, |a|, |c| < 2^62.5, b^2 + d^2 <= 2^122, the products of the low words included
 LCQ_HD i64 fx_dot2(FxS a, FxS b, FxS c, FxS d) {
-  const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h) + fx_swide(c.h, d.l) + fx_swide(c.l, d.h);
-  return ((fx_swide(a.h, b.h) + fx_swide(c.h, d.h)) << 3) + (t >> 28);
+  const i64 l = fx_swide(a.l, b.l) + fx_swide(c.l, d.l);
+  const i64 t = fx_swide(a.h, b.l) + fx_swide(a.l, b.h) + fx_swide(c.h, d.l) + fx_swide(c.l, d.h) +
+                (l >> 31);
+  return ((fx_swide(a.h, b.h) + fx_swide(c.h, d.h)) << 3) + ((t + (1 << 27)) >> 28);
 }
 
 LCQ_HD u64 fx_bits(double x) {
@@ -116,19 +121,33 @@ LCQ_HD i64 fx_fix(double x, int e) {
   return s < 0 ? m * 2 : fx_sra(m, s);
 }
 
+// A constant x = m 2^(e - 62), |m| < 2^62 with the leading bit set.
+struct FxConst {
+  FxS m;
+  int e;
+};
+LCQ_HD FxConst fx_const(double x) {
+  FxConst c;
+  c.m = fx_split(fx_mant(x, &c.e));
+  return c;
+}
+
 // Constants of a kernel (one patch's, or one launch's): kind 0: S, else the general form.
 struct FxKernel {
-  u64 kt;        // |kr| / (2 pi) = kt 2^(ek - 62)
-  u64 kd;        // ki / ln 2 = kd 2^(ed - 62), 0: none
-  FxS ar, ai;    // alpha 2^(62 - ea)
-  FxS p, q;      // (p, q) 2^(62 - ep)
-  FxS br, bi;    // beta 2^(62 - eb)
-  int ek, ed, ea, ep, eb;
-  int neg;       // kr < 0: the phase's sign
-  int single;    // the single layer alone (alpha = 0, beta = 1)
-  int cplx;      // Im(alpha) or p not zero
-  int has;       // 1: Re(beta) not zero, 2: Im(beta) not zero, 4: Re(alpha) = 1
+  u64 kt;                // |kr| / (2 pi) = kt 2^(ek - 62)
+  u64 ku;                // |kr| = ku 2^(eu - 62), 0: none
+  u64 kd;                // ki / ln 2 = kd 2^(ed - 62), 0: none
+  FxConst ar, ai;        // alpha
+  FxConst p, q;          // Re(alpha) ki, Im(alpha) ki
+  FxConst br, bi;        // beta
+  int ek, eu, ed;
+  int neg;               // kr < 0: the phase's sign
+  int single;            // the single layer alone (alpha = 0, beta = 1)
+  int has;               // bits kFxBr ... below: the terms that are not zero
+  int many;              // 1: more than two of T, U, ki T and the beta terms
 };
+constexpr int kFxBr = 1, kFxBi = 2, kFxAr = 4, kFxAi = 8, kFxP = 16, kFxQ = 32;
+constexpr int kFxUnit = 64;  // Re(alpha) = 1
 
 // kind, k, alpha, beta as KernelParams holds them (kind 0: S, 1 and 3: D form, 2: CFIE).
 LCQ_HD FxKernel fx_kernel(int kind, double kr, double ki, double ar, double ai, double br,
@@ -145,6 +164,8 @@ LCQ_HD FxKernel fx_kernel(int kind, double kr, double ki, double ar, double ai, 
   int e;
   // kr / (2 pi) and ki / ln 2 to 58 bits: 2^64 / (2 pi) and 2^62 / ln 2 times the mantissas
   u64 m = (u64)fx_mant(fabs(kr), &e);
+  f.ku = m;
+  f.eu = e;
   m = fx_umul(m, 0x28be60db9391054aull);
   for (f.ek = e; m != 0 && m < (1ull << 61); m <<= 1) --f.ek;
   f.kt = m;
@@ -152,28 +173,20 @@ LCQ_HD FxKernel fx_kernel(int kind, double kr, double ki, double ar, double ai, 
   m = fx_umul(m, 0x5c551d94ae0bf85eull);
   for (f.ed = e + 2; m != 0 && m < (1ull << 61); m <<= 1) --f.ed;
   f.kd = m;
-  const double p = ar * ki + ai * kr, q = ai * ki - ar * kr;
-  int e1, e2;
+  const double p = ar * ki, q = ai * ki;
   // a product of the constants that overflows: no phase counts as covered, so that every pair
   // takes the FP64 kernel
   if (!(fabs(p) < 1e300 && fabs(q) < 1e300)) f.ek = 100000;
-  fx_mant(ar, &e1);
-  fx_mant(ai, &e2);
-  f.ea = fx_max(e1, e2);
-  f.ar = fx_split(fx_fix(ar, f.ea));
-  f.ai = fx_split(fx_fix(ai, f.ea));
-  fx_mant(p, &e1);
-  fx_mant(q, &e2);
-  f.ep = fx_max(e1, e2);
-  f.p = fx_split(fx_fix(p, f.ep));
-  f.q = fx_split(fx_fix(q, f.ep));
-  fx_mant(br, &e1);
-  fx_mant(bi, &e2);
-  f.eb = fx_max(e1, e2);
-  f.br = fx_split(fx_fix(br, f.eb));
-  f.bi = fx_split(fx_fix(bi, f.eb));
-  f.cplx = ai != 0.0 || p != 0.0;
-  f.has = (br != 0.0 ? 1 : 0) | (bi != 0.0 ? 2 : 0) | (ar == 1.0 && ai == 0.0 ? 4 : 0);
+  f.ar = fx_const(ar);
+  f.ai = fx_const(ai);
+  f.p = fx_const(p);
+  f.q = fx_const(q);
+  f.br = fx_const(br);
+  f.bi = fx_const(bi);
+  f.has = (br != 0.0 ? kFxBr : 0) | (bi != 0.0 ? kFxBi : 0) | (ar != 0.0 ? kFxAr : 0) |
+          (ai != 0.0 ? kFxAi : 0) | (p != 0.0 ? kFxP : 0) | (q != 0.0 ? kFxQ : 0) |
+          (ar == 1.0 ? kFxUnit : 0);
+  f.many = (ar != 0.0) + (ai != 0.0) + (p != 0.0 || q != 0.0) + (br != 0.0 || bi != 0.0) > 2;
   return f;
 }
 
@@ -316,15 +329,133 @@ LCQ_HD FxRoot fx_root(FxS D0, FxS D1, FxS D2) {
   return o;
 }
 
+// Zeros above the leading bit of |v|, by the high word: at most 32 (a shift below 32 bits is two
+// instructions, and no value here means anything 2^-32 below its scale).
+LCQ_HD int fx_clz_hi(i64 v) {
+  const int h = (int)(v >> 32);
+#ifdef __CUDA_ARCH__
+  return __clz(h ^ (h >> 31));
+#else
+  return (h ^ (h >> 31)) == 0 ? 32 : __builtin_clz((unsigned)(h ^ (h >> 31)));
+#endif
+}
+// v 2^e brought to full length, 2^62 <= |v| < 2^63, or by 31 bits.
+LCQ_HD void fx_full(i64& v, int& e) {
+  const int k = fx_clz_hi(v) - 1;
+  v = (i64)((u64)v << (k & 31));
+  e -= k;
+}
+
+// A number m 2^(e - 62) of a sum, and the sum of two.
+struct FxTerm {
+  i64 m;
+  int e;
+};
+LCQ_HD FxTerm fx_plus(FxTerm a, FxTerm b) {  // |m| below 2^61.9 and 2^60
+  const int e = fx_max(a.e, b.e);
+  return {fx_sra(a.m, e - a.e) + fx_sra(b.m, e - b.e), e};
+}
+// a b, the factors' magnitudes below 2^62 (the product's below 2^61)
+LCQ_HD FxTerm fx_times(FxS a, int ea, FxS b, int eb) { return {fx_smul_sl<1>(a, b), ea + eb + 1}; }
+
+// sin th and, if g is asked for, g = sin th - th cos th for th = t 2^(et - 62), 2^58 <= t < 2^62, th <
+// 2 pi / 256, to full length with relative errors below 2^-56 (the series' next terms are below 2^-61):
+// sin = th (1 - z / 6 + z^2 / 120 - z^3 / 5040), g = th z (1 / 3 - z / 30 + z^2 / 840 - z^3 / 45360),
+// z = th^2.
+LCQ_HD void fx_small(u64 t, int et, FxTerm* sn, FxTerm* g) {
+  const int l = fx_clz(t) - 2;
+  t <<= l;
+  et -= l;
+  const u64 zm = fx_umul(t, t);                          // z = zm 2^(2 et - 60), in [2^58, 2^60)
+  const u64 z = zm >> fx_min(-(2 * et + 4), 63);         // unit 2^-64, below 2^53.4
+  const uint32_t y = (uint32_t)(z >> 22);                // unit 2^-42
+  const u64 z9 = z << 9;                                 // unit 2^-73
+  uint32_t c = 0x88888889u - (uint32_t)(fx_wide(y, 0xd00d00d0u) >> 48);   // 2^38 / 120, 2^44 / 5040
+  u64 a = 0x2aaaaaaaaaaaaaabull - (fx_wide(y, c) >> 16);                  // 2^64 / 6
+  u64 m = fx_umul(t, (1ull << 62) - (fx_umul(z9, a) >> 11));              // [2^58.9, 2^60)
+  *sn = {(i64)(m << 2), et};
+  if (g == nullptr) return;
+  c = 0x9c09c09cu - (uint32_t)(fx_wide(y, 0xb8ef1d2bu) >> 48);            // 2^41 / 840, 2^47 / 45360
+  a = 0x2222222222222222ull - (fx_wide(y, c) >> 17);                      // 2^66 / 30
+  a = 0x2aaaaaaaaaaaaaabull - (fx_umul(z9, a) >> 12);                     // 2^63 / 3
+  m = fx_umul(fx_umul(t, zm << 2) << 2, a);              // g = m 2^(3 et - 61), in [2^56.3, 2^59.5)
+  const int k = fx_clz(m) - 2;
+  *g = {(i64)(m << k), 3 * et + 1 - k};
+}
+
+// The value where th = |kr| r < 2 pi / 256, from the cosine cs of th (sg its and the sine's signs), h and
+// eg of W e^{-ki r} / r = h 2^(eg) (fx_core), and n.d = nd 2^(E - 60): the sine and g by their series, and
+// every term at its own exponent.  Out of line: pairs nearer than a 256th of a wavelength.
+template <bool INT>
+LCQ_HD_NOINLINE void fx_small_value(const FxKernel& K, u64 RI, u64 R, int E, u64 cs, u64 h, int eg, i64 nd,
+                                    double* re, double* im) {
+  const u64 th = fx_umul(R, K.ku) << 1;                 // kr r = th 2^(et - 62), [2^59, 2^61.8)
+  const int et = E + K.eu + 1;
+  const i64 mt = -(i64)K.neg;
+  FxTerm sv, g;
+  fx_small(th, et, &sv, K.single ? nullptr : &g);
+  if (K.single) {
+    *re = fx_pack<INT>((i64)fx_umul(cs, h << 2), eg);
+    *im = fx_pack<INT>(((i64)fx_umul((u64)sv.m, h << 2) ^ mt) - mt, eg + sv.e);
+    return;
+  }
+  // W / r^2 to full length: G 2^(eG - 63)
+  u64 G = fx_umul(RI, h << 2);                          // W / r^2 = G 2^(eg - E + 1)
+  const int lG = fx_clz(G) - 1;
+  G <<= lG;
+  const int eG = eg - E + 64 - lG;
+  const int lc = fx_min(fx_clz((u64)(nd ^ (nd >> 63))) - 2, 61);
+  const FxS c = fx_split(fx_smul_sl<2>(fx_split(nd << lc), fx_split((i64)RI)));
+  const int ec = 3 - lc;                                // c = n.d / r = . 2^(ec - 62)
+  sv.m = (sv.m ^ mt) - mt;
+  g.m = (g.m ^ mt) - mt;
+  const FxS ct = fx_split((i64)cs), st = fx_split(sv.m), gs = fx_split(g.m), Rs = fx_split((i64)R);
+  // f = cos + th sin at the exponent 1
+  const FxS f = fx_split((i64)(cs >> 1) +
+                         fx_sra(fx_smul_sl<1>(fx_split((i64)th), fx_split(sv.m ^ mt)), -et - sv.e));
+  const FxTerm none = {0, kFxZero};
+  FxTerm A = none, B = none, vr = none, vi = none;
+  if (K.has & kFxBr) A = fx_times(K.br.m, K.br.e, Rs, E);
+  if (K.has & kFxBi) B = fx_times(K.bi.m, K.bi.e, Rs, E);
+  if (K.has & kFxP) {
+    const FxTerm v = fx_times(K.p.m, K.p.e, Rs, E);
+    A = fx_plus(A, fx_times(fx_split(v.m), v.e, c, ec));
+  }
+  if (K.has & kFxQ) {
+    const FxTerm v = fx_times(K.q.m, K.q.e, Rs, E);
+    B = fx_plus(B, fx_times(fx_split(v.m), v.e, c, ec));
+  }
+  if (K.has & kFxAr) {
+    const FxTerm T = fx_times(K.ar.m, K.ar.e, c, ec);
+    const FxS m = fx_split(T.m);
+    vr = fx_times(m, T.e, f, 1);
+    vi = fx_times(m, T.e, gs, g.e);
+  }
+  if (K.has & kFxAi) {
+    const FxTerm U = fx_times(K.ai.m, K.ai.e, c, ec);
+    const FxS m = fx_split(U.m), mn = {-m.h, -m.l};
+    vr = fx_plus(vr, fx_times(mn, U.e, gs, g.e));
+    vi = fx_plus(vi, fx_times(m, U.e, f, 1));
+  }
+  const FxS Am = fx_split(A.m), Bm = fx_split(B.m), Bn = {-Bm.h, -Bm.l};
+  vr = fx_plus(fx_plus(vr, fx_times(Am, A.e, ct, 0)), fx_times(Bn, B.e, st, sv.e));
+  vi = fx_plus(fx_plus(vi, fx_times(Am, A.e, st, sv.e)), fx_times(Bm, B.e, ct, 0));
+  // . 2^(e - 62) G 2^(eG - 63)
+  const FxS Gs = fx_split((i64)G);
+  *re = fx_pack<INT>(fx_smul(fx_split(vr.m), Gs), vr.e + eG - 61);
+  *im = fx_pack<INT>(fx_smul(fx_split(vi.m), Gs), vi.e + eG - 61);
+}
+
 // The kernel value of one pair from d = x - X = D 2^(E - 62), 2^61 <= max |D_c| < 2^62.  False
 // (and nothing written) for arguments that it does not cover: a phase above 2^22 turns, a decay
 // above 2^9 halvings, a node that is not finite (ew above kFxBad).  With env the rounding
 // envelope |G| Jw (eb + ea |1 - ikr| R / r^2) in FP32 (fk: |kr|, fki: ki, feb = eb, feaR = ea R,
 // fw = W in FP32).
+// Km: K in memory, for a caller that holds K in registers (the call of fx_small_value takes its address).
 template <bool INT>
 LCQ_HD bool fx_core(const FxKernel& K, const FxTables& tab, FxS D0, FxS D1, FxS D2, int E,
                     const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
-                    float fki, float feb, float feaR, float fw) {
+                    float fki, float feb, float feaR, float fw, const FxKernel* Km = nullptr) {
   const int sh = E + K.ek + 8;
   if (sh > 30 || ew > kFxBad) return false;
   const FxRoot rt = fx_root(D0, D1, D2);
@@ -370,39 +501,72 @@ LCQ_HD bool fx_core(const FxKernel& K, const FxTables& tab, FxS D0, FxS D1, FxS 
     if (fki != 0.0f) g *= expf(-fki * fr);
     *env = g * (feb + feaR * fab * fri * fri);
   }
+  const int et = E + K.eu + 1;
+  const bool small = et <= -2 && ph < (1ull << 56) && K.ku != 0;
   const i64 ma = -(i64)(sg & 1), mb = -(i64)(sg >> 1);
+  i64 nd = 0;
+  if (!K.single) {
+    const i64 n01 = fx_swide(n[0].h, D0.l) + fx_swide(n[0].l, D0.h) + fx_swide(n[1].h, D1.l) +
+                    fx_swide(n[1].l, D1.h);
+    const i64 n2 = fx_swide(n[2].h, D2.l) + fx_swide(n[2].l, D2.h);
+    nd = fx_swide(n[0].h, D0.h) + fx_swide(n[1].h, D1.h) + fx_swide(n[2].h, D2.h) +
+         (n01 >> 31) + (n2 >> 31);                      // n.d 2^(60 - E)
+  }
+  if (small) {
+    fx_small_value<INT>(Km ? *Km : K, RI, R, E, cs, h, eg, nd, re, im);
+    return true;
+  }
   if (K.single) {
     const u64 a = fx_umul(cs, h << 2), b = fx_umul(sn, h << 2);   // unit 2^eg
     *re = fx_pack<INT>(((i64)a ^ ma) - ma, eg);
     *im = fx_pack<INT>(((i64)b ^ mb) - mb, eg);
     return true;
   }
-  const u64 g = fx_umul(RI, h << 2);                    // W / r^2 = g 2^(eg - E + 1)
-  const FxS ec = fx_split((i64)fx_umul(cs, g << 2) ^ ma);   // e^{ikr} W / r^2, the same unit
-  const FxS es = fx_split((i64)fx_umul(sn, g << 2) ^ mb);
-  // c = n.d / r, unit 2^-62
-  const i64 n01 = fx_swide(n[0].h, D0.l) + fx_swide(n[0].l, D0.h) + fx_swide(n[1].h, D1.l) +
-                  fx_swide(n[1].l, D1.h);
-  const i64 n2 = fx_swide(n[2].h, D2.l) + fx_swide(n[2].l, D2.h);
-  const i64 nd = fx_swide(n[0].h, D0.h) + fx_swide(n[1].h, D1.h) + fx_swide(n[2].h, D2.h) +
-                 (n01 >> 31) + (n2 >> 31);              // n.d 2^(60 - E)
-  const FxS c = fx_split(fx_smul(fx_split(nd << 2), fx_split((i64)RI)) << 3);
-  // A and B, unit 2^(eA - 60)
+  u64 g = fx_umul(RI, h << 2);                          // W / r^2 = g 2^(eg - E + 1)
+  const int lg = fx_clz_hi((i64)g) - 1;                 // g >= 2^56
+  g <<= lg & 31;                                        // [2^62, 2^63)
+  const FxS ec = fx_split((i64)fx_umul(cs, g) ^ ma);    // e^{ikr} W / r^2, unit 2^(eg - E + 3 - lg)
+  const FxS es = fx_split((i64)fx_umul(sn, g) ^ mb);
+  // c = n.d / r to full length, T = Re(alpha) c = . 2^(eT - 63)
+  const int lc = fx_clz_hi(nd) - 2;                     // |nd| < 2^61
+  i64 Tm = fx_smul_sl<3>(fx_split((i64)((u64)nd << (lc & 31))), fx_split((i64)RI));
+  int eT = 3 - lc;
+  fx_full(Tm, eT);
+  const FxS c = fx_split(Tm);
+  const int e0 = eT;
+  if (!(K.has & kFxUnit)) {  // (branches on the constants are uniform)
+    Tm = fx_smul_sl<2>(K.ar.m, c);
+    eT += K.ar.e;
+    fx_full(Tm, eT);
+  }
   const FxS Rs = fx_split((i64)R);
-  const int eb = K.eb + E, ep = K.ep + E;
-  const int eA = fx_max(K.ea, fx_max(eb, ep));
-  const int sb = eA - eb, sa = eA - K.ea, sp = eA - ep;
-  // (branches on the constants are uniform; alpha = 1 has ea = 1)
-  i64 A = fx_sra((K.has & 4) ? ((i64)c.h << 29) + (c.l >> 2) : fx_smul(K.ar, c), sa);
-  i64 B = fx_sra(fx_smul(fx_split(fx_smul(K.q, Rs) << 2), c), sp);
-  if (K.has & 1) A += fx_sra(fx_smul(K.br, Rs), sb);
-  if (K.has & 2) B += fx_sra(fx_smul(K.bi, Rs), sb);
-  if (K.cplx) {
-    A += fx_sra(fx_smul(fx_split(fx_smul(K.p, Rs) << 2), c), sp);
-    B += fx_sra(fx_smul(K.ai, c), sa);
+  const i64 mt = -(i64)K.neg;
+  const FxS ts = fx_split(((i64)(fx_umul(R, K.ku) << 1) ^ mt) - mt);   // kr r = . 2^(et - 62)
+  // A and B, the sums beside cos and sin, unit 2^(eA - 61) of the largest term
+  const int ebr = K.br.e + E, ebi = K.bi.e + E;
+  int eA = fx_max(fx_max(eT, eT + et), fx_max(ebr, ebi));
+  int eU = kFxZero, ep = kFxZero, eq = kFxZero;
+  i64 U = 0;
+  if (K.has & (kFxAi | kFxP | kFxQ)) {
+    U = fx_smul_sl<2>(K.ai.m, c);
+    eU = e0 + K.ai.e;
+    fx_full(U, eU);
+    ep = K.p.e + E + e0 + 1;
+    eq = K.q.e + E + e0 + 1;
+    eA = fx_max(fx_max(eA, fx_max(eU, eU + et)), fx_max(ep, eq)) + K.many;
+  }
+  i64 A = (fx_sra(Tm, eA - eT + 1) + 1) >> 1;
+  i64 B = -fx_sra(fx_smul(ts, fx_split(Tm)), eA - eT - et);
+  if (K.has & kFxBr) A += fx_sra(fx_smul_sl<1>(K.br.m, Rs), eA - ebr);
+  if (K.has & kFxBi) B += fx_sra(fx_smul_sl<1>(K.bi.m, Rs), eA - ebi);
+  if (K.has & (kFxAi | kFxP | kFxQ)) {
+    A += (fx_sra(fx_smul_sl<1>(ts, fx_split(U)), eA - eU - et) + 1) >> 1;
+    B += (fx_sra(U, eA - eU + 1) + 1) >> 1;
+    A += fx_sra(fx_smul(fx_split(fx_smul(K.p.m, Rs) << 1), c), eA - ep);
+    B += fx_sra(fx_smul(fx_split(fx_smul(K.q.m, Rs) << 1), c), eA - eq);
   }
   const FxS As = fx_split(A), Bs = fx_split(B), Bn = {-Bs.h, -Bs.l};
-  const int ev = eA + eg - E + 2;
+  const int ev = eA + eg - E + 3 - lg;
   *re = fx_pack<INT>(fx_dot2(As, ec, Bn, es), ev);
   *im = fx_pack<INT>(fx_dot2(As, es, Bs, ec), ev);
   return true;
@@ -442,11 +606,11 @@ LCQ_HD bool fx_vector_int(i64 d0, i64 d1, i64 d2, int S, FxS* D, int* E) {
 template <bool INT>
 LCQ_HD bool fx_eval(const FxKernel& K, const FxTables& tab, double d0, double d1, double d2,
                     const FxS* n, u64 w, int ew, double* re, double* im, float* env, float fk,
-                    float fki, float feb, float feaR, float fw) {
+                    float fki, float feb, float feaR, float fw, const FxKernel* Km = nullptr) {
   FxS D[3];
   int E;
   return fx_vector(d0, d1, d2, D, &E) &&
-         fx_core<INT>(K, tab, D[0], D[1], D[2], E, n, w, ew, re, im, env, fk, fki, feb, feaR, fw);
+         fx_core<INT>(K, tab, D[0], D[1], D[2], E, n, w, ew, re, im, env, fk, fki, feb, feaR, fw, Km);
 }
 template <bool INT>
 LCQ_HD bool fx_eval_int(const FxKernel& K, const FxTables& tab, i64 d0, i64 d1, i64 d2, int S,

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kFarThreads) k_far_sum(const double* __restric
       const double d0 = x0 - fx_double(a.x), d1 = x1 - fx_double(a.y), d2 = x2 - fx_double(b.x);
       cplx g;
       if (!fx_eval<true>(kf, tab, d0, d1, d2, n, d.x, (int)d.y, &g.re, &g.im, nullptr, 0.0f, 0.0f,
-                         0.0f, 0.0f, 0.0f))
+                         0.0f, 0.0f, 0.0f, &kt->fx))
         g = fx_fallback(*kt, d0, d1, d2, n[0], n[1], n[2], d.x, (int)d.y, 0.0, nullptr);
       const double sr = fx_double(s[4][k].x), si = fx_double(s[4][k].y);
       re = fma(g.re, sr, re);

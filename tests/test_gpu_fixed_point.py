@@ -120,3 +120,39 @@ def test_coarse_patches(ctx, deg, kind, precision, eps):
         assert all(p == q for p, q, _ in leaves_by_pair(g, oc))
     tol = 1e-10 if precision == "fp64" else eps
     assert np.linalg.norm(g["u"] - uo) <= tol * np.linalg.norm(uo)
+
+
+@pytest.mark.parametrize("deg", [3, 6])
+@pytest.mark.parametrize("kind", ["S", "D", "Sp"])
+def test_low_frequency_imaginary_part(ctx, deg, kind):
+    """The imaginary part at |k| r near zero, far below the real one, through generation, apply and
+    adjoint with real densities: S ~ k against the oracle; D and S' ~ k^3, whose ratio at two wave
+    numbers is the cube of theirs up to (k r)^2 < 1e-11."""
+    import torch
+    from paper_2006_02545_gb300 import lcq
+    s = W.ellipsoid(1, deg, axes=(1.0, 1.2, 0.9))
+    xs, ts = W.onsurface_targets(s)
+    x = np.ascontiguousarray(np.concatenate([xs[:, ::3] * 1.05, xs], axis=1))
+    tn = np.concatenate([-np.ones(xs[:, ::3].shape[1], np.int64), ts])
+    nrm = np.random.default_rng(3).standard_normal(x.shape) if kind == "Sp" else None
+    sig = np.random.default_rng(1).standard_normal(s.n_points) + 0j
+    gt = np.random.default_rng(2).standard_normal(x.shape[1]) + 0j
+    fn = {"S": lcq.apply_corrected_S, "D": lcq.apply_corrected_D, "Sp": lcq.apply_corrected_Sp}[kind]
+    parts = []
+    ks = (1e-12,) if kind == "S" else (1e-6, 1e-8)
+    for k in ks:
+        g = run_gpu(ctx, s, x, tn, kind, k, 1e-7, tgt_normal=nrm)
+        assert g["status"] == 0
+        u = fn(ctx, g["ds"], g["near"], g["corr"], torch.from_numpy(sig).cuda(), x.shape[1])
+        z = lcq.apply_adjoint(ctx, g["ds"], g["near"], g["corr"], torch.from_numpy(gt).cuda())
+        assert ctx.sync(60000) == 0
+        parts.append((u.cpu().numpy().imag, z.cpu().numpy().imag))
+    if kind == "S":
+        oc, uo = run_oracle(s, x, tn, kind, ks[0], 1e-7, sigma=sig)
+        u, z = parts[0]
+        assert np.linalg.norm(u - uo.imag) <= 1e-10 * np.linalg.norm(uo.imag)
+        # <g, A sigma> = <A^H g, sigma>, the imaginary part
+        assert abs(gt.real @ u + z @ sig.real) <= 1e-10 * np.linalg.norm(u) * np.linalg.norm(gt)
+    else:
+        for a, b in zip(*parts):
+            assert np.linalg.norm(a * (ks[1] / ks[0]) ** 3 - b) <= 1e-10 * np.linalg.norm(b)
