@@ -141,6 +141,11 @@ __global__ void __launch_bounds__(kSumTThreads) k_far_sum_T(
         sx[k][threadIdx.x] = dv.tgt[k * dv.NT + t];
         if (sp) sn[k][threadIdx.x] = fx_join(fx_split(fx_fix(-dv.tnrm[k * dv.NT + t], 0)));
       }
+      if (sp)  // a normal that is not finite: a NaN, passed on by the differences
+        for (int k = 0; k < 3; ++k) {
+          const double nk = dv.tnrm[k * dv.NT + t];
+          if (!isfinite(nk)) sx[0][threadIdx.x] = nk - nk;
+        }
       sg[threadIdx.x] = g[t];
       stp[threadIdx.x] = dv.tpatch[t];
       sgr[threadIdx.x] = tgroup ? tgroup[t] : 0;

@@ -193,11 +193,13 @@ struct TgtAdaptive {  // targets of a union-tree node: local ids -> pairs -> tar
 };
 
 // Unit normal of a target (S') as fx_eval takes a node's, negated: S' is the double-layer
-// form with -n_x in the place of the source's normal.
+// form with -n_x in the place of the source's normal.  A normal that is not finite (the caller's of
+// length zero) has no integers for it: it makes the position xrel a NaN, which every form passes on.
 template <class TA>
-__device__ __forceinline__ void load_fx_normal(const TA& ta, int i, const double* xrel, u64* out) {
+__device__ __forceinline__ void load_fx_normal(const TA& ta, int i, double* xrel, u64* out) {
   double n[3];
   ta.nrm(i, xrel, n);
+  if (!isfinite(n[0] + n[1] + n[2])) xrel[0] = __longlong_as_double(0x7ff8000000000000ll);
 #pragma unroll
   for (int c = 0; c < 3; ++c) out[c] = fx_join(fx_split(fx_fix(-n[c], 0)));
 }
@@ -542,9 +544,11 @@ __device__ __forceinline__ void block_moments_form(
       ta.pos(t0 + threadIdx.x, xp);
       bool near = fixed && !GEO64;
 #pragma unroll
+      for (int c = 0; c < 3; ++c) xp[c] -= cen[c];
+      if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
+#pragma unroll
       for (int c = 0; c < 3; ++c) {
         int e;
-        xp[c] -= cen[c];
         fx_mant(xp[c], &e);
         near = near && e < S;
       }
@@ -554,7 +558,6 @@ __device__ __forceinline__ void block_moments_form(
         else tx[3 * threadIdx.x + c] = xp[c];
       }
       te[threadIdx.x] = !near;
-      if (kp.kind == 3) load_fx_normal(ta, t0 + threadIdx.x, xp, tn + 3 * threadIdx.x);
     }
   };
   if (T <= C::TT) {

@@ -108,8 +108,13 @@ __global__ void __launch_bounds__(kFarThreads) k_far_sum(const double* __restric
     x0 = tgt[t];
     x1 = tgt[NT + t];
     x2 = tgt[2 * NT + t];
-    if (tnrm)  // S': the double-layer form with -n_x in the place of the source's normal
-      for (int c = 0; c < 3; ++c) nx[c] = fx_split(fx_fix(-tnrm[c * NT + t], 0));
+    if (tnrm) {  // S': the double-layer form with -n_x in the place of the source's normal
+      for (int c = 0; c < 3; ++c) {
+        const double n = tnrm[c * NT + t];
+        nx[c] = fx_split(fx_fix(-n, 0));
+        if (!isfinite(n)) x0 = n - n;  // a NaN, passed on by the differences
+      }
+    }
     const int tp = tpatch[t];
     if (tp >= 0) {
       skip0 = src_off[tp];

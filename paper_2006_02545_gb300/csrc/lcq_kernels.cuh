@@ -534,6 +534,7 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
     const FxTables tab = fx_tables();
     FxS nPx[3];  // S': the source's normal replaced by -n_x
     for (int c = 0; c < 3; ++c) nPx[c] = fx_split(fx_fix(-nP[c], 0));
+    const bool nbad = kps.kind == 3 && !isfinite(nP[0] + nP[1] + nP[2]);
     const int nent = total / ns;
     for (int e = threadIdx.x; e < nent && e < kSelfTab; e += blockDim.x)
       self_entry(sg, nseg, ns, nt, glx, glw, Mm, e, tabl + 3 * e);
@@ -588,6 +589,7 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
           });
           fx_node_from_normal(N, sn + 1, w, nn, &wm, &ew);
         }
+        if (nbad) ew = kFxBad + 1;
         // the target is the chart's value at the node: x - X(P + delta) = -dX
         FxS dm[3];
         int E = 0;

@@ -156,3 +156,26 @@ def test_low_frequency_imaginary_part(ctx, deg, kind):
     else:
         for a, b in zip(*parts):
             assert np.linalg.norm(a * (ks[1] / ks[0]) ** 3 - b) <= 1e-10 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("deg", [3, 6])
+def test_target_normal_of_length_zero(ctx, deg):
+    """S' at a target whose normal is zero is not a number, in the corrections, the potential and the
+    adjoint, and the other targets stay what they are without it."""
+    import torch
+    from paper_2006_02545_gb300 import lcq
+    s = one_patch(deg)
+    x = near_points(s, 6)
+    tn = -np.ones(6, np.int64)
+    nrm = np.random.default_rng(5).standard_normal((3, 6))
+    ok = run_gpu(ctx, s, x, tn, "Sp", 2.0, 1e-6, tgt_normal=nrm)
+    nrm[:, 2] = 0.0
+    g = run_gpu(ctx, s, x, tn, "Sp", 2.0, 1e-6, tgt_normal=nrm)
+    assert ok["status"] == 0 and g["status"] != 0
+    v, w = g["val"].reshape(6, -1), ok["val"].reshape(6, -1)
+    rest = [0, 1, 3, 4, 5]
+    assert np.isnan(v[2]).all() and np.isnan(g["u"][2])
+    assert np.array_equal(v[rest], w[rest]) and np.array_equal(g["u"][rest], ok["u"][rest])
+    z = lcq.apply_adjoint(ctx, g["ds"], g["near"], g["corr"], torch.ones(6, dtype=torch.complex128).cuda())
+    ctx.sync(60000)
+    assert np.isnan(z.cpu().numpy()).all()
