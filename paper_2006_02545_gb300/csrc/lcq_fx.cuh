@@ -174,9 +174,11 @@ LCQ_HD FxKernel fx_kernel(int kind, double kr, double ki, double ar, double ai, 
   for (f.ed = e + 2; m != 0 && m < (1ull << 61); m <<= 1) --f.ed;
   f.kd = m;
   const double p = ar * ki, q = ai * ki;
-  // a product of the constants that overflows: no phase counts as covered, so that every pair
-  // takes the FP64 kernel
-  if (!(fabs(p) < 1e300 && fabs(q) < 1e300)) f.ek = 100000;
+  // constants that are not finite, or whose product overflows: no phase counts as covered, so that
+  // every pair takes the FP64 kernel
+  if (!(fabs(p) < 1e300 && fabs(q) < 1e300 && fabs(ar) + fabs(ai) <= 1.7e308 &&
+        fabs(br) + fabs(bi) <= 1.7e308))
+    f.ek = 100000;
   f.ar = fx_const(ar);
   f.ai = fx_const(ai);
   f.p = fx_const(p);

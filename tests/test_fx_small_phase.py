@@ -57,6 +57,11 @@ def fx(tmp_path_factory):
                out.ctypes.data_as(C.c_void_p))
         assert ok
         return out
+
+    one.covers = lambda kind, kp, d, n, W, ints: bool(f(
+        cs.ctypes.data_as(C.c_void_p), dec.ctypes.data_as(C.c_void_p), kind,
+        *[np.ascontiguousarray(v, dtype=np.float64).ctypes.data_as(C.c_void_p) for v in (kp, d, n)],
+        C.c_double(W), int(ints), np.zeros(2).ctypes.data_as(C.c_void_p)))
     return one
 
 
@@ -120,3 +125,11 @@ def test_zero_wave_number(fx):
     d, n = np.array([0.3, -0.2, 0.5]), np.array([0.6, 0.0, 0.8])
     for kind in (0, 1):
         assert fx(kind, (0.0, 0, 0, 0, 0, 0), d, n, 1.0, True)[1] == 0.0
+
+
+@pytest.mark.parametrize("kp", [(1.0, 0, 1, 0, np.inf, 0), (1.0, 0, 1, 0, 0, np.nan),
+                                (1.0, 0, np.inf, 0, 0, 0), (1.0, 0, 0, np.nan, 1, 0),
+                                (np.nan, 0, 1, 0, 1, 0), (1.0, np.inf, 1, 0, 1, 0)])
+def test_constants_not_finite(fx, kp):
+    """Constants that are not finite are left to the FP64 kernel, which passes them on."""
+    assert not fx.covers(2, kp, np.array([0.3, -0.2, 0.5]), np.array([0.6, 0.0, 0.8]), 1.0, True)

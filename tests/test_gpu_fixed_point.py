@@ -179,3 +179,22 @@ def test_target_normal_of_length_zero(ctx, deg):
     z = lcq.apply_adjoint(ctx, g["ds"], g["near"], g["corr"], torch.ones(6, dtype=torch.complex128).cuda())
     ctx.sync(60000)
     assert np.isnan(z.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("deg", [3, 6])
+@pytest.mark.parametrize("bad", [dict(beta=np.inf), dict(beta=complex(0, np.nan)), dict(alpha=np.inf)])
+def test_constants_not_finite(ctx, deg, bad):
+    """The allocation-free entry takes any constants; those that are not finite make every correction
+    a NaN and the status says so."""
+    import torch
+    from paper_2006_02545_gb300 import lcq
+    s = one_patch(deg)
+    n = W.n_nodes(deg)
+    x = torch.from_numpy(near_points(s, 5)).cuda()
+    out = torch.zeros((5, n), dtype=torch.complex128, device="cuda")
+    kw = dict(alpha=1.0, beta=0.0, max_depth=6)
+    kw.update(bad)
+    st = lcq.adaptive_corrections_noalloc(deg, torch.from_numpy(s.xyz).cuda(), x, "CFIE", 1.0, 8, 1e-6,
+                                          out, **kw)
+    assert st == 2                                    # LCQ_ERR_NONFINITE
+    assert not torch.isfinite(torch.view_as_real(out)).all(-1).any()
