@@ -205,23 +205,26 @@ __device__ __forceinline__ void load_fx_normal(const TA& ta, int i, double* xrel
 }
 
 // Kernel value of target x and the node at X (stride sx), normal nn (stride sn), W = w 2^(ew-62);
-// env: the rounding envelope (FP32) for patch radius R.
+// env: the rounding envelope (FP32 where its range allows, else FP64) for patch radius R.
 __device__ __forceinline__ cplx fx_value(const KernelParams& kp, const FxKernel& fx,
                                          const KernelParamsF& kf, const FxTables& tab,
                                          const double* x, const double* X, int sx, const u64* nn,
-                                         int sn, u64 w, int ew, float R, float* env) {
+                                         int sn, u64 w, int ew, double R, double* env) {
   const double d0 = x[0] - X[0], d1 = x[1] - X[sx], d2 = x[2] - X[2 * sx];
   const FxS n[3] = {fx_unjoin(nn[0]), fx_unjoin(nn[sn]), fx_unjoin(nn[2 * sn])};
   cplx g;
   // W in FP32 for the envelope: its leading 24 bits at its exponent
-  float fw = 0.0f;
+  float fw = 0.0f, ev = 0.0f;
   if (env) {
     const int e = min(max(ew, -120), 120);
     fw = (float)(uint32_t)(w >> 32) * 9.31322575e-10f * __int_as_float((127 + e) << 23);
   }
-  if (!fx_eval<false>(fx, tab, d0, d1, d2, n, w, ew, &g.re, &g.im, env, kf.kr, kf.ki, kf.eb,
-                      kf.ea * R, fw))
-    g = fx_fallback(kp, d0, d1, d2, n[0], n[1], n[2], w, ew, (double)R, env);
+  if (fx_eval<false>(fx, tab, d0, d1, d2, n, w, ew, &g.re, &g.im, env ? &ev : nullptr, kf.kr, kf.ki,
+                     kf.eb, kf.ea * (float)R, fw)) {
+    if (env) *env = (double)ev;
+  } else {
+    g = fx_fallback(kp, d0, d1, d2, n[0], n[1], n[2], w, ew, R, env);
+  }
   return g;
 }
 
@@ -260,7 +263,6 @@ __device__ void block_moments(const double* cf, const double* cfd, const double*
   const KernelParamsF kf = to_f32(kp);
   const FxKernel& fx = kp.fx;  // read at its uses: as a register copy it spills (224 B)
   const FxTables tab = fx_tables();
-  const float fR = (float)R;
   const int total = nseg * Q;
   // The rules are conical products, rows of mr nodes sharing v, and every segment map
   // here keeps v a function of the rule's v alone (e1y = 0: T0 and all its midpoint
@@ -334,10 +336,8 @@ __device__ void block_moments(const double* cf, const double* cfd, const double*
         const int i = e / nch, ql = e - i * nch;
         const u64* nn = kp.kind == 3 ? tn + 3 * i : Ns + ql;
         const int st = kp.kind == 3 ? 1 : C::CH;
-        float ev = 0.0f;
         G[i * C::CH + ql] = fx_value(kp, fx, kf, tab, tx + 3 * i, Xs + ql, C::CH, nn, st, Ws[ql],
-                                     (int)Es[ql], fR, ENV ? &ev : nullptr);
-        if (ENV) Ev[i * C::CH + ql] = (double)ev;
+                                     (int)Es[ql], R, ENV ? Ev + i * C::CH + ql : nullptr);
       }
       __syncthreads();
       // one thread per (target, nm), outputs packed densely; with ENV the extra index nm = n
@@ -762,9 +762,11 @@ __device__ __forceinline__ void block_moments_form(
                           : fx_vector_int(txi[3 * i] - Xi[0], txi[3 * i + 1] - Xi[1],
                                           txi[3 * i + 2] - Xi[2], S, dm, &de);
                 if (!ok || !fx_core<false>(fx, tab, dm[0], dm[1], dm[2], de, nt3, wm, ew, &g.re,
-                                           &g.im, &ev, kf.kr, kf.ki, kf.eb, kf.ea * fR, Jf))
-                  g = fx_fallback(kp, diff(0), diff(1), diff(2), nt3[0], nt3[1], nt3[2], wm, ew,
-                                  (double)fR, &ev);
+                                           &g.im, &ev, kf.kr, kf.ki, kf.eb, kf.ea * fR, Jf)) {
+                  double e = 0.0;
+                  g = fx_fallback(kp, diff(0), diff(1), diff(2), nt3[0], nt3[1], nt3[2], wm, ew, R, &e);
+                  ev = (float)e;
+                }
               }
             }
             ex = ((uint32_t)exp_field(g.re) << 16) | (uint32_t)exp_field(g.im);

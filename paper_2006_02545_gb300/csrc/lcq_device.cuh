@@ -648,18 +648,14 @@ __device__ __forceinline__ cplx kernel_eval(const KernelParams& kp, double x0, d
 // values that are not finite.  n, w, ew: the node as fx_eval takes it.  Rare, so out of line.
 static __device__ __noinline__ cplx fx_fallback(const KernelParams& kp, double d0, double d1,
                                                 double d2, FxS n0, FxS n1, FxS n2, u64 w, int ew,
-                                                double R, float* env) {
+                                                double R, double* env) {
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
   const double Jw = ew > kFxBad ? nan : ldexp((double)w, ew - 62) * 12.566370614359172954;
   const double s = Jw * 2.168404344971008868e-19;  // 2^-62
   auto val = [](FxS a) { return (double)a.h * 4294967296.0 + 2.0 * (double)a.l; };
   KernelParams k = kp;
   if (k.kind == 3) k.kind = 1;
-  double e = 0.0;
-  const cplx g = kernel_eval(k, d0, d1, d2, 0.0, 0.0, 0.0, val(n0) * s, val(n1) * s, val(n2) * s,
-                             Jw, R, env ? &e : nullptr);
-  if (env) *env = (float)e;
-  return g;
+  return kernel_eval(k, d0, d1, d2, 0.0, 0.0, 0.0, val(n0) * s, val(n1) * s, val(n2) * s, Jw, R, env);
 }
 
 // A node for fx_eval from its unnormalized normal N (|N| the area element) and rule weight:

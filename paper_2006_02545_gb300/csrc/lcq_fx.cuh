@@ -452,7 +452,8 @@ LCQ_HD_NOINLINE void fx_small_value(const FxKernel& K, u64 RI, u64 R, int E, u64
 // (and nothing written) for arguments that it does not cover: a phase above 2^22 turns, a decay
 // above 2^9 halvings, a node that is not finite (ew above kFxBad).  With env the rounding
 // envelope |G| Jw (eb + ea |1 - ikr| R / r^2) in FP32 (fk: |kr|, fki: ki, feb = eb, feaR = ea R,
-// fw = W in FP32).
+// fw = W in FP32); false too where its factors could leave FP32's range (r or W / r beyond 2^+-60
+// and 2^+-120: surfaces of a size far from 1).
 // Km: K in memory, for a caller that holds K in registers (the call of fx_small_value takes its address).
 template <bool INT>
 LCQ_HD bool fx_core(const FxKernel& K, const FxTables& tab, FxS D0, FxS D1, FxS D2, int E,
@@ -460,6 +461,9 @@ LCQ_HD bool fx_core(const FxKernel& K, const FxTables& tab, FxS D0, FxS D1, FxS 
                     float fki, float feb, float feaR, float fw, const FxKernel* Km = nullptr) {
   const int sh = E + K.ek + 8;
   if (sh > 30 || ew > kFxBad) return false;
+  if (env && ((unsigned)(E + 60) > 120u || (unsigned)(ew + 120) > 240u ||
+              (unsigned)(ew - E + 120) > 240u))
+    return false;
   const FxRoot rt = fx_root(D0, D1, D2);
   const u64 RI = rt.RI, R = rt.R;
   // the phase in turns 2^-64 and e^{ikr}
@@ -488,13 +492,12 @@ LCQ_HD bool fx_core(const FxKernel& K, const FxTables& tab, FxS D0, FxS D1, FxS 
     eg -= nn;
   }
   if (env) {
-    // 1/r and r in FP32 from the estimate (E within 300: out-of-range scales saturate)
-    const int eb = fx_max(fx_min(E, 120), -120);
+    // 1/r and r in FP32 from the estimate
 #ifdef __CUDA_ARCH__
-    const float sc = __int_as_float((127 - eb) << 23);
-    const float rs = __int_as_float((127 + eb) << 23);
+    const float sc = __int_as_float((127 - E) << 23);
+    const float rs = __int_as_float((127 + E) << 23);
 #else
-    const float sc = ldexpf(1.0f, -eb), rs = ldexpf(1.0f, eb);
+    const float sc = ldexpf(1.0f, -E), rs = ldexpf(1.0f, E);
 #endif
     const float fri = rt.y * 16384.0f * sc, fr = rt.f * rt.y * rs * 6.103515625e-05f;
     const float fo = fki * fr + 1.0f, f1 = fk * fr;

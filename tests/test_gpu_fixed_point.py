@@ -198,3 +198,23 @@ def test_constants_not_finite(ctx, deg, bad):
                                           out, **kw)
     assert st == 2                                    # LCQ_ERR_NONFINITE
     assert not torch.isfinite(torch.view_as_real(out)).all(-1).any()
+
+
+@pytest.mark.parametrize("deg,kind", [(1, "S"), (2, "D"), (3, "CFIE")])
+@pytest.mark.parametrize("scale", [1e-25, 1e25])
+def test_surfaces_of_any_size(ctx, deg, kind, scale):
+    """The smallest degrees in units far from 1: refinement (whose rounding floor comes from the
+    kernel's envelope) and potential as the oracle's."""
+    s = one_patch(deg)
+    s.xyz[:] *= scale
+    x = near_points(s, 9)
+    tn = -np.ones(9, np.int64)
+    k = 2.0 / scale
+    a, b = (1.0, -1j * k) if kind == "CFIE" else (1.0, 0.0)
+    kw = dict(max_depth=8, self_order=6)
+    eps = 1e-9 / (1.0 if kind == "S" else scale)      # the tolerance is eps times a length
+    g = run_gpu(ctx, s, x, tn, kind, k, eps, alpha=a, beta=b, leaf_order=6, **kw)
+    oc, uo = run_oracle(s, x, tn, kind, k, eps, alpha=a, beta=b, sigma=g["sigma"], leaf_order=6, **kw)
+    assert g["status"] in (0, 4)
+    assert all(p == q for p, q, _ in leaves_by_pair(g, oc))
+    assert np.linalg.norm(g["u"] - uo) <= 1e-10 * np.linalg.norm(uo)
