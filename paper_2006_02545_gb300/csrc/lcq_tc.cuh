@@ -362,7 +362,8 @@ __device__ __forceinline__ void grad_add(GradSum& s, const KernelParams& kp, con
   const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
   if (r2 == 0.0) return;
   const double ir = rsqrt_nr(r2);
-  const double r = r2 * ir;
+  double r = r2 * ir;
+  r = fma(0.5 * ir, fma(-r, r, r2), r);  // the phase k r feels its last bit
   double sn, cs;
   sincos_tab(kp.kr * r, g_sct, &sn, &cs);
   double g = ir;
