@@ -171,8 +171,8 @@ __device__ __forceinline__ void fx_chart_store(const double* cf, int i0, int ste
 }
 
 // By the block's threads, from the coefficients cf and the projections duv (load_coef_derivs);
-// begins and ends with a barrier.
-template <int D>
+// begins and ends with a barrier.  FP64: the chart stays in FP64 whatever its scales.
+template <int D, bool FP64 = false>
 __device__ void load_fx_chart(const double* cf, const double* __restrict__ duv, FxChart<D>* ch) {
   __syncthreads();
   load_coef_derivs<D>(cf, duv, reinterpret_cast<double*>(ch->d));
@@ -184,7 +184,10 @@ __device__ void load_fx_chart(const double* cf, const double* __restrict__ duv, 
     for (int k = 0; k < 12; ++k)
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
-    if (threadIdx.x == 0) fx_chart_scales<D>(s, ch);
+    if (threadIdx.x == 0) {
+      fx_chart_scales<D>(s, ch);
+      if (FP64) ch->fp64 = 1;
+    }
   }
   __syncthreads();
   fx_chart_store<D>(cf, threadIdx.x, blockDim.x, ch);

@@ -382,12 +382,19 @@ struct SelfSeg {
 // factors are formed once per (panel, angle) instead of per node, basis, tangents and chord are
 // fixed-point (lcq_fxgeom.cuh), and the contraction runs on the tensor cores (tc_tile with one
 // target: the chunk's 128 kernel values are one row).  1280 patches, generation: 262 -> 244 ms.
+// The largest degrees keep FP64 basis values and an FP64 contraction: the fixed-point basis and its
+// slices are fractions of the bound 2^E_nm, reached at a corner only, which is 2^16 at degree 10.
+// Error of one patch's self weights against 80 bits beyond what the chart's coefficients give all
+// forms, of the imaginary part, fixed and FP64: degree 6 5.3e-15 and 5.1e-15, degree 8 1.7e-14 and
+// 1.3e-14, degree 9 3.0e-14 and 2.6e-14, degree 10 8.0e-14 and 3.8e-14.
+constexpr int kSelfFp64Deg = 9;
 constexpr int kSelfThreads = 128;
 constexpr int kSelfTab = 384;  // (panel, angle) entries kept; longer rules form them per node
 template <int D>
 struct SelfCfg {
   static constexpr int n = (D + 1) * (D + 2) / 2;
-  static constexpr int BST = kSelfThreads + 8;
+  static constexpr bool fp64 = D >= kSelfFp64Deg;
+  static constexpr int BST = kSelfThreads + (fp64 ? 1 : 8);
   static constexpr size_t taylor = ((D + 1) * n + 2 * n * n) * sizeof(double);
   static constexpr size_t basis = (size_t)n * BST * 8;
   static constexpr size_t OFF_G = ((taylor > basis ? taylor : basis) + 15) / 16 * 16;
@@ -416,8 +423,8 @@ __device__ __forceinline__ void self_entry(const SelfSeg* sg, int nseg, int ns, 
   out[2] = glw[ti] * (hi - lo) * g.mu * (0.5 * (ex + exi)) * g.area2 * Mm[4];
 }
 
-// Basis slices (column B, stride st) and normal X_u x X_v of a node of a chart that the fixed-point
-// scales do not fit.  Rare, so out of line.
+// Basis slices (column B, stride st; of the largest degrees the FP64 values) and normal X_u x X_v of
+// a node in FP64: of a chart that the fixed-point scales do not fit, or of the largest degrees.
 template <int D>
 __device__ __noinline__ void self_node_fp64(double u, double v, const FxChart<D>& ch, uint2* B, int st,
                                             double* N) {
@@ -426,7 +433,9 @@ __device__ __noinline__ void self_node_fp64(double u, double v, const FxChart<D>
                       reinterpret_cast<const double*>(ch.d), X, Xu, Xv, K);
 #pragma unroll 1
   for (int k = 0; k < (D + 1) * (D + 2) / 2; ++k)
-    B[k * st] = slice_bytes(fix_mag<8>(K[k], c_kwexp[k]), __double2hiint(K[k]) < 0);
+    B[k * st] = SelfCfg<D>::fp64
+                    ? make_uint2((uint32_t)__double2loint(K[k]), (uint32_t)__double2hiint(K[k]))
+                    : slice_bytes(fix_mag<8>(K[k], c_kwexp[k]), __double2hiint(K[k]) < 0);
   cross3(Xu, Xv, N);
 }
 
@@ -465,7 +474,7 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
       kps = patch_kp(dv, j, kp);
       ord = dv.pgroup ? dv.grp[dv.pgroup[j]].self_order : order;
     }
-    load_fx_chart<D>(cf, dv.duv[D], &ch);
+    load_fx_chart<D, SC::fp64>(cf, dv.duv[D], &ch);
     const int ns = ord, nt = ord;
     const double* glx = dv.gl_x + dv.gl_off[ord];
     const double* glw = dv.gl_w + dv.gl_off[ord];
@@ -577,7 +586,7 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
         FxS nn[3];
         u64 wm;
         int ew;
-        if (ch.fp64) {
+        if (SC::fp64 || ch.fp64) {
           double Nd[3];
           self_node_fp64<D>(P[0] + du, P[1] + dvv, ch, Bs + threadIdx.x, SC::BST, Nd);
           fx_make_node(Nd, w, nn, &wm, &ew);
@@ -616,7 +625,25 @@ __global__ void __launch_bounds__(kSelfThreads, 4) k_self(Dev dv, const int32_t*
           gk = fx_fallback(kps, -dX[0], -dX[1], -dX[2], nu[0], nu[1], nu[2], wm, ew, 0.0, nullptr);
         }
       } else {
-        for (int k = 0; k < n; ++k) Bs[k * SC::BST + threadIdx.x] = make_uint2(kZeroSlices, kZeroSlices);
+        const uint32_t z = SC::fp64 ? 0u : kZeroSlices;
+        for (int k = 0; k < n; ++k) Bs[k * SC::BST + threadIdx.x] = make_uint2(z, z);
+      }
+      if constexpr (SC::fp64) {
+        reinterpret_cast<cplx*>(G)[threadIdx.x] = gk;
+        __syncthreads();
+        for (int k = threadIdx.x; k < n; k += kSelfThreads) {
+          const double* K = reinterpret_cast<const double*>(Bs) + k * SC::BST;
+          cplx s = {0.0, 0.0};
+          for (int q = 0; q < kSelfThreads; ++q) {
+            const cplx gq = reinterpret_cast<const cplx*>(G)[q];
+            s.re = fma(gq.re, K[q], s.re);
+            s.im = fma(gq.im, K[q], s.im);
+          }
+          acc[k].re += s.re;
+          acc[k].im += s.im;
+        }
+        __syncthreads();
+        continue;
       }
       const int fr = __reduce_max_sync(0xffffffffu, exp_field(gk.re));
       const int fi = __reduce_max_sync(0xffffffffu, exp_field(gk.im));
