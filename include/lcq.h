@@ -67,8 +67,10 @@ typedef enum {
  *              from the patch centroid.  LCQ_MIXED falls back to FP64 for S'. */
 typedef enum { LCQ_S = 0, LCQ_D = 1, LCQ_CFIE = 2, LCQ_SP = 3 } lcq_kernel;
 
-/* LCQ_FP64: every step in FP64 (the contraction of kernel values with basis values on the
- * tensor cores by an exact split of the FP64 operands).
+/* LCQ_FP64: every step in FP64 or, for kernel values, charts, basis values and normals, in 64-bit
+ * fixed point of no less precision (charts whose range does not fit it stay FP64; the real and the
+ * imaginary part of a kernel value each keep their digits down to k = 0); the contraction of kernel
+ * values with basis values runs on the tensor cores by an exact split of the operands.
  * LCQ_MIXED: the (target, node) kernel values of the adaptive near integration and of the
  * smooth-rule and annulus moments move to the FP32 pipe, always from the FP64 difference
  * x - X; the chart geometry, self rules, far orders, refinement tests (on the moments),
@@ -250,7 +252,10 @@ lcq_status lcq_corr_export_stats(lcq_corr* corr, int32_t* q, int32_t* q_near, in
  * sigma device complex128 [N] at the nodes, out device complex128 [NT].
  * jump != 0 adds jump * sigma(x_t) for on-surface targets (e.g. 0.5 for the
  * exterior limit of D).  The kernel must match the one the corrections were
- * generated for. */
+ * generated for.  The far sum is cut into parts, each added in order and the parts in a fixed
+ * order, so a call repeats bit for bit; their number follows from the numbers of targets and
+ * sources and the GPU's SMs, so the same target's potential may differ in its last bits between
+ * calls with unlike numbers of targets (lcq_apply_adjoint likewise per source). */
 lcq_status lcq_apply_corrected_S(lcq_ctx* ctx, const lcq_surface* surf, const lcq_near* near,
                                  const lcq_corr* corr, const double* sigma, double jump,
                                  double* out);
@@ -364,7 +369,8 @@ lcq_status lcq_stage_times(lcq_ctx* ctx, float* ms6, int64_t* launches);
  * every byte of the device).  The paper has no counterpart; this is a library facility.
  *
  * Computes the adaptive near corrections of ONE patch for targets that are all treated
- * as adaptive, exactly as lcq_gen_corrections computes them for adaptive near pairs: out[t][l] = sum_nm V[nm][l] (I^adaptive_nm(x_t) - I^{rule q}_nm(x_t)).
+ * as adaptive, exactly as lcq_gen_corrections computes them for adaptive near pairs (they may lie at
+ * any distance; a target's row does not depend on the others): out[t][l] = sum_nm V[nm][l] (I^adaptive_nm(x_t) - I^{rule q}_nm(x_t)).
  *   deg       patch degree, 1..8
  *   y         device double SoA [3][n] node coordinates, n = (deg+1)(deg+2)/2
  *   n_targets 1..128; tgt_xyz device double SoA [3][n_targets] (off-surface points)

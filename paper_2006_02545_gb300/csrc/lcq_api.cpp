@@ -807,8 +807,10 @@ static Dev make_dev(lcq_ctx* ctx, const lcq_near* nr, const int32_t* q, int ldI,
 }
 
 // Per-block workspace of the adaptive kernel (sized by the largest work item and the depth
-// cap) and its grid: as many blocks as fit the device, no more than one degree's work items, and
-// within 64 GB of workspace.
+// cap) and its grid: as many blocks as fit the device and no more than one degree's work items.  A
+// second block per SM is left out where it would take the workspace above 64 GB: of the card's 280 GB
+// the moments, the CSR and the caller need the rest (patches with 10^5 and more adaptive targets; the
+// first block per SM is allocated whatever it takes).
 static void adaptive_stride(lcq_ctx* ctx, const lcq_near* nr, int64_t A, int levels, int64_t items,
                             int64_t* stride_out, int* grid_out) {
   const int64_t n = nr->n_max;

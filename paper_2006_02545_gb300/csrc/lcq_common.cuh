@@ -233,7 +233,8 @@ struct SegMap {
 };
 
 // Moments I[i][seg][nm] = sum_{q in seg} w_q K(x_i, X_q) J_q K_nm(u_q, v_q) for a smooth
-// rule (Q nodes) pushed onto nseg affine images of T0, for T targets, in FP64 throughout
+// rule (Q nodes) pushed onto nseg affine images of T0, for T targets, geometry and contraction in FP64,
+// kernel values in fixed point
 // (the far order q_j, whose decisions compare these moments, and the moments of the
 // smallest degrees, block_moments_any).  Geometry is evaluated once per chunk of nodes and
 // shared by all targets (Sec. 4.3 reuse).
@@ -496,7 +497,8 @@ __device__ __forceinline__ void tc_tile(const uint2* Bs, const uint4* G, const i
 // mma.sync on fragments built from the slice bytes.  Storing an operand as 8 bytes (not as 8
 // f16) lets a chunk hold 256 columns where it held 128, so that every thread has a node and the
 // barriers come half as often; they, not the pipes, bounded the kernel (1280-patch CFIE, eps
-// 1e-9: adaptive walk 295 ms at 32% of the issue slots before, 180 ms at 47% since).
+// 1e-9: adaptive walk 295 ms at 32% of the issue slots before, 180 ms at 47% with it;
+// 206 at 48% since the kernel values keep the digits of their small parts).
 // Positions in fixed point are relative to the centroid at the exponent S = sx + 3 of the patch's own
 // chart (|X_c| < 2^sx, no bit of it dropped); a target beyond 2^(S - 1) in some coordinate, over
 // four times the chart's bound away, takes the FP64 difference (nothing cancels there).  So a
@@ -904,7 +906,9 @@ __device__ void block_moments_tc(const FxChart<D>& ch, const double* __restrict_
 // small to pay for the tensor-core pipeline's fixed cost per 8-target tile (barriers, the
 // slices).  2400 patches, S, generation with this engine and with the tensor one: degree 1 eps
 // 5e-3 12.6 and 17.9 ms, degree 2 eps 5e-7 43.3 and 46.4, degree 3 eps 5e-3 22.6 and 26.8, eps 5e-7
-// 77.7 and 76.1 (the smooth rules alone: 5.8 and 14.6).  Every other case: block_moments_tc.  smb holds either engine's workspace.
+// 77.7 and 76.1 (the smooth rules alone: 5.8 and 14.6, the adaptive walk alone 60.3 and 56.6: one
+// switch serves both, and the walk gains less than the rules lose, except there).  Every other case:
+// block_moments_tc.  smb holds either engine's workspace.
 constexpr int kFp64MomentsMaxDeg = 3;
 template <int D, class TA, class OR>
 __device__ __forceinline__ void block_moments_any(
@@ -1135,7 +1139,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adaptive(const int* __restrict_
   SegMap* segs = reinterpret_cast<SegMap*>(cf + n * 3);
   int* ism = reinterpret_cast<int*>(segs + 4);  // [64]: scan scratch + misc
   unsigned long long* stk = reinterpret_cast<unsigned long long*>(ism + 64);  // [4 * 32]
-  // tensor-core moment workspace, 128-byte aligned (ldmatrix needs 16)
+  // tensor-core moment workspace, 128-byte aligned (its 128-bit accesses need 16)
   unsigned char* smb = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(stk + 4 * 32) + 127) & ~static_cast<uintptr_t>(127));
   double* ws = reinterpret_cast<double*>(smb);

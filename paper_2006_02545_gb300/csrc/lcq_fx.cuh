@@ -1,10 +1,11 @@
 // Helmholtz kernel values in 64-bit fixed-point arithmetic on the integer pipe.
 //
-// On this GPU a warp's FP64 instruction occupies its pipe for 64 cycles, a 32 x 32 + 64 bit
-// integer multiply-add for 2 and a 64-bit addition for 1.  A product of two 62-bit mantissas
-// to 62 bits is three such multiply-adds, so the whole kernel value costs less than seven
-// FP64 instructions would, with more bits: every quantity below is a 57- to 63-bit mantissa
-// on a scale that is known beforehand (or one exponent per pair), where FP64 has 53.
+// On this GPU a warp's FP64 instruction occupies its pipe for 64 cycles, a 32 x 32 + 64 bit integer
+// multiply-add for 4, a shift or logic instruction for 2 and a 64-bit addition for 1 (measured).  A
+// product of two 62-bit mantissas to 62 bits is three such multiply-adds, so the whole kernel value, some
+// 450 (S) to 730 (CFIE) instructions, takes about 770 to 1,200 cycles a pair and warp in the far sum,
+// where 41 FP64 instructions took 3,600, and with more bits: every quantity below is a 57- to 63-bit
+// mantissa on a scale of its own, where FP64 has 53.
 //
 // The value is written without the node's area element in it:
 //   K~ = W e^{-ki r} e^{i th} (A + iB) / r^2,   W = Jw / (4 pi),  th = kr r,

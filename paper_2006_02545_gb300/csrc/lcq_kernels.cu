@@ -70,14 +70,14 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
 
 // Direct far sum over the oversampled sources, one thread per target and range of sources
 // (tiles staged through shared memory): block (b, s) sums part s of gridDim.y equal parts of
-// the sources of target block b into part[s][t], and k_csr_apply adds the parts in order.  Few
+// the sources of target block b into part[s][t], and k_csr_apply adds the parts in a fixed order.  Few
 // targets alone leave the chip idle (1000 targets are 8 blocks on 152 SMs), so the launch cuts
 // the sources until there are several waves of blocks (far_sum_parts).
 // The kernel values are fixed-point (fx_eval): of FP64 there are only the difference x - X and
 // the four multiply-adds of the density (448 cycles of the FP64 pipe a pair and warp, beside
-// about 440 integer instructions for the single layer).  35,840 targets x 127,606 sources, CFIE:
-// 407 ms with FP64 kernel values (41 FP64 instructions a pair), 126 ms so; 8,960 x 25,920, S: 15.7
-// and 4.4 ms.  More warps per SM (128, 96, 80, 64 registers) and two sources a step: within 3%.
+// about 440 integer instructions for the single layer, 720 for the CFIE).  35,840 targets x 127,606 sources, CFIE:
+// 407 ms with FP64 kernel values (41 FP64 instructions a pair), 137 ms so; 8,960 x 25,920, S: 15.7
+// and 4.6 ms.  More warps per SM (128, 96, 80, 64 registers) and two sources a step: within 3%.
 // The sources of an on-surface target's own patch are skipped (their contribution is
 // carried entirely by the self correction).  In a batch of independent surfaces a target
 // sums only its own surface's sources [gsrc[g], gsrc[g+1]) with that surface's kernel.
