@@ -703,6 +703,10 @@ def run_ours(args, rank, world, local_rank):
                            " kernel values, fixed-point geometry; contraction on the f16 tensor "
                            "cores by an exact slice split"),
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                "frac_is": "an FP64-equivalent rate over the FP64 FMA peak, not a utilisation (no "
+                           "ceiling at 1): kernel values and geometry run on the integer pipes and "
+                           "the contraction on the tensor cores; what bounds the kernel is the "
+                           "issue of integer instructions (profiles/)",
                 "traffic": traffic_for("k_adaptive"),
                 "peak_source": "measured in this run: FP64 FMA chains on every SM "
                                "(lcq_pipe_peaks), CUDA events",
